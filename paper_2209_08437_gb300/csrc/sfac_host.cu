@@ -95,18 +95,17 @@ int padded_length(int n) {
     return L;
 }
 
-void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P) {
+void increment_columns(const AxisHost& T, double tau, std::vector<double>* g, std::vector<double>* h) {
     const int n = T.n;
-    const int L = padded_length(n);
-    P->n = n;
-    P->L = L;
     std::vector<double> cs(2 * n), sn(2 * n);
     for (int m = 0; m < 2 * n; ++m) sincospi_frac(m, n, &cs[m], &sn[m]);
-    // First columns of e^{t C} - I and e^{tau S} - I from expm1 of the spectra:
+    // From expm1 of the spectra:
     //   g_d = (1/n) sum_j expm1(t lambda_j) cos(2 pi j d / n),     d = 0 .. n-1
     //   h_d = (1/n) sum_j expm1(tau mu_j) cos(pi d (2j - 1) / n),  d = 0 .. n-1 (h_{-d} = h_d)
     // (the identity's share sum_j cos(...) vanishes for d != 0 mod n).
-    std::vector<double> xc(n), xs(n), g1(n), h1(n);
+    std::vector<double> xc(n), xs(n);
+    g->resize(n);
+    h->resize(n);
     for (int j = 0; j < n; ++j) {
         xc[j] = std::expm1(0.5 * tau * T.lambda[j]);
         xs[j] = std::expm1(tau * T.mu[j]);
@@ -125,9 +124,18 @@ void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P) {
             mh += step;
             if (mh >= two_n) mh -= two_n;
         }
-        g1[d] = sg.value() / n;
-        h1[d] = sh.value() / n;
+        (*g)[d] = sg.value() / n;
+        (*h)[d] = sh.value() / n;
     }
+}
+
+void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P) {
+    const int n = T.n;
+    const int L = padded_length(n);
+    P->n = n;
+    P->L = L;
+    std::vector<double> g1, h1;
+    increment_columns(T, tau, &g1, &h1);
     // Padded, symmetric columns: offset d in (-n, n) at index d mod L. The
     // circulant part repeats its column with period n (c_d = g_{d mod n}).
     auto spectrum = [&](const std::vector<double>& col, bool circulant, double diag_add, std::vector<double>* out) {

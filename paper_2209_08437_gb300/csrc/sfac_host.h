@@ -30,6 +30,10 @@ bool is_pow2(int v);
 // Smallest power of two >= 2n - 1 (at least 4).
 int padded_length(int n);
 
+// First columns of e^{tau/2 C} - I and e^{tau S} - I (both symmetric Toeplitz, n
+// values each) of the axis in T.
+void increment_columns(const AxisHost& T, double tau, std::vector<double>* g, std::vector<double>* h);
+
 // Padded tables of one axis (needs the spectra of compute_axis in T).
 void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P);
 

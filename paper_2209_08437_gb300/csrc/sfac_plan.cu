@@ -16,6 +16,7 @@
 #include "sfac_host.h"
 #include "sfac_internal.h"
 #include "sfac_steps.h"
+#include "sfac_tc.h"
 
 using sfac::AxisHost;
 using sfac::compute_axis;
@@ -106,6 +107,7 @@ struct sfac_plan {
         const double* dB;
         const void* dtwist;
         const void* dtwid;
+        sfac::TcAxis tc;  // FP64 lines with a tensor-core pass (tc.img != NULL)
     } ax[3] = {};
     double3* diag_partial = nullptr;
     double* diag_out = nullptr;
@@ -174,7 +176,9 @@ sfac_status launch_axis(sfac_plan* P, void* u, int ax, int jq_in, int jq_out, cu
     a.host_io = host_io ? 1 : 0;
     const int N = P->ax[ax].fft_len;
     cudaError_t err;
-    if (P->ax[ax].padded) {
+    if (P->ax[ax].tc.img) {
+        err = sfac::launch_pass_tc_f64(P->ax[ax].tc, a, st);
+    } else if (P->ax[ax].padded) {
         err = (P->p.prec == SFAC_FP64) ? sfac::launch_pass_padded_f64(N, a, st) : sfac::launch_pass_padded_f32(N, a, st);
     } else if (P->p.prec == SFAC_FP64) {
         err = sfac::launch_pass_f64(N, a, st);
@@ -360,14 +364,18 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
         delete P;
         return cuda_fail(err, "cudaGetDevice");
     }
-    // FP64 ratio twiddles of each axis's FFT length.
-    std::vector<double> rtw[3];
+    // FP64 ratio twiddles of each axis's FFT length; first columns of the
+    // exponentials' increments for axes with a tensor-core pass.
+    std::vector<double> rtw[3], gcol[3], hcol[3];
+    bool tc[3] = {false, false, false};
     if (params->prec == SFAC_FP64) {
         try {
             for (int l = 0; l < params->dim; ++l) {
                 const int N = padded[l] ? pad[l].L : params->n[l];
                 const int E = sfac::f64_elems_per_thread(N);
                 if (E <= 16) rtw[l] = sfac::ratio_twiddles(N, E);
+                tc[l] = params->n[l] >= sfac::kTcMinN && params->n[l] <= sfac::kTcMaxN;
+                if (tc[l]) sfac::increment_columns(host[l], params->tau, &gcol[l], &hcol[l]);
             }
         } catch (const std::bad_alloc&) {
             delete P;
@@ -377,16 +385,17 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     // One device block: per axis eC[n], eS[n], twist[2n], twid[2n] reals, the
     // FP64 diagnostic tables, and the ratio twiddles.
     const size_t rs = real_size(P);
-    size_t off[3][9], total = 0;
+    size_t off[3][11], total = 0;
     long long max_partials = 1;
     {
         long long inner = 1;
         for (int l = 0; l < params->dim; ++l) {
             const size_t n = padded[l] ? (size_t)pad[l].L : (size_t)params->n[l];
-            const size_t sz[9] = {n * rs, n * rs, padded[l] ? 0 : 2 * n * rs, 2 * n * rs,
+            const size_t sz[11] = {n * rs, n * rs, padded[l] ? 0 : 2 * n * rs, 2 * n * rs,
                                   n * 8,  padded[l] ? 0 : n * 8, padded[l] ? 0 : 2 * n * 8, 2 * n * 8,
-                                  rtw[l].size() * sizeof(double)};
-            for (int q = 0; q < 9; ++q) {
+                                  rtw[l].size() * sizeof(double),
+                                  gcol[l].size() * sizeof(double), hcol[l].size() * sizeof(double)};
+            for (int q = 0; q < 11; ++q) {
                 off[l][q] = total;
                 total += align256(sz[q]);
             }
@@ -404,6 +413,17 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     total += align256(sizeof(unsigned int));
     const size_t off_bar = total;
     total += align256(2 * sizeof(unsigned int));
+    // Not part of the upload: the digit images of the tensor-core passes and the
+    // builder's scratch (used by one axis after the other).
+    size_t off_img[3] = {0, 0, 0}, alloc = total, scratch = 0;
+    for (int l = 0; l < params->dim; ++l) {
+        if (!tc[l]) continue;
+        off_img[l] = alloc;
+        alloc += align256(sfac::tc_image_bytes(params->n[l]));
+        scratch = std::max(scratch, sfac::tc_scratch_bytes(params->n[l]));
+    }
+    const size_t off_scratch = alloc;
+    alloc += align256(scratch);
     std::vector<unsigned char> blob;
     try {
         blob.assign(total, 0);
@@ -441,6 +461,10 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
                 std::memcpy(blob.data() + off[l][4 + q], dsrc[q]->data(), dsrc[q]->size() * sizeof(double));
         if (!rtw[l].empty())
             std::memcpy(blob.data() + off[l][8], rtw[l].data(), rtw[l].size() * sizeof(double));
+        if (tc[l]) {
+            std::memcpy(blob.data() + off[l][9], gcol[l].data(), gcol[l].size() * sizeof(double));
+            std::memcpy(blob.data() + off[l][10], hcol[l].data(), hcol[l].size() * sizeof(double));
+        }
         for (int q = 0; q < 4; ++q) {
             unsigned char* dst = blob.data() + off[l][q];
             const std::vector<double>& v = *src[q];
@@ -452,21 +476,29 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
             }
         }
     }
-    err = cudaMalloc(&P->dev_tables, total);
+    err = cudaMalloc(&P->dev_tables, alloc);
     if (err != cudaSuccess) {
         delete P;
         cudaGetLastError();
         return fail(SFAC_ENOMEM, std::string("cudaMalloc of tables: ") + cudaGetErrorString(err));
     }
     cudaStream_t st_ = static_cast<cudaStream_t>(stream);
+    unsigned char* base = static_cast<unsigned char*>(P->dev_tables);
+    int report[3][8] = {};
     err = cudaMemcpyAsync(P->dev_tables, blob.data(), total, cudaMemcpyHostToDevice, st_);
+    for (int l = 0; l < params->dim && err == cudaSuccess; ++l)
+        if (tc[l])
+            err = sfac::tc_build(params->n[l], reinterpret_cast<const double*>(base + off[l][9]),
+                                 reinterpret_cast<const double*>(base + off[l][10]), base + off_img[l],
+                                 base + off_scratch, report[l], st_);
     if (err == cudaSuccess) err = cudaStreamSynchronize(st_);
     if (err != cudaSuccess) {
         cudaFree(P->dev_tables);
         delete P;
         return cuda_fail(err, "table upload");
     }
-    unsigned char* base = static_cast<unsigned char*>(P->dev_tables);
+    for (int l = 0; l < params->dim; ++l)
+        if (tc[l]) sfac::tc_accept(params->n[l], base + off_img[l], report[l], &P->ax[l].tc);
     for (int l = 0; l < params->dim; ++l) {
         P->ax[l].eC = base + off[l][0];
         P->ax[l].eS = base + off[l][1];

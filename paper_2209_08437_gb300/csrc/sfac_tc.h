@@ -1,0 +1,47 @@
+// sfac_tc.h - axis passes as exact digit products on the tensor cores.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "sfac_internal.h"
+
+namespace sfac {
+
+// The linear factor of one axis as a dense operator D = P - I, cut into
+// fixed-point digits (see sfac_tc_pass.cuh). `img` holds the digit blocks in the
+// order the pass streams them.
+struct TcAxis {
+    const void* img = nullptr;  // NULL: the axis has no tensor-core pass
+    int n = 0;                  // line length
+    int parts = 0;              // 1: D itself; 2: its even and odd halves
+    int rows = 0;               // rows (outputs) per part: n, or ceil(n/2)
+    int kp = 0;                 // rows rounded up to a multiple of 32 (K of the products)
+    int scale = 0;              // exponent f: the entries are below 2^(f-1) in size
+};
+
+// Digits per operand entry, and their width in bits.
+constexpr int kTcSlices = 6;
+constexpr int kTcBits = 9;
+// Lengths with a tensor-core FP64 pass.
+constexpr int kTcMinN = 32, kTcMaxN = 256;
+
+// Device bytes of the digit image of an axis of n points, and of the scratch
+// the builder needs (n x n doubles twice, and a few words).
+size_t tc_image_bytes(int n);
+size_t tc_scratch_bytes(int n);
+
+// Builds the image from the first columns g, h (device, n doubles each) of
+// e^{tau/2 C} - I and e^{tau S} - I, on stream s. The host words
+// report[0..6] receive, after the stream is synchronised: the scale exponent,
+// then for each digit place the largest sum of |digit| over a row.
+cudaError_t tc_build(int n, const double* g, const double* h, void* img, void* scratch, int* report_host,
+                     cudaStream_t s);
+
+// Fills *ax from the builder's report; false where the sums could leave the
+// range in which the products are exact (the axis then keeps its FFT pass).
+bool tc_accept(int n, const void* img, const int* report, TcAxis* ax);
+
+// One FP64 axis pass (the arguments of launch_pass_f64) through the tensor cores.
+cudaError_t launch_pass_tc_f64(const TcAxis& ax, const PassArgs& a, cudaStream_t s);
+
+}  // namespace sfac

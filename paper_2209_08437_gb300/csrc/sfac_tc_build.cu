@@ -1,0 +1,149 @@
+// sfac_tc_build.cu - the dense operator of one axis and its digit image.
+//
+// With E_C = I + G and E_S = I + H (G circulant, H skew-circulant, both
+// symmetric Toeplitz with first columns g, h) the linear factor of an axis is
+//   P = (I + G)(I + H)(I + G) = I + D,  D = G + W + G W,  W = H + G + H G.
+// D is formed in FP64 from the increments, so its rounding is relative to D
+// itself. It runs once per plan (n = 256: 34 M multiply-adds).
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "sfac_tc.h"
+
+namespace sfac {
+namespace {
+
+constexpr int NS = kTcSlices, B = kTcBits;
+
+int parts_of(int n) { return n <= 128 ? 1 : 2; }
+int rows_of(int n) { return n <= 128 ? n : (n + 1) / 2; }
+int kp_of(int n) { return (rows_of(n) + 31) / 32 * 32; }
+
+// out = X + Y + X Y with X[i][p] = x[|i - p|]; Y = y[|p - j|] (first product) or
+// the stored matrix Ym.
+__global__ void __launch_bounds__(256) tc_product(int n, const double* __restrict__ x, const double* __restrict__ y,
+                                                  const double* __restrict__ Ym, double* __restrict__ out) {
+    const int j = blockIdx.x * 32 + threadIdx.x, i = blockIdx.y * 8 + threadIdx.y;
+    if (i >= n || j >= n) return;
+    double s[4] = {0, 0, 0, 0};
+    for (int p0 = 0; p0 < n; p0 += 4) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int p = p0 + q;
+            if (p < n) s[q] = fma(x[abs(i - p)], Ym ? Ym[(size_t)p * n + j] : y[abs(p - j)], s[q]);
+        }
+    }
+    const double yij = Ym ? Ym[(size_t)i * n + j] : y[abs(i - j)];
+    out[(size_t)i * n + j] = ((s[0] + s[1]) + (s[2] + s[3])) + (x[abs(i - j)] + yij);
+}
+
+// Entry (k, j) of part p of the operator: D itself, or its action on the sums
+// (p = 0) and differences (p = 1) of a line's mirrored values:
+//   D x |_k = (1/2) sum_j [ E_kj (x_j + x_{n-1-j}) + O_kj (x_j - x_{n-1-j}) ].
+__device__ double tc_entry(const double* D, int n, int parts, int rows, int p, int k, int j) {
+    if (k >= rows || j >= rows) return 0.0;
+    const double a = D[(size_t)k * n + j];
+    if (parts == 1) return a;
+    const double b = D[(size_t)k * n + (n - 1 - j)];
+    const bool mid_j = j == n - 1 - j, mid_k = k == n - 1 - k;
+    if (p == 0) return mid_j ? a : a + b;
+    return (mid_j || mid_k) ? 0.0 : a - b;
+}
+
+__global__ void __launch_bounds__(256) tc_max(int n, int parts, int rows, const double* __restrict__ D,
+                                              unsigned long long* out) {
+    double m = 0.0;
+    const int total = parts * rows * rows;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const int p = t / (rows * rows), r = t % (rows * rows);
+        m = fmax(m, fabs(tc_entry(D, n, parts, rows, p, r / rows, r % rows)));
+    }
+    atomicMax(out, (unsigned long long)__double_as_longlong(m));
+}
+
+// Digits of every entry, written as 8 KB blocks of 128 rows x 32 columns per
+// (part, 32 columns, digit place): core matrices of 8 rows x 8 columns, rows
+// first. One CTA per (row, part); report as in tc_build.
+__global__ void __launch_bounds__(128) tc_digits(int n, int parts, int rows, int kp, const double* __restrict__ D,
+                                                 const unsigned long long* __restrict__ maxbits,
+                                                 __half* __restrict__ img, int* report) {
+    const int row = blockIdx.x, p = blockIdx.y;
+    const double m = __longlong_as_double((long long)*maxbits);
+    int f = 0;
+    if (m > 0.0) {
+        f = ilogb(m) + 2;  // m < 2^(f-1)
+        f = f < -200 ? -200 : f;
+    }
+    if (row == 0 && p == 0 && threadIdx.x == 0) report[0] = f;
+    __shared__ int sum[NS];
+    if (threadIdx.x < NS) sum[threadIdx.x] = 0;
+    __syncthreads();
+    for (int j = threadIdx.x; j < kp; j += blockDim.x) {
+        const double v = tc_entry(D, n, parts, rows, p, row, j);
+        long long F = __double2ll_rn(scalbn(v, B * NS - f));
+        for (int i = 0; i < NS; ++i) F += 1LL << (B * i + B - 1);
+        for (int q = 0; q < NS; ++q) {  // q = 0: most significant
+            const int sh = B * (NS - 1 - q);
+            int d = (int)(F >> sh);
+            if (q > 0) d &= (1 << B) - 1;
+            d -= 1 << (B - 1);
+            const size_t block = ((size_t)p * (kp / 32) + j / 32) * NS + q;
+            img[block * (128 * 32) + (size_t)((j % 32) / 8) * (128 * 8) + (row / 8) * 64 + (row % 8) * 8 + j % 8] =
+                __int2half_rn(d);
+            if (d) atomicAdd(&sum[q], abs(d));
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < NS) atomicMax(&report[1 + threadIdx.x], sum[threadIdx.x]);
+}
+
+}  // namespace
+
+size_t tc_image_bytes(int n) { return (size_t)parts_of(n) * (kp_of(n) / 32) * NS * 8192; }
+size_t tc_scratch_bytes(int n) { return 2 * sizeof(double) * (size_t)n * n + 64; }
+
+cudaError_t tc_build(int n, const double* g, const double* h, void* img, void* scratch, int* report_host,
+                     cudaStream_t s) {
+    const int parts = parts_of(n), rows = rows_of(n), kp = kp_of(n);
+    double* W = static_cast<double*>(scratch);
+    double* D = W + (size_t)n * n;
+    unsigned long long* mx = reinterpret_cast<unsigned long long*>(D + (size_t)n * n);
+    int* report = reinterpret_cast<int*>(mx + 1);
+    cudaError_t err = cudaMemsetAsync(mx, 0, 64, s);
+    if (err != cudaSuccess) return err;
+    const dim3 grid((n + 31) / 32, (n + 7) / 8), block(32, 8);
+    tc_product<<<grid, block, 0, s>>>(n, h, g, nullptr, W);
+    tc_product<<<grid, block, 0, s>>>(n, g, nullptr, W, D);
+    tc_max<<<std::max(1, std::min(64, n / 4)), 256, 0, s>>>(n, parts, rows, D, mx);
+    tc_digits<<<dim3(128, parts), 128, 0, s>>>(n, parts, rows, kp, D, mx, static_cast<__half*>(img), report);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    return cudaMemcpyAsync(report_host, report, (1 + NS) * sizeof(int), cudaMemcpyDeviceToHost, s);
+}
+
+bool tc_accept(int n, const void* img, const int* report, TcAxis* ax) {
+    // Largest sum the accumulator of order s = i + j can reach: digits of x are at
+    // most 2^(B-1) in size. Orders up to 5 must stay within 2^24 (FP32 holds every
+    // integer of that size), order 6 within 2^25 and orders 7, 8 anywhere: a unit
+    // lost there is below 2^-54 of the line's largest value.
+    for (int s = 2; s <= 6; ++s) {
+        double bound = 0.0;
+        for (int j = 1; j < s; ++j) bound += std::ldexp((double)report[j], B - 1);
+        if (bound > std::ldexp(1.0, s <= 5 ? 24 : 25)) return false;
+    }
+    // |sum of a row| / 2^f, so that the 64-bit sums of the pass cannot overflow
+    double rowsum = 0.0;
+    for (int j = 1; j <= NS; ++j) rowsum += std::ldexp((double)report[j], -B * j);
+    if (rowsum > 8.0 || report[0] > 40) return false;
+    ax->img = img;
+    ax->n = n;
+    ax->parts = parts_of(n);
+    ax->rows = rows_of(n);
+    ax->kp = kp_of(n);
+    ax->scale = report[0];
+    return true;
+}
+
+}  // namespace sfac

@@ -1,0 +1,104 @@
+"""FP64 passes of 32..256 points on the tensor cores (csrc/sfac_tc_pass.cu):
+the edges of their tiles (lengths around the folding limit 128 and the K step
+32, odd lengths, line counts around the tile widths 8..64), the scaling of each
+line, non-finite values, and the bounded wait."""
+import numpy as np
+import pytest
+
+import paper_2209_08437_gb300 as S
+import sfac_inputs as I
+from oracle import sfac_oracle as O
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+# Rounding of y (1.1e-16), digits below order 9 and the fixed-point rounding of x
+# (together below 5e-16), and the dense oracle factor's own rounding at n = 256
+# (5e-15, pinned in test_oracle_pins.py).
+TOL = 6e-15
+
+
+def passes(prob, u0, jq=(0, 0)):
+    out = []
+    with S.Plan.for_problem(prob) as plan:
+        for ax in range(prob.dim):
+            u = torch.tensor(np.ascontiguousarray(u0), device="cuda")
+            plan.axis_pass(u, ax, *jq)
+            plan.check()
+            out.append(u.cpu().numpy())
+    return out
+
+
+@pytest.mark.parametrize("n", [(32, 33), (63, 64), (65, 96), (127, 128), (129, 130), (255, 256), (7, 256), (256, 9),
+                               (160, 200), (32, 8, 33), (129, 3, 5)], ids=str)
+def test_lengths_around_the_tile_edges(n):
+    prob = I.Problem(n=n, alpha=(1.2, 1.8, 1.5)[: len(n)], eps=0.08, tau=0.01)
+    u0 = I.random_field(prob, 71, -1.0, 1.0)
+    sch = O.Scheme.for_problem(prob)
+    for ax, got in enumerate(passes(prob, u0)):
+        ref = O.apply_axis(u0, sch.P[ax], ax + 1)
+        assert np.abs(got - ref).max() <= TOL * np.abs(ref).max(), ax
+
+
+@pytest.mark.parametrize("n", [(64, 13, 187), (48, 5, 973), (256, 3, 811), (33, 23, 423), (130, 10, 973)], ids=str)
+def test_tile_widths(n):
+    """Line counts just below and above 16, 32 and 64 times the device's 152
+    SMs, where the tile widens to 16, 32 and 64 lines, with a partly filled last
+    tile; the contiguous axis and the last one."""
+    for m, ax in ((n, 0), ((n[1], n[2], n[0]), 2)):
+        prob = I.Problem(n=m, alpha=(1.3, 1.7, 1.5), eps=0.08, tau=0.01)
+        u0 = I.random_field(prob, 72, -1.0, 1.0)
+        P = O.Scheme.for_problem(I.Problem(n=(n[0],), alpha=(prob.alpha[ax],), eps=0.08, tau=0.01)).P[0]
+        with S.Plan.for_problem(prob) as plan:
+            u = torch.tensor(np.ascontiguousarray(u0), device="cuda")
+            plan.axis_pass(u, ax, 0, 0)
+            plan.check()
+        ref = O.apply_axis(u0, P, ax + 1)
+        assert np.abs(u.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [(64, 16), (256, 16), (16, 256)], ids=str)
+def test_lines_scale_exactly(n):
+    """A line times a power of two gives its result times that power, bit for
+    bit: each line is scaled by its own largest value."""
+    prob = I.Problem(n=n, alpha=(1.4, 1.6), eps=0.1, tau=0.01)
+    ax = int(np.argmax(n))
+    u0 = I.random_field(prob, 73, -1.0, 1.0)
+    k = np.arange(16) * 25 - 200                                   # 2^-200 .. 2^175
+    scale = np.ldexp(1.0, k)
+    scale = scale[:, None] if ax == 0 else scale[None, :]
+    a, b = passes(prob, u0)[ax], passes(prob, u0 * scale)[ax]
+    assert np.array_equal(a * scale, b)
+
+
+def test_zero_and_non_finite_lines():
+    prob = I.Problem(n=(256, 16), alpha=(1.4, 1.6), eps=0.1, tau=0.01)
+    u0 = I.random_field(prob, 74, -1.0, 1.0)
+    want = passes(prob, u0)[0]
+    u0[3] = 0.0
+    u0[5, 17] = np.inf
+    u0[9, 200] = np.nan
+    got = passes(prob, u0)[0]
+    assert np.array_equal(got[3], np.zeros(256))
+    assert np.isnan(got[5]).all() and np.isnan(got[9]).all()
+    rest = [i for i in range(16) if i not in (3, 5, 9)]
+    assert np.array_equal(got[rest], want[rest])
+
+
+@pytest.mark.parametrize("n", [(256, 96), (64, 96)], ids=str)
+def test_wait_runs_out_and_the_plan_stays_usable(n):
+    prob = I.Problem(n=n, alpha=(1.4, 1.6), eps=0.1, tau=1e-2)
+    u0 = I.random_field(prob, 75)
+    with S.Plan.for_problem(prob) as plan:
+        u = torch.tensor(u0, device="cuda")
+        S.sfac_plan_set_wait_limit(plan.handle, 100_000, 1)
+        plan.axis_pass(u, 0, 0, 0)
+        with pytest.raises(S.SfacError) as ei:
+            plan.check()
+        assert ei.value.status == S.sfac.SFAC_ETIMEOUT
+        plan.check()                                  # the flag was cleared
+        S.sfac_plan_set_wait_limit(plan.handle, 1 << 32, 0)
+        a = torch.tensor(u0, device="cuda")
+        plan.axis_pass(a, 0, 1, 2)
+        plan.check()
+    assert np.array_equal(a.cpu().numpy(), passes(prob, u0, (1, 2))[0])
