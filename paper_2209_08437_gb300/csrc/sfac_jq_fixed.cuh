@@ -1,0 +1,66 @@
+// sfac_jq_fixed.cuh - the nonlinear flow J^Q in FP64 precision on the integer pipe.
+//
+// J^Q_s(v) = v / sqrt(E + (1 - E) v^2). In FP64 that is about nine operations of
+// the FP64 pipe a value (half a cycle of a whole SM each on sm_103a); the tensor-core
+// passes leave that pipe idle otherwise, and the flow then took most of their
+// time (n = 256: 76,000 of 160,000 cycles a tile of 64 lines). In 64-bit fixed
+// point it takes about 80 integer operations, which the SM does 64 to 128 of a
+// cycle. Error: below 0.51 units in the last place plus 2^-4 (fixed-point
+// residual of 2^-56).
+#pragma once
+
+#include "sfac_pass.cuh"
+
+namespace sfac {
+
+// Constants of one flow: 1 - E in units of 2^-64, E in units of 2^-60, and both as
+// doubles for the values outside the fixed-point range.
+struct JqFixed {
+    double E, omE;
+    unsigned long long om64, E60;
+    int fixed;  // E >= 1/4: below, s could lose its leading bits
+};
+
+inline __host__ __device__ JqFixed make_jq_fixed(double E, double omE) {
+    JqFixed c;
+    c.E = E;
+    c.omE = omE;
+    c.fixed = E >= 0.25 && omE >= 0.0 && omE <= 0.75;
+    c.om64 = c.fixed ? (unsigned long long)(omE * 18446744073709551616.0) : 0;
+    c.E60 = c.fixed ? (unsigned long long)(E * 1152921504606846976.0) : 0;
+    return c;
+}
+
+__device__ __forceinline__ double jq_flow_fixed(double v, const JqFixed& q) {
+    const int hi = __double2hiint(v);
+    const int ex = (hi >> 20) & 0x7ff;
+    // zero, below 2^-1018, |v| >= 4, infinities and NaN, and large time steps
+    if (!q.fixed || (unsigned)(ex - 5) >= 1020u) return v == 0.0 ? v : jq_flow(v, q.E, q.omE);
+    const unsigned long long m =
+        ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);  // 53 bits
+    // |v| in units of 2^-62, v^2 and s = E + (1 - E) v^2 < 16 in units of 2^-60
+    const int up = ex - 1013;
+    const unsigned long long a = up >= 0 ? m << up : m >> min(-up, 63);
+    const unsigned long long w = __umul64hi(a, a);
+    const unsigned long long s = q.E60 + __umul64hi(w, q.om64);
+    // y0 ~ s^-1/2 from the FP32 unit, in units of 2^-30 (y0 <= 2)
+    const float y0 = rsqrtf(__uint2float_rn((unsigned)(s >> 32)) * 0x1p-28f);
+    const unsigned Y = __float2uint_rn(y0 * 0x1p30f);
+    // e = 1 - s y0^2 (below 2^-21 in size), in units of 2^-56
+    const long long e = (1LL << 56) - (long long)__umul64hi(s, (unsigned long long)Y * Y);
+    // y = y0 (1 + c), c = e/2 + 3 e^2/8; the next term is below 2^-63
+    const int e32 = (int)(e >> 5);
+    const long long c = (e >> 1) + ((__mulhi(e32, e32) * 3) >> 17);
+    // y in units of 2^-62
+    const unsigned long long g = ((unsigned long long)Y << 32) +
+                                 (unsigned long long)(((c >> 32) * (long long)Y) << 8) +
+                                 (((c & 0xffffffffLL) * (unsigned long long)Y) >> 24);
+    // |v| y: 64-bit mantissa product (units of 2^-61 of v's power of two), rounded to 53 bits
+    const unsigned long long r = __umul64hi(m << 11, g);
+    const int lz = __clzll((long long)r);
+    const unsigned long long t = ((r >> (10 - lz)) + 1) >> 1;
+    const long long bits = (long long)t + ((long long)(ex - lz + 1) << 52);
+    return __longlong_as_double(bits | ((long long)(hi & 0x80000000) << 32));
+}
+
+}  // namespace sfac

@@ -12,7 +12,7 @@
 
 #include "sfac.h"
 #include "sfac_internal.h"
-#include "sfac_pass.cuh"
+#include "sfac_jq_fixed.cuh"
 
 namespace {
 
@@ -65,7 +65,8 @@ __global__ void __launch_bounds__(256) jq_probe_kernel(const R* v, R* out, long 
     if (i >= n) return;
     sfac::C2<R> x[1] = {{v[i], i + 1 < n ? v[i + 1] : R(0)}};
     if constexpr (sizeof(R) == 8) {
-        sfac::jq_all<R, 1>(x, E0, om);
+        const sfac::JqFixed q = sfac::make_jq_fixed(E0, om);
+        x[0] = {sfac::jq_flow_fixed(x[0].x, q), sfac::jq_flow_fixed(x[0].y, q)};
     } else {
         const float omf = float(om);
         x[0] = {x[0].x + sfac::jq_increment(x[0].x, omf), x[0].y + sfac::jq_increment(x[0].y, omf)};

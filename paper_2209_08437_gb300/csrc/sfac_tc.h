@@ -16,7 +16,8 @@ struct TcAxis {
     int parts = 0;              // 1: D itself; 2: its even and odd halves
     int rows = 0;               // rows (outputs) per part: n, or ceil(n/2)
     int kp = 0;                 // rows rounded up to a multiple of 32 (K of the products)
-    int scale = 0;              // exponent f: the entries are below 2^(f-1) in size
+    int scale = 0;              // exponent f: the entries are below 2^f in size
+    int headroom = 0;           // more bits above a line's largest value (0 or 1)
 };
 
 // Digits per operand entry, and their width in bits.

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(128) tc_digits(int n, int parts, int rows, int
     const double m = __longlong_as_double((long long)*maxbits);
     int f = 0;
     if (m > 0.0) {
-        f = ilogb(m) + 2;  // m < 2^(f-1)
+        f = ilogb(m) + 1;  // m < 2^f: the top digit has one bit more
         f = f < -200 ? -200 : f;
     }
     if (row == 0 && p == 0 && threadIdx.x == 0) report[0] = f;
@@ -125,24 +125,32 @@ cudaError_t tc_build(int n, const double* g, const double* h, void* img, void* s
 
 bool tc_accept(int n, const void* img, const int* report, TcAxis* ax) {
     // Largest sum the accumulator of order s = i + j can reach: digits of x are at
-    // most 2^(B-1) in size. Orders up to 5 must stay within 2^24 (FP32 holds every
-    // integer of that size), order 6 within 2^25 and orders 7, 8 anywhere: a unit
-    // lost there is below 2^-54 of the line's largest value.
-    for (int s = 2; s <= 6; ++s) {
-        double bound = 0.0;
-        for (int j = 1; j < s; ++j) bound += std::ldexp((double)report[j], B - 1);
-        if (bound > std::ldexp(1.0, s <= 5 ? 24 : 25)) return false;
+    // most 2^(B-1) in size, the top one 2^B, or 2^(B-1) too if lines are scaled by
+    // one more bit. Orders up to 5 must stay within 2^24 (FP32 holds every integer
+    // of that size), order 6 within 2^25 and order 7 anywhere: a unit lost there is
+    // below 2^-56 of the line's largest value.
+    int headroom = -1;
+    for (int h = 0; h < 2 && headroom < 0; ++h) {
+        bool ok = true;
+        for (int s = 2; s <= 6; ++s) {
+            double bound = std::ldexp((double)report[s - 1], B - h);
+            for (int j = 1; j < s - 1; ++j) bound += std::ldexp((double)report[j], B - 1);
+            ok = ok && bound <= std::ldexp(1.0, s <= 5 ? 24 : 25);
+        }
+        if (ok) headroom = h;
     }
+    if (headroom < 0) return false;
     // |sum of a row| / 2^f, so that the 64-bit sums of the pass cannot overflow
     double rowsum = 0.0;
     for (int j = 1; j <= NS; ++j) rowsum += std::ldexp((double)report[j], -B * j);
-    if (rowsum > 8.0 || report[0] > 40) return false;
+    if (rowsum > 4.0 || report[0] > 2) return false;
     ax->img = img;
     ax->n = n;
     ax->parts = parts_of(n);
     ax->rows = rows_of(n);
     ax->kp = kp_of(n);
     ax->scale = report[0];
+    ax->headroom = headroom;
     return true;
 }
 

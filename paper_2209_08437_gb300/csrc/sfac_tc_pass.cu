@@ -11,13 +11,13 @@
 //    54 fractional bits, cut into six signed digits of 9 bits (FP16 integers);
 //    D's entries likewise, once per plan (sfac_tc_build.cu);
 //  - the products of digit place i of x with place j of D are summed by
-//    tcgen05.mma into one FP32 accumulator per order i + j = 2..8. All of them
+//    tcgen05.mma into one FP32 accumulator per order i + j = 2..7. All of them
 //    are whole numbers of at most 2^24, so every sum is exact (tc_accept checks
-//    the bound for the plan's own D); orders from 9 on are below 2^-61;
-//  - the seven sums are added with their weights in 64-bit integers, and
+//    the bound for the plan's own D); orders from 8 on are left out;
+//  - the six sums are added with their weights in 64-bit integers, and
 //    y = x + D x is rounded once.
-// Measured against 80-bit arithmetic the increment is within 1e-16 (2-norm,
-// relative to the line), a fifth of the FFT passes' error.
+// Against 80-bit arithmetic the increment is within 0.1e-16 to 3e-16 (2-norm,
+// relative to the line, for |D| from 0.05 to 2), the FFT passes within 5e-16.
 //
 // Lines of more than 128 points are folded: D is centrosymmetric (C and S are
 // symmetric Toeplitz), so it maps the sums x_k + x_{n-1-k} and the differences
@@ -29,7 +29,7 @@
 // streamed from L2 in 8 KB blocks through a ring of bulk copies.
 #include <atomic>
 
-#include "sfac_pass.cuh"
+#include "sfac_jq_fixed.cuh"
 #include "sfac_tc.h"
 #include "sfac_tcgen05.cuh"
 
@@ -37,64 +37,80 @@ namespace sfac {
 namespace {
 
 constexpr int NS = kTcSlices, DB = kTcBits;
-constexpr int kOrders = 7;        // accumulated orders 2..8
+constexpr int kOrders = 6;        // accumulated orders 2..7
 constexpr unsigned kBlock = 8192;  // a streamed block: 128 rows x 32 columns of FP16
 constexpr unsigned long long kBias = [] {
     unsigned long long b = 0;
     for (int i = 0; i < NS; ++i) b += 1ULL << (DB * i + DB - 1);
-    return b;
+    return b + (1ULL << (DB * NS - 1));  // the top digit has one bit more
 }();
 
-template <int LT>
+template <int PARTS, int LT>
 struct TcShape {
     static constexpr int THREADS = LT >= 64 ? 512 : (LT == 32 ? 256 : 128);
     static constexpr int UPT = LT * 16 / THREADS;       // units (line, 8 columns) a thread holds
-    static constexpr int STAGES = LT >= 64 ? 4 : 6;     // ring of operator blocks
-    static constexpr int LBO = NS * LT * 16 + 16;       // digits: bytes between 8-column chunks (+16: banks)
-    static constexpr int PITCH = LT * 8 + 16;           // results: bytes between rows
-    static constexpr int REGION = LT == 8 ? 8 * LT : kOrders * LT;  // accumulator columns of a part
+    // Digits: bytes between 8-column chunks. Core matrices must stay aligned to
+    // their 128 bytes (16 bytes of padding here made the products 2x slower).
+    static constexpr int LBO = NS * LT * 16;
+    static constexpr int PITCH = LT * 8 + 8;            // results: bytes between rows (8 mod 128: banks)
+    // accumulator columns of a part (LT = 8: a place more, see consume)
+    static constexpr int REGION = LT == 8 ? 8 * LT : kOrders * LT;
     __host__ __device__ static constexpr int part_bytes(int kp) { return kp / 8 * LBO; }
-    __host__ __device__ static constexpr int ring_offset(int parts, int kp) {
-        return (parts * part_bytes(kp) + 127) / 128 * 128;
-    }
-    __host__ __device__ static constexpr int smem(int parts, int kp) {
-        return ring_offset(parts, kp) + STAGES * (int)kBlock;
-    }
+    // Ring of operator blocks: what shared memory the digits leave, at most 24
+    // blocks. A block's copy from L2 takes 1300 to 1800 cycles, so narrow tiles,
+    // whose products are short, want many in flight.
+    static constexpr int RING_OFFSET = PARTS * part_bytes(128);
+    static constexpr int STAGES = (231000 - RING_OFFSET) / (int)kBlock < 24 ? (231000 - RING_OFFSET) / (int)kBlock : 24;
+    static constexpr int SMEM = RING_OFFSET + STAGES * (int)kBlock;
 };
 
-// Order in which a 32-column step visits D's digit places (most significant
-// first = 0): place 5 writes orders 6..8 and place 1 orders 2..5 first, so that
-// the first products of an accumulator can overwrite it.
-__device__ __forceinline__ int place_of(int jj) { return jj == 0 ? 4 : (jj < 5 ? jj - 1 : 5); }
+template <int J>
+struct Place {
+    static constexpr int value = J;
+};
 
-// x rounded to a multiple of 2^-(54 - ..) of the line's scale: |x| 2^(..) with
-// the line's exponent field E and `extra` more bits of headroom.
-__device__ __forceinline__ long long tc_fixed(double v, int E, int extra) {
+// A value of a line whose largest one has the exponent field E, in units of
+// 2^(E - 1082): at most 2^60, the grid far below the FP64 rounding of the
+// line's largest values.
+__device__ __forceinline__ long long tc_fixed(double v, int E) {
     const int hi = __double2hiint(v);
     const int ex = (hi >> 20) & 0x7ff;
     const unsigned mh = (hi & 0xfffff) | (ex ? 0x100000u : 0u);
-    unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(v)) << 1;
-    int sh = E - (ex ? ex : 1) + extra;
+    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(v)) << 8;
+    int sh = E - (ex ? ex : 1);
     sh = sh > 63 ? 63 : sh;
     const long long f = (long long)(((m >> sh) + 1) >> 1);
     return hi < 0 ? -f : f;
 }
 
-// The eight biased values F[0..7] of one line and chunk -> six FP16 digits each,
-// stored as 16-byte rows of the B operand (row = place * LT + line).
-template <int LT>
+// Back to FP64, rounded to nearest (ties away). E >= 64: the result is normal.
+__device__ __forceinline__ double tc_to_double(long long y, int E) {
+    if (y == 0) return 0.0;
+    const unsigned long long m = y < 0 ? 0ULL - (unsigned long long)y : (unsigned long long)y;
+    const int lz = __clzll((long long)m);
+    const unsigned long long t = (((m << lz) >> 10) + 1) >> 1;  // 2^52 .. 2^53
+    const int e = E + 3 - lz;                                   // exponent field less one
+    const long long bits = e >= 2046 ? 0x7ff0000000000000LL : (long long)t + ((long long)e << 52);
+    return __longlong_as_double(bits | (y & (long long)0x8000000000000000ULL));
+}
+
+// The eight biased values F[0..7] of one line and chunk -> six FP16 digits each
+// (the lowest at bit SB), stored as 16-byte rows of the B operand (row = place *
+// LT + line).
+template <int LT, int SB>
 __device__ __forceinline__ void tc_put_digits(unsigned char* chunk, int line, const unsigned long long (&F)[8]) {
 #pragma unroll
     for (int q = 0; q < NS; ++q) {
-        const int sh = DB * (NS - 1 - q);
-        const unsigned mask = q == 0 ? 0x3ffu : 0x1ffu;
+        const int sh = SB + DB * (NS - 1 - q);
+        const unsigned mask = q == 0 ? 0x7ffu : 0x1ffu;
+        const unsigned short off = q == 0 ? 0x6600 : 0x6500;  // 1024 + 512, 1024 + 256
         uint32_t w[4];
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
             const unsigned a = (unsigned)(F[2 * p] >> sh) & mask;
             const unsigned b = (unsigned)(F[2 * p + 1] >> sh) & mask;
-            const unsigned h = a | (b << 16) | 0x64006400u;  // 1024 + field, twice
-            const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6500)));
+            const unsigned h = (a | (b << 16)) + 0x64006400u;  // 1024 + field, twice
+            const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(off)));
             w[p] = *reinterpret_cast<const uint32_t*>(&d);
         }
         const int r = q * LT + line;
@@ -102,12 +118,12 @@ __device__ __forceinline__ void tc_put_digits(unsigned char* chunk, int line, co
     }
 }
 
-// The seven order sums of one output -> the 64-bit integer sum in units of
-// 2^-6 of order 6.
+// The order sums of one output -> the 64-bit integer sum in units of 2^-6 of
+// order 6.
 __device__ __forceinline__ long long tc_combine(const float (&a)[kOrders]) {
     const long long hi = (long long)__float2int_rn(a[0]) * (1 << 18) + (long long)__float2int_rn(a[1]) * (1 << 9) +
                          __float2int_rn(a[2]);
-    const int r = __float2int_rn(fmaf(a[6], 1.f / 4096.f, a[5] * 0.125f));
+    const int r = __float2int_rn(a[5] * 0.125f);
     const long long lo = (long long)__float2int_rn(a[3]) * (1 << 15) + (long long)__float2int_rn(a[4]) * 64 + r;
     return (hi << 24) + lo;
 }
@@ -116,12 +132,13 @@ struct TcArgs {
     PassArgs a;
     const unsigned char* img;
     long long lines, ntiles;
-    int n, rows, kp, scale;
+    int n, rows, kp, scale, headroom;
+    JqFixed jin, jout;
 };
 
 template <int PARTS, int LT, bool STRIDED>
-__global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pass_kernel(const TcArgs g) {
-    using Sh = TcShape<LT>;
+__global__ void __launch_bounds__(TcShape<PARTS, LT>::THREADS, 1) tc_pass_kernel(const TcArgs g) {
+    using Sh = TcShape<PARTS, LT>;
     constexpr int NT = Sh::THREADS, UPT = Sh::UPT, STAGES = Sh::STAGES, LBO = Sh::LBO;
     constexpr int VPU = PARTS == 2 ? 16 : 8;  // values of a unit
     constexpr bool TWO_PHASES = PARTS == 2 && LT >= 64;
@@ -138,7 +155,7 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n = g.n, rows = g.rows, kp = g.kp, nkc = kp >> 5;
     const int part_bytes = Sh::part_bytes(kp);
-    unsigned char* ring = smem + Sh::ring_offset(PARTS, kp);
+    unsigned char* ring = smem + Sh::RING_OFFSET;
     const double* src = static_cast<const double*>(a.u);
     double* dst = static_cast<double*>(a.u) + a.out_shift;
 
@@ -173,25 +190,58 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
         return true;
     };
 
-    const int phase_chunks = (TWO_PHASES ? 1 : PARTS) * nkc * NS;  // ring blocks of a phase
+    // Ring of operator blocks, in the order part, 32-column step, digit place.
+    // Blocks are counted modulo the ring only (one thread issues, one thread
+    // consumes: a 64-bit division in either loop cost more than the products).
+    const int phase_chunks = (TWO_PHASES ? 1 : PARTS) * nkc * NS;
     const int tile_chunks = PARTS * nkc * NS;
     const long long my_tiles = (g.ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
-    const long long total_chunks = my_tiles * tile_chunks;
-    long long produced = 0, consumed = 0;  // consumed: blocks of the finished phases
-
-    auto produce = [&](long long until) -> bool {  // thread 32 only
-        for (; produced < until; ++produced) {
-            const int st = (int)(produced % STAGES);
-            const long long use = produced / STAGES;
-            if (use > 0 && !wait(&bar_empty[st], (unsigned)((use - 1) & 1))) return false;
-            const int c = (int)(produced % tile_chunks);
-            const int block = c / NS * NS + place_of(c % NS);
-            mbar_expect_tx(&bar_full[st], kBlock);
-            bulk_load(ring + st * kBlock, g.img + (size_t)block * kBlock, kBlock, &bar_full[st]);
+    long long to_produce = my_tiles * tile_chunks;  // thread 32: blocks not issued yet
+    int p_stage = 0, p_chunk = 0;                   // thread 32: next stage, block of the tile
+    unsigned p_parity = 1;                          // of bar_empty: the first round passes at once
+    int c_stage = 0;                                // thread 0: next stage
+    unsigned c_parity = 0;
+    auto produce = [&](int count) -> bool {
+        for (; count > 0 && to_produce > 0; --count, --to_produce) {
+            if (!wait(&bar_empty[p_stage], p_parity)) return false;
+            mbar_expect_tx(&bar_full[p_stage], kBlock);
+            bulk_load(ring + p_stage * kBlock, g.img + (size_t)p_chunk * kBlock, kBlock, &bar_full[p_stage]);
+            if (++p_chunk == tile_chunks) p_chunk = 0;
+            if (++p_stage == STAGES) {
+                p_stage = 0;
+                p_parity ^= 1u;
+            }
         }
         return true;
     };
-    if (tid == 32) produce(total_chunks < STAGES ? total_chunks : STAGES);
+    // One 8 KB block: D's digit place J against the places of x, K = 32.
+    const uint64_t a_desc0 = tc_desc(smem_u32(ring), 2048, 128), b_desc0 = tc_desc(smem_u32(smem), LBO, 128);
+    auto consume = [&](auto place, uint32_t d0, uint64_t bd, bool first) -> bool {
+        constexpr int J = decltype(place)::value;
+        constexpr int M = 7 - J;  // places of x: orders J + 1 .. 7
+        // a first MMA of up to W places, then the rest; N is a multiple of 16, so
+        // LT = 8 takes an even number of places, whose last may go to an unused order
+        constexpr int W = LT >= 64 ? (M < 4 ? M : 4) : (LT == 8 ? (M + 1) / 2 * 2 : M);
+        if (!wait(&bar_full[c_stage], c_parity)) return false;
+        const uint64_t ad = a_desc0 + (uint32_t)c_stage * (kBlock >> 4);
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+            const uint64_t b0 = bd + ks * (2 * LBO >> 4);
+            // place 1 reaches every order: its first products overwrite them
+            const uint32_t acc = (J == 1 && ks == 0 && first) ? 0u : 1u;
+            tc_mma_f16(d0 + (J - 1) * LT, ad + ks * (4096 >> 4), b0, tc_idesc_f16(128, W * LT), acc);
+            if constexpr (M > W)
+                tc_mma_f16(d0 + (J - 1 + W) * LT, ad + ks * (4096 >> 4), b0 + (W * LT * 16 >> 4),
+                           tc_idesc_f16(128, (M - W) * LT), acc);
+        }
+        tc_commit(&bar_empty[c_stage]);
+        if (++c_stage == STAGES) {
+            c_stage = 0;
+            c_parity ^= 1u;
+        }
+        return true;
+    };
+    if (tid == 32) produce(STAGES);
 
     unsigned done_parity = 0;
     bool alive = true;
@@ -199,16 +249,19 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
         // ---- load: units (line, chunk c of 8 columns, and their mirror images) ----
         for (int i = tid; i < LT; i += NT) s_max[i] = 0;
         __syncthreads();
-        double x[UPT][VPU];
+        double x[UPT][VPU];  // then, as integers, the fixed-point values
         int uline[UPT], uc[UPT];
         const int nch = kp >> 3;
 #pragma unroll
         for (int it = 0; it < UPT; ++it) {
             const int u = tid + it * NT;
-            const int line = STRIDED ? u % LT : u / nch, c = STRIDED ? u / LT : u % nch;
+            // strided axis: lanes along the lines; contiguous axis: a warp takes
+            // 4 chunks (256 bytes) of 8 lines
+            const int line = STRIDED ? u % LT : (u / 32) % (LT / 8) * 8 + (u & 7);
+            const int c = STRIDED ? u / LT : (u / 32) / (LT / 8) * 4 + ((u >> 3) & 3);
             uline[it] = line;
             uc[it] = c;
-            const bool in_tile = STRIDED ? c < nch : line < LT;
+            const bool in_tile = c < nch;
             if (!in_tile) uline[it] = -1;
             const long long L = tile * LT + line;
 #pragma unroll
@@ -253,7 +306,7 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
             }
             if (a.jq_in) {
 #pragma unroll
-                for (int r = 0; r < VPU; ++r) x[it][r] = jq_flow(x[it][r], a.jq_in_E, a.jq_in_1mE);
+                for (int r = 0; r < VPU; ++r) x[it][r] = jq_flow_fixed(x[it][r], g.jin);
             }
             unsigned m = 0;
 #pragma unroll
@@ -266,20 +319,28 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
 #pragma unroll
         for (int it = 0; it < UPT; ++it) {
             if (uline[it] < 0) continue;
-            const int E = max((int)(s_max[uline[it]] >> 20), Emin);
+            const int E = max((int)(s_max[uline[it]] >> 20), Emin) + g.headroom;
             unsigned char* chunk = smem + uc[it] * LBO;
+#pragma unroll
+            for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(tc_fixed(x[it][r], E));
+            // sums and differences in units of 2^(E - 1075), values themselves in
+            // units of 2^(E - 1076): at most 2^54 in size, rounded
+            constexpr int SB = PARTS == 2 ? 7 : 6;
+            constexpr unsigned long long bias = (kBias << SB) + (1ULL << (SB - 1));
             unsigned long long F[8];
             if constexpr (PARTS == 2) {
 #pragma unroll
-                for (int r = 0; r < 8; ++r) F[r] = kBias + tc_fixed(x[it][r], E, 1) + tc_fixed(x[it][8 + r], E, 1);
-                tc_put_digits<LT>(chunk, uline[it], F);
+                for (int r = 0; r < 8; ++r)
+                    F[r] = bias + __double_as_longlong(x[it][r]) + __double_as_longlong(x[it][8 + r]);
+                tc_put_digits<LT, SB>(chunk, uline[it], F);
 #pragma unroll
-                for (int r = 0; r < 8; ++r) F[r] = kBias + tc_fixed(x[it][r], E, 1) - tc_fixed(x[it][8 + r], E, 1);
-                tc_put_digits<LT>(chunk + part_bytes, uline[it], F);
+                for (int r = 0; r < 8; ++r)
+                    F[r] = bias + __double_as_longlong(x[it][r]) - __double_as_longlong(x[it][8 + r]);
+                tc_put_digits<LT, SB>(chunk + part_bytes, uline[it], F);
             } else {
 #pragma unroll
-                for (int r = 0; r < 8; ++r) F[r] = kBias + tc_fixed(x[it][r], E, 0);
-                tc_put_digits<LT>(chunk, uline[it], F);
+                for (int r = 0; r < 8; ++r) F[r] = bias + __double_as_longlong(x[it][r]);
+                tc_put_digits<LT, SB>(chunk, uline[it], F);
             }
         }
         fence_proxy_async_smem();
@@ -290,42 +351,23 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
             // ---- products ----
             if (tid == 0) {
                 tc_fence_after_sync();
-                long long ci = consumed;
                 bool ok = true;
-                if (a.hold && consumed == 0) ok = wait(&bar_never, 0);
-                for (int b = 0; ok && b < phase_chunks; ++b, ++ci) {
-                    const int jj = b % NS, kcs = b / NS;  // kcs: 32-column step within the phase
-                    const int part = TWO_PHASES ? ph : kcs / nkc, kc = TWO_PHASES ? kcs : kcs % nkc;
-                    const int st = (int)(ci % STAGES);
-                    ok = wait(&bar_full[st], (unsigned)((ci / STAGES) & 1));
-                    if (!ok) break;
-                    const int j = place_of(jj) + 1;  // 1-based digit place of D
+                if (a.hold && tile == blockIdx.x && ph == 0) ok = wait(&bar_never, 0);
+#pragma unroll 1
+                for (int part = TWO_PHASES ? ph : 0; ok && part < (TWO_PHASES ? ph + 1 : PARTS); ++part) {
                     const uint32_t d0 = tmem + (TWO_PHASES ? 0 : part * Sh::REGION);
-                    const uint32_t ab = smem_u32(ring + st * kBlock);
-                    const uint32_t bb = smem_u32(smem) + part * part_bytes + kc * 4 * LBO;
-#pragma unroll
-                    for (int ks = 0; ks < 2; ++ks) {
-                        const uint64_t ad = tc_desc(ab + ks * 4096, 2048, 128);
-                        const uint32_t b0 = bb + ks * 2 * LBO;
-                        const bool first = kc == 0 && ks == 0;
-                        const int m = j <= 2 ? 6 : 8 - j;  // places of x: orders j + 1 .. j + m
-                        // first block of up to `w` places, then the rest
-                        const int w = (LT >= 64 || j == 1) ? (m < 4 ? m : 4) : (LT == 8 ? (m + 1) / 2 * 2 : m);
-                        tc_mma_f16(d0 + (j - 1) * LT, ad, tc_desc(b0, LBO, 128), tc_idesc_f16(128, w * LT),
-                                   (first && (j == 5 || j == 1)) ? 0u : 1u);
-                        if (m > w)
-                            tc_mma_f16(d0 + (j - 1 + w) * LT, ad, tc_desc(b0 + w * LT * 16, LBO, 128),
-                                       tc_idesc_f16(128, (m - w) * LT), 1u);
-                    }
-                    tc_commit(&bar_empty[st]);
+                    uint64_t bd = b_desc0 + (uint32_t)(part * part_bytes >> 4);
+#pragma unroll 1
+                    for (int kc = 0; ok && kc < nkc; ++kc, bd += 4 * LBO >> 4)
+                        ok = consume(Place<1>(), d0, bd, kc == 0) && consume(Place<2>(), d0, bd, kc == 0) &&
+                             consume(Place<3>(), d0, bd, kc == 0) && consume(Place<4>(), d0, bd, kc == 0) &&
+                             consume(Place<5>(), d0, bd, kc == 0) && consume(Place<6>(), d0, bd, kc == 0);
                 }
                 tc_commit(&bar_done);
             } else if (tid == 32) {
-                const long long until = consumed + phase_chunks + STAGES;
-                produce(until < total_chunks ? until : total_chunks);
+                produce(phase_chunks);
             }
             __syncwarp();
-            consumed += phase_chunks;
             if (!wait(&bar_done, done_parity)) alive = false;
             done_parity ^= 1;
             if (!__syncthreads_and(alive && !*reinterpret_cast<volatile int*>(&s_abort))) {
@@ -333,8 +375,7 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
                 break;
             }
             tc_fence_after_sync();
-            // ---- the order sums -> integers, through shared memory (row, line);
-            // lines rotated by row / 8 so that both access patterns spread over the banks
+            // ---- the order sums -> integers, through shared memory (row, line) ----
             {
                 constexpr int GROUPS = NT / 128, CPG = LT / GROUPS < 4 ? 4 : LT / GROUPS;
                 const int row = (warp & 3) * 32 + lane;
@@ -373,7 +414,7 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
                     if (row < kp) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const int off = ((cc + q + (row >> 3)) & (LT - 1)) * 8;
+                            const int off = (cc + q) * 8;
                             long long* p0 = reinterpret_cast<long long*>(r0 + off);
                             long long* p1 = reinterpret_cast<long long*>(r1 + off);
                             if constexpr (PARTS == 1) {
@@ -405,24 +446,27 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
             const long long L = tile * LT + line;
             if (line < 0 || L >= g.lines) continue;
             const int Eb = (int)(s_max[line] >> 20);
-            const int E = max(Eb, Emin);
-            // 2^(E - 1081 + f); NaN for a line that holds an infinity or a NaN
-            const double sc = Eb == 2047 ? __longlong_as_double(0x7ff8000000000000LL)
-                                         : __longlong_as_double((long long)(E - 58 + g.scale) << 52);
+            const int E = max(Eb, Emin) + g.headroom;
+            // the sums are in units of 2^(E - 1082 + f)
+            const int left = max(g.scale, 0), right = min(max(-g.scale, 0), 62);
+            const long long half = right > 0 ? 1LL << (right - 1) : 0;
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-                const int k = 8 * c + r;
-                const int off = k * Sh::PITCH + ((line + c) & (LT - 1)) * 8;
+                const int off = (8 * c + r) * Sh::PITCH + line * 8;
                 const long long v = *reinterpret_cast<const long long*>(smem + off);
-                x[it][r] = fma((double)v, sc, x[it][r]);
+                x[it][r] = tc_to_double(__double_as_longlong(x[it][r]) + ((v << left) + half >> right), E);
                 if constexpr (PARTS == 2) {
                     const long long w = *reinterpret_cast<const long long*>(smem + part_bytes + off);
-                    x[it][8 + r] = fma((double)w, sc, x[it][8 + r]);
+                    x[it][8 + r] = tc_to_double(__double_as_longlong(x[it][8 + r]) + ((w << left) + half >> right), E);
                 }
+            }
+            if (Eb == 2047) {  // a line that holds an infinity or a NaN
+#pragma unroll
+                for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(0x7ff8000000000000LL);
             }
             if (a.jq_out) {
 #pragma unroll
-                for (int r = 0; r < VPU; ++r) x[it][r] = jq_flow(x[it][r], a.jq_out_E, a.jq_out_1mE);
+                for (int r = 0; r < VPU; ++r) x[it][r] = jq_flow_fixed(x[it][r], g.jout);
             }
             if constexpr (STRIDED) {
                 const long long o = L / a.inner, i = L - o * a.inner;
@@ -464,8 +508,12 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
         // a wait ran out: let this CTA's copies and products in flight finish
         // (bounded), record the timeout
         if (tid == 32) {
-            for (long long c = produced > STAGES ? produced - STAGES : 0; c < produced; ++c)
-                mbar_wait_bounded(&bar_full[c % STAGES], (unsigned)((c / STAGES) & 1), a.wait_cycles);
+            // the copies issued last, one a stage at most: each one's phase of bar_full
+            // is the one before the phase its stage would be issued for next
+            for (int st = 0; st < STAGES; ++st) {
+                const unsigned next = st < p_stage ? p_parity ^ 1u : p_parity;  // bar_empty parity of its next use
+                mbar_wait_bounded(&bar_full[st], next, a.wait_cycles);
+            }
             if (a.status) atomicOr(a.status, SFAC_PASS_TIMEOUT);
         }
         if (tid == 0) mbar_wait_bounded(&bar_done, done_parity ^ 1u, a.wait_cycles);
@@ -478,11 +526,11 @@ __global__ void __launch_bounds__(TcShape<LT>::THREADS, LT >= 32 ? 1 : 2) tc_pas
 
 template <int PARTS, int LT, bool STRIDED>
 cudaError_t launch_tc(const TcAxis& ax, const PassArgs& a, long long lines, cudaStream_t s) {
-    using Sh = TcShape<LT>;
+    using Sh = TcShape<PARTS, LT>;
     auto kern = tc_pass_kernel<PARTS, LT, STRIDED>;
     // shared memory is sized for the largest operator, so that one attribute and
     // one resident count hold for every kp (and tensor memory suffices for them)
-    const size_t smem_max = (size_t)Sh::smem(PARTS, 128);
+    const size_t smem_max = Sh::SMEM;
     static LaunchSetup setup;
     int dev = 0, resident = 0;
     cudaError_t err = set_smem(kern, smem_max, setup, &dev);
@@ -497,6 +545,9 @@ cudaError_t launch_tc(const TcAxis& ax, const PassArgs& a, long long lines, cuda
     g.rows = ax.rows;
     g.kp = ax.kp;
     g.scale = ax.scale;
+    g.headroom = ax.headroom;
+    g.jin = make_jq_fixed(a.jq_in_E, a.jq_in_1mE);
+    g.jout = make_jq_fixed(a.jq_out_E, a.jq_out_1mE);
     if (g.ntiles <= 0) return cudaSuccess;
     const long long grid = g.ntiles < resident ? g.ntiles : resident;
     kern<<<(unsigned)grid, Sh::THREADS, smem_max, s>>>(g);
