@@ -31,16 +31,25 @@ inline __host__ __device__ JqFixed make_jq_fixed(double E, double omE) {
     return c;
 }
 
-__device__ __forceinline__ double jq_flow_fixed(double v, const JqFixed& q) {
+// Whether v has the fixed-point form (not: zero, below 2^-1018, |v| >= 4,
+// infinities, NaN; large time steps).
+__device__ __forceinline__ bool jq_in_range(double v, const JqFixed& q) {
+    const int ex = (__double2hiint(v) >> 20) & 0x7ff;
+    return q.fixed && (unsigned)(ex - 5) < 1020u;
+}
+__device__ __forceinline__ double jq_out_of_range(double v, const JqFixed& q) {
+    return v == 0.0 ? v : jq_flow(v, q.E, q.omE);
+}
+
+// The fixed-point form; any value may be passed, the result holds for those in range.
+__device__ __forceinline__ double jq_fixed_body(double v, const JqFixed& q) {
     const int hi = __double2hiint(v);
     const int ex = (hi >> 20) & 0x7ff;
-    // zero, below 2^-1018, |v| >= 4, infinities and NaN, and large time steps
-    if (!q.fixed || (unsigned)(ex - 5) >= 1020u) return v == 0.0 ? v : jq_flow(v, q.E, q.omE);
     const unsigned long long m =
         ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);  // 53 bits
-    // |v| in units of 2^-62, v^2 and s = E + (1 - E) v^2 < 16 in units of 2^-60
+    // |v| (below 4) in units of 2^-62, v^2 and s = E + (1 - E) v^2 < 16 in units of 2^-60
     const int up = ex - 1013;
-    const unsigned long long a = up >= 0 ? m << up : m >> min(-up, 63);
+    const unsigned long long a = (m << 11) >> min(max(11 - up, 0), 63);
     const unsigned long long w = __umul64hi(a, a);
     const unsigned long long s = q.E60 + __umul64hi(w, q.om64);
     // y0 ~ s^-1/2 from the FP32 unit, in units of 2^-30 (y0 <= 2)
@@ -61,6 +70,32 @@ __device__ __forceinline__ double jq_flow_fixed(double v, const JqFixed& q) {
     const unsigned long long t = ((r >> (10 - lz)) + 1) >> 1;
     const long long bits = (long long)t + ((long long)(ex - lz + 1) << 52);
     return __longlong_as_double(bits | ((long long)(hi & 0x80000000) << 32));
+}
+
+__device__ __forceinline__ double jq_flow_fixed(double v, const JqFixed& q) {
+    return jq_in_range(v, q) ? jq_fixed_body(v, q) : jq_out_of_range(v, q);
+}
+
+// V values: the fixed-point forms first, without branches between them (their
+// long chains of dependent operations overlap), then the values out of range.
+template <int V>
+__device__ __forceinline__ void jq_flow_fixed_all(double (&x)[V], const JqFixed& q) {
+    unsigned rare = 0;
+#pragma unroll
+    for (int r = 0; r < V; ++r) {
+        const bool in = jq_in_range(x[r], q);
+        if (!in && x[r] != 0.0) rare |= 1u << r;
+        x[r] = in ? jq_fixed_body(x[r], q) : x[r];
+    }
+    if (rare) {
+#pragma unroll 1
+        for (int r = 0; r < V; ++r) {
+            if (!((rare >> r) & 1u)) continue;
+#pragma unroll
+            for (int s = 0; s < V; ++s)
+                if (s == r) x[s] = jq_out_of_range(x[s], q);
+        }
+    }
 }
 
 }  // namespace sfac

@@ -269,7 +269,14 @@ sfac_status run_steps(sfac_plan* P, void* u, long long nsteps, cudaStream_t st, 
                       void* host_out = nullptr) {
     const int d = P->p.dim;
     if (!host_in && !host_out && steps_used(P, nsteps)) {
-        const cudaError_t err = sfac::launch_steps(P->p.prec, steps_args(P, u, nsteps), st);
+        sfac::TcAxis tc[3];
+        bool all_tc = true;
+        for (int ax = 0; ax < d; ++ax) {
+            tc[ax] = P->ax[ax].tc;
+            all_tc = all_tc && tc[ax].img;
+        }
+        const cudaError_t err = all_tc ? sfac::launch_tc_steps(tc, steps_args(P, u, nsteps), st)
+                                       : sfac::launch_steps(P->p.prec, steps_args(P, u, nsteps), st);
         if (err != cudaSuccess) return cuda_fail(err, "small-grid launch");
         return SFAC_OK;
     }

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "sfac_internal.h"
+#include "sfac_steps.h"
 
 namespace sfac {
 
@@ -44,5 +45,11 @@ bool tc_accept(int n, const void* img, const int* report, TcAxis* ax);
 
 // One FP64 axis pass (the arguments of launch_pass_f64) through the tensor cores.
 cudaError_t launch_pass_tc_f64(const TcAxis& ax, const PassArgs& a, cudaStream_t s);
+
+// The same with tiles of 8 lines (few lines: latency bound).
+cudaError_t launch_pass_tc_small(const TcAxis& ax, const PassArgs& a, cudaStream_t s);
+
+// A whole call on a small grid (as launch_steps) with the operators ax[0..dim-1].
+cudaError_t launch_tc_steps(const TcAxis* ax, const StepsArgs& a, cudaStream_t s);
 
 }  // namespace sfac

@@ -1,0 +1,606 @@
+// sfac_tc_tile.cuh - FP64 lines as exact digit products on the tensor cores.
+//
+// The linear factor of an axis, P = e^{tau/2 C} e^{tau S} e^{tau/2 C}, is a real
+// n x n matrix, and a pass computes y = x + D x, D = P - I, for every line. The
+// FP64 pipe of sm_103a does 4 flops a clock per SM, so the six FFTs of a line
+// were bound by it (93% busy); the tensor cores do 8192 FP16 flops a clock. D x
+// is therefore formed from digits (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, "Error-free transformations of matrix multiplication by using
+// fast routines of matrix multiplication", Numer. Algorithms 59, 2012):
+//  - a line is scaled by a power of two above its largest value and rounded to
+//    54 fractional bits, cut into six signed digits of 9 bits (FP16 integers);
+//    D's entries likewise, once per plan (sfac_tc_build.cu);
+//  - the products of digit place i of x with place j of D are summed by
+//    tcgen05.mma into one FP32 accumulator per order i + j = 2..7. All of them
+//    are whole numbers of at most 2^24, so every sum is exact (tc_accept checks
+//    the bound for the plan's own D); orders from 8 on are left out;
+//  - the six sums are added with their weights in 64-bit integers, and
+//    y = x + D x is rounded once.
+// Against 80-bit arithmetic the increment is within 0.1e-16 to 3e-16 (2-norm,
+// relative to the line, for |D| from 0.05 to 2), the FFT passes within 5e-16.
+//
+// Lines of more than 128 points are folded: D is centrosymmetric (C and S are
+// symmetric Toeplitz), so it maps the sums x_k + x_{n-1-k} and the differences
+// x_k - x_{n-1-k} each into themselves, two operators of half the size (half the
+// products). The operator is the A operand (128 outputs are the M of the MMA),
+// the digits of LT lines are the B operand: digit places stacked along N, so
+// that one MMA multiplies a digit place of D with up to four places of x and
+// writes the orders, neighbouring in tensor memory, in one go. D's digits are
+// streamed from L2 in 8 KB blocks through a ring of bulk copies.
+//
+// A CTA is THREADS computing threads (one warp of them also issues the
+// products) and one more warp that issues the copies of the ring. Both issuing
+// loops run on whole warps with uniform control flow and elect a lane for each
+// instruction: run by a single thread of a divergent branch they took 460
+// cycles a block, four times as long as its products.
+#pragma once
+
+#include "sfac_jq_fixed.cuh"
+#include "sfac_tc.h"
+#include "sfac_tcgen05.cuh"
+
+namespace sfac {
+
+constexpr int kTcOrders = 6;         // accumulated orders 2..7
+constexpr unsigned kTcBlock = 8192;  // a streamed block: 128 rows x 32 columns of FP16
+constexpr int kTcMaxStages = 24;
+
+template <int PARTS, int LT>
+struct TcShape {
+    static constexpr int THREADS = LT >= 64 ? 512 : (LT == 32 ? 256 : 128);
+    static constexpr int UPT = LT * 16 / THREADS;       // units (line, 8 columns) a thread holds
+    // Digits: bytes between 8-column chunks. Core matrices must stay aligned to
+    // their 128 bytes.
+    static constexpr int LBO = kTcSlices * LT * 16;
+    static constexpr int PITCH = LT * 8 + 8;            // results: bytes between rows (8 mod 128: banks)
+    // accumulator columns of a part (LT = 8: a place more, see tc_products)
+    static constexpr int REGION = LT == 8 ? 8 * LT : kTcOrders * LT;
+    // A warp of its own for the ring's copies; with 16 computing warps it would
+    // cost them a quarter of their registers (128 -> 96), there one of them issues
+    // the copies while the others wait for the products.
+    static constexpr bool OWN_PRODUCER = THREADS < 512;
+    static constexpr int TOTAL = THREADS + (OWN_PRODUCER ? 32 : 0);
+    // LT = 64: the accumulators of one part fill tensor memory, the parts run in turn
+    static constexpr bool TWO_PHASES = PARTS == 2 && LT >= 64;
+    static constexpr int COLS = LT >= 64 ? 512 : (PARTS * REGION <= 64 ? 64 : PARTS * REGION <= 128 ? 128
+                                                  : PARTS * REGION <= 256 ? 256 : 512);
+    __host__ __device__ static constexpr int part_bytes(int kp) { return kp / 8 * LBO; }
+    // Ring of operator blocks: what shared memory the digits leave, at most 24.
+    static constexpr int RING_OFFSET = PARTS * part_bytes(128);
+    static constexpr int FIT = (231000 - RING_OFFSET) / (int)kTcBlock;
+    static constexpr int STAGES = FIT < kTcMaxStages ? FIT : kTcMaxStages;
+    static constexpr int SMEM = RING_OFFSET + STAGES * (int)kTcBlock;
+};
+
+// One pass over lines: element k of line L sits at
+// (L / inner) * n * inner + L % inner + k * inner.
+struct TcPass {
+    const double* src;
+    double* dst;
+    long long inner, lines, ntiles;
+    int n, rows, kp, scale, headroom;
+    int jq_in, jq_out;
+    JqFixed jin, jout;
+};
+
+inline TcPass tc_pass_of(const TcAxis& ax, const PassArgs& a) {
+    TcPass p;
+    p.src = static_cast<const double*>(a.u);
+    p.dst = static_cast<double*>(a.u) + a.out_shift;
+    p.inner = a.inner;
+    p.lines = a.outer * a.inner;
+    p.ntiles = 0;
+    p.n = ax.n;
+    p.rows = ax.rows;
+    p.kp = ax.kp;
+    p.scale = ax.scale;
+    p.headroom = ax.headroom;
+    p.jq_in = a.jq_in;
+    p.jq_out = a.jq_out;
+    p.jin = make_jq_fixed(a.jq_in_E, a.jq_in_1mE);
+    p.jout = make_jq_fixed(a.jq_out_E, a.jq_out_1mE);
+    return p;
+}
+
+// Barriers and flags of a CTA, in shared memory.
+struct TcShared {
+    uint64_t full[kTcMaxStages], empty[kTcMaxStages], done, never;
+    uint32_t tmem;
+    int abort;
+};
+
+// Ring and barrier positions of a CTA's warps; every lane of a warp holds the
+// same values. The warp that issues the copies keeps its own ring position, the
+// next block of the image, and how many blocks are still to come.
+struct TcState {
+    int stage = 0;
+    unsigned parity = 0;       // consumer: of full; producer: of empty (starts at 1)
+    unsigned done_parity = 0;
+    int block = 0;
+    long long left = 0;
+};
+
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
+// Waits on `bar` with the whole (converged) warp, at most `limit` cycles; a wait
+// that runs out, or that sees another warp's that did, returns false. NAP: polls
+// seldom (the producer: its polls took issue slots from the other warps).
+template <bool NAP = false>
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, unsigned parity, long long limit, int* abort) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    for (;;) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        const bool late = clock64() - t0 > limit;
+        if (__any_sync(0xffffffffu, late || *reinterpret_cast<volatile int*>(abort) != 0)) {
+            *reinterpret_cast<volatile int*>(abort) = 1;
+            return false;
+        }
+        if (NAP) __nanosleep(100);
+    }
+}
+
+// Barrier 1 among the NT computing threads; the second form also ANDs a flag.
+template <int NT>
+__device__ __forceinline__ void tc_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+}
+template <int NT>
+__device__ __forceinline__ bool tc_sync_and(bool v) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)v), "n"(NT)
+        : "memory");
+    return r != 0;
+}
+
+constexpr unsigned long long kTcBias = [] {
+    unsigned long long b = 0;
+    for (int i = 0; i < kTcSlices; ++i) b += 1ULL << (kTcBits * i + kTcBits - 1);
+    return b + (1ULL << (kTcBits * kTcSlices - 1));  // the top digit has one bit more
+}();
+
+// A value of a line whose largest one has the exponent field E, in units of
+// 2^(E - 1082): at most 2^60, the grid far below the FP64 rounding of the
+// line's largest values.
+__device__ __forceinline__ long long tc_fixed(double v, int E) {
+    const int hi = __double2hiint(v);
+    const int ex = (hi >> 20) & 0x7ff;
+    const unsigned mh = (hi & 0xfffff) | (ex ? 0x100000u : 0u);
+    const unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(v)) << 7;
+    int sh = E - (ex ? ex : 1);
+    sh = sh > 63 ? 63 : sh;
+    const long long f = (long long)(m >> sh);
+    return hi < 0 ? -f : f;
+}
+
+// Back to FP64, rounded to nearest (ties away). E >= 64: the result is normal.
+__device__ __forceinline__ double tc_to_double(long long y, int E) {
+    if (y == 0) return 0.0;
+    const unsigned long long m = y < 0 ? 0ULL - (unsigned long long)y : (unsigned long long)y;
+    const int lz = __clzll((long long)m);
+    const unsigned long long t = (((m << lz) >> 10) + 1) >> 1;  // 2^52 .. 2^53
+    const int e = E + 3 - lz;                                   // exponent field less one
+    const long long bits = e >= 2046 ? 0x7ff0000000000000LL : (long long)t + ((long long)e << 52);
+    return __longlong_as_double(bits | (y & (long long)0x8000000000000000ULL));
+}
+
+// Digit place q (0: most significant) of two biased values whose lowest digit is at
+// bit SB, as two FP16 integers.
+template <int SB>
+__device__ __forceinline__ uint32_t tc_digit_pair(unsigned long long f0, unsigned long long f1, int q) {
+    const int sh = SB + kTcBits * (kTcSlices - 1 - q);
+    const unsigned mask = q == 0 ? 0x7ffu : 0x1ffu;
+    const unsigned short off = q == 0 ? 0x6600 : 0x6500;  // 1024 + 512, 1024 + 256
+    const unsigned a = (unsigned)(f0 >> sh) & mask, b = (unsigned)(f1 >> sh) & mask;
+    const unsigned h = (a | (b << 16)) + 0x64006400u;  // 1024 + field, twice
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(off)));
+    return *reinterpret_cast<const uint32_t*>(&d);
+}
+
+// The eight biased values F[0..7] of one line and chunk -> six FP16 digits each,
+// stored as 16-byte rows of the B operand (row = place * LT + line).
+template <int LT, int SB>
+__device__ __forceinline__ void tc_put_digits(unsigned char* chunk, int line, const unsigned long long (&F)[8]) {
+#pragma unroll
+    for (int q = 0; q < kTcSlices; ++q) {
+        const int r = q * LT + line;
+        *reinterpret_cast<uint4*>(chunk + (r >> 3) * 128 + (r & 7) * 16) =
+            make_uint4(tc_digit_pair<SB>(F[0], F[1], q), tc_digit_pair<SB>(F[2], F[3], q),
+                       tc_digit_pair<SB>(F[4], F[5], q), tc_digit_pair<SB>(F[6], F[7], q));
+    }
+}
+
+// A sum in units of 2^(E - 1082 + f) in units of 2^(E - 1082), rounded.
+__device__ __forceinline__ long long tc_align(long long v, int f) {
+    if (f >= 0) return v << f;
+    const int right = min(-f, 62);
+    return (v + (1LL << (right - 1))) >> right;
+}
+
+// The order sums of one output -> the 64-bit integer sum in units of 2^-6 of
+// order 6.
+__device__ __forceinline__ long long tc_combine(const float (&a)[kTcOrders]) {
+    const long long hi = (long long)__float2int_rn(a[0]) * (1 << 18) + (long long)__float2int_rn(a[1]) * (1 << 9) +
+                         __float2int_rn(a[2]);
+    const int r = __float2int_rn(a[5] * 0.125f);
+    const long long lo = (long long)__float2int_rn(a[3]) * (1 << 15) + (long long)__float2int_rn(a[4]) * 64 + r;
+    return (hi << 24) + lo;
+}
+
+template <bool CG, typename T>
+__device__ __forceinline__ T tc_ld(const T* p) {
+    if constexpr (CG) return __ldcg(p);
+    else return *p;
+}
+
+// The producer: up to `count` more blocks of an image of tile_chunks blocks.
+template <int STAGES>
+__device__ __forceinline__ bool tc_produce(TcShared& sh, TcState& st, unsigned char* ring, const unsigned char* img,
+                                           int tile_chunks, long long count, long long limit) {
+    if (count > st.left) count = st.left;
+#pragma unroll 1
+    for (long long c = 0; c < count; ++c) {
+        if (!tc_wait<true>(&sh.empty[st.stage], st.parity, limit, &sh.abort)) return false;
+        if (elect_one()) {
+            mbar_expect_tx(&sh.full[st.stage], kTcBlock);
+            bulk_load(ring + st.stage * kTcBlock, img + (size_t)st.block * kTcBlock, kTcBlock, &sh.full[st.stage]);
+        }
+        __syncwarp();
+        --st.left;
+        if (++st.block == tile_chunks) st.block = 0;
+        if (++st.stage == STAGES) {
+            st.stage = 0;
+            st.parity ^= 1u;
+        }
+    }
+    return true;
+}
+
+// The products of parts [part0, part1), issued by one whole warp; they arrive on
+// sh.done. A block holds one digit place J of D for 32 columns; it meets the
+// places 1 .. 7 - J of x (orders J + 1 .. 7). One compact loop: unrolled over the
+// places, a narrow tile spent most of the time fetching instructions.
+template <int PARTS, int LT, int STAGES>
+__device__ __forceinline__ void tc_products(TcShared& sh, TcState& st, unsigned char* digits, unsigned char* ring,
+                                            uint32_t tmem, int part0, int part1, int kp, long long limit) {
+    using Sh = TcShape<PARTS, LT>;
+    const uint64_t a0 = tc_desc(smem_u32(ring), 2048, 128), b0 = tc_desc(smem_u32(digits), Sh::LBO, 128);
+    const int blocks = (kp >> 5) * kTcSlices;
+    bool ok = true;
+#pragma unroll 1
+    for (int part = part0; ok && part < part1; ++part) {
+        const uint32_t d0 = tmem + (Sh::TWO_PHASES ? 0 : part * Sh::REGION);
+        uint64_t bd = b0 + (uint32_t)(part * Sh::part_bytes(kp) >> 4);
+        int j = 0;  // J - 1
+        uint32_t later = 0;
+#pragma unroll 1
+        for (int b = 0; b < blocks; ++b) {
+            ok = tc_wait(&sh.full[st.stage], st.parity, limit, &sh.abort);
+            if (!ok) break;
+            const uint64_t ad = a0 + (uint32_t)(st.stage * (kTcBlock >> 4));
+            const int m = 6 - j;
+            // N is a multiple of 16 (LT = 8: an even number of places, whose last may
+            // go to an unused order) and at most 256 (LT = 64: 4 places, then the rest)
+            const int w = LT >= 64 ? min(m, 4) : (LT == 8 ? (m + 1) & ~1 : m);
+            const uint32_t d = d0 + j * LT;
+            const uint32_t idesc = tc_idesc_f16(128, 0) + ((uint32_t)(w * LT) >> 3 << 17);
+            // place 1 reaches every order: its first products overwrite them
+            const uint32_t acc = j == 0 ? later : 1u;
+            if (elect_one()) {
+                tc_mma_f16(d, ad, bd, idesc, acc);
+                if (LT >= 64 && m > 4)
+                    tc_mma_f16(d + 4 * LT, ad, bd + (4 * LT * 16 >> 4),
+                               tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), acc);
+                tc_mma_f16(d, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4), idesc, 1u);
+                if (LT >= 64 && m > 4)
+                    tc_mma_f16(d + 4 * LT, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4) + (4 * LT * 16 >> 4),
+                               tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), 1u);
+                tc_commit(&sh.empty[st.stage]);
+            }
+            __syncwarp();
+            if (++st.stage == STAGES) {
+                st.stage = 0;
+                st.parity ^= 1u;
+            }
+            if (++j == kTcSlices) {
+                j = 0;
+                later = 1;
+                bd += 4 * Sh::LBO >> 4;
+            }
+        }
+    }
+    if (elect_one()) tc_commit(&sh.done);
+    __syncwarp();
+}
+
+// One tile of LT lines, by the computing threads: false if a wait ran out.
+// smem: the digits (then the results); smax: LT words.
+template <int PARTS, int LT, bool STRIDED, bool CG, int STAGES>
+__device__ __forceinline__ bool tc_tile(const TcPass& g, long long tile, unsigned char* smem, unsigned char* ring,
+                                        unsigned* smax, TcShared& sh, TcState& st, uint32_t tmem,
+                                        const unsigned char* img, int tid, long long limit) {
+    using Sh = TcShape<PARTS, LT>;
+    constexpr int NT = Sh::THREADS, UPT = Sh::UPT, LBO = Sh::LBO;
+    constexpr int VPU = PARTS == 2 ? 16 : 8;  // values of a unit
+    constexpr bool TWO_PHASES = Sh::TWO_PHASES;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int n = g.n, rows = g.rows, kp = g.kp;
+    const int part_bytes = Sh::part_bytes(kp);
+
+    // ---- load: units (line, chunk c of 8 columns, and their mirror images) ----
+    for (int i = tid; i < LT; i += NT) smax[i] = 0;
+    tc_sync<NT>();
+    double x[UPT][VPU];  // then, as integers, the fixed-point values
+    int uline[UPT], uc[UPT];
+    const int nch = kp >> 3;
+#pragma unroll
+    for (int it = 0; it < UPT; ++it) {
+        const int u = tid + it * NT;
+        // strided axis: lanes along the lines; contiguous axis: a warp takes
+        // 4 chunks (256 bytes) of 8 lines
+        const int line = STRIDED ? u % LT : (u / 32) % (LT / 8) * 8 + (u & 7);
+        const int c = STRIDED ? u / LT : (u / 32) / (LT / 8) * 4 + ((u >> 3) & 3);
+        uline[it] = line;
+        uc[it] = c;
+        const bool in_tile = c < nch;
+        if (!in_tile) uline[it] = -1;
+        const long long L = tile * LT + line;
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) x[it][r] = 0.0;
+        if (in_tile && L < g.lines) {
+            if constexpr (STRIDED) {
+                const long long o = L / g.inner, i = L - o * g.inner;
+                const double* p = g.src + o * n * g.inner + i;
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const int k = 8 * c + r;
+                    if (k < rows) {
+                        x[it][r] = tc_ld<CG>(p + (long long)k * g.inner);
+                        if constexpr (PARTS == 2) x[it][8 + r] = tc_ld<CG>(p + (long long)(n - 1 - k) * g.inner);
+                    }
+                }
+            } else {
+                const double* p = g.src + L * n;
+                if ((n & 1) == 0 && 8 * c + 8 <= rows) {
+#pragma unroll
+                    for (int r = 0; r < 8; r += 2) {
+                        const double2 v = tc_ld<CG>(reinterpret_cast<const double2*>(p + 8 * c + r));
+                        x[it][r] = v.x;
+                        x[it][r + 1] = v.y;
+                        if constexpr (PARTS == 2) {
+                            const double2 w = tc_ld<CG>(reinterpret_cast<const double2*>(p + n - 2 - 8 * c - r));
+                            x[it][8 + r] = w.y;
+                            x[it][9 + r] = w.x;
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) {
+                        const int k = 8 * c + r;
+                        if (k < rows) {
+                            x[it][r] = tc_ld<CG>(p + k);
+                            if constexpr (PARTS == 2) x[it][8 + r] = tc_ld<CG>(p + n - 1 - k);
+                        }
+                    }
+                }
+            }
+        }
+        if (g.jq_in) {
+            jq_flow_fixed_all(x[it], g.jin);
+        }
+        unsigned m = 0;
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) m = max(m, (unsigned)__double2hiint(x[it][r]) & 0x7fffffffu);
+        if (in_tile) atomicMax(&smax[line], m);
+    }
+    tc_sync<NT>();
+    // ---- digits ----
+    const int Emin = max(1, 64 - g.scale);
+#pragma unroll
+    for (int it = 0; it < UPT; ++it) {
+        if (uline[it] < 0) continue;
+        const int E = max((int)(smax[uline[it]] >> 20), Emin) + g.headroom;
+        unsigned char* chunk = smem + uc[it] * LBO;
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(tc_fixed(x[it][r], E));
+        // sums and differences in units of 2^(E - 1075), values themselves in
+        // units of 2^(E - 1076): at most 2^54 in size, rounded
+        constexpr int SB = PARTS == 2 ? 7 : 6;
+        constexpr unsigned long long bias = (kTcBias << SB) + (1ULL << (SB - 1));
+        unsigned long long F[8];
+        if constexpr (PARTS == 2) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+                F[r] = bias + __double_as_longlong(x[it][r]) + __double_as_longlong(x[it][8 + r]);
+            tc_put_digits<LT, SB>(chunk, uline[it], F);
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+                F[r] = bias + __double_as_longlong(x[it][r]) - __double_as_longlong(x[it][8 + r]);
+            tc_put_digits<LT, SB>(chunk + part_bytes, uline[it], F);
+        } else {
+#pragma unroll
+            for (int r = 0; r < 8; ++r) F[r] = bias + __double_as_longlong(x[it][r]);
+            tc_put_digits<LT, SB>(chunk, uline[it], F);
+        }
+    }
+    fence_proxy_async_smem();
+    tc_sync<NT>();
+
+#pragma unroll 1
+    for (int ph = 0; ph < (TWO_PHASES ? 2 : 1); ++ph) {
+        // ---- products: the other warps wait at the barrier, not polling ----
+        bool ok = true;
+        if (warp == 0) {
+            tc_fence_after_sync();
+            tc_products<PARTS, LT, STAGES>(sh, st, smem, ring, tmem, TWO_PHASES ? ph : 0, TWO_PHASES ? ph + 1 : PARTS,
+                                           kp, limit);
+            ok = tc_wait(&sh.done, st.done_parity, limit, &sh.abort);
+        }
+        if (!Sh::OWN_PRODUCER && warp == 1)
+            tc_produce<STAGES>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices,
+                               (TWO_PHASES ? 1 : PARTS) * (kp >> 5) * kTcSlices, limit);
+        st.done_parity ^= 1u;
+        if (!tc_sync_and<NT>(ok && *reinterpret_cast<volatile int*>(&sh.abort) == 0)) return false;
+        tc_fence_after_sync();
+        // ---- the order sums -> integers, through shared memory (row, line) ----
+        {
+            constexpr int GROUPS = NT / 128, CPG = LT / GROUPS < 4 ? 4 : LT / GROUPS;
+            const int row = (warp & 3) * 32 + lane;
+            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+            const int col0 = (warp >> 2) * CPG;
+            unsigned char* r0 = smem + row * Sh::PITCH;
+            unsigned char* r1 = smem + part_bytes + row * Sh::PITCH;
+#pragma unroll 1
+            for (int cc = col0; cc < col0 + CPG; cc += 4) {
+                __syncwarp();
+                uint32_t t[kTcOrders][4];
+#pragma unroll
+                for (int s = 0; s < kTcOrders; ++s) tmem_ld4(taddr + s * LT + cc, t[s]);
+                tc_wait_ld();
+                long long v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float f[kTcOrders];
+#pragma unroll
+                    for (int s = 0; s < kTcOrders; ++s) f[s] = __uint_as_float(t[s][q]);
+                    v[q] = tc_combine(f);
+                }
+                long long w[4];
+                if constexpr (PARTS == 2 && !TWO_PHASES) {
+#pragma unroll
+                    for (int s = 0; s < kTcOrders; ++s) tmem_ld4(taddr + Sh::REGION + s * LT + cc, t[s]);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float f[kTcOrders];
+#pragma unroll
+                        for (int s = 0; s < kTcOrders; ++s) f[s] = __uint_as_float(t[s][q]);
+                        w[q] = tc_combine(f);
+                    }
+                }
+                if (row < kp) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int off = (cc + q) * 8;
+                        long long* p0 = reinterpret_cast<long long*>(r0 + off);
+                        long long* p1 = reinterpret_cast<long long*>(r1 + off);
+                        if constexpr (PARTS == 1) {
+                            *p0 = v[q];
+                        } else if constexpr (TWO_PHASES) {
+                            if (ph == 0) {
+                                *p0 = v[q];
+                            } else {
+                                const long long e = *p0;
+                                *p0 = e + v[q];
+                                *p1 = e - v[q];
+                            }
+                        } else {
+                            *p0 = v[q] + w[q];
+                            *p1 = v[q] - w[q];
+                        }
+                    }
+                }
+            }
+        }
+        tc_fence_before_sync();
+        tc_sync<NT>();
+    }
+    // ---- y = x + D x, the closing flow, store ----
+#pragma unroll
+    for (int it = 0; it < UPT; ++it) {
+        const int line = uline[it], c = uc[it];
+        const long long L = tile * LT + line;
+        if (line < 0 || L >= g.lines) continue;
+        const int Eb = (int)(smax[line] >> 20);
+        const int E = max(Eb, Emin) + g.headroom;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int off = (8 * c + r) * Sh::PITCH + line * 8;
+            const long long v = *reinterpret_cast<const long long*>(smem + off);
+            x[it][r] = tc_to_double(__double_as_longlong(x[it][r]) + tc_align(v, g.scale), E);
+            if constexpr (PARTS == 2) {
+                const long long w = *reinterpret_cast<const long long*>(smem + part_bytes + off);
+                x[it][8 + r] = tc_to_double(__double_as_longlong(x[it][8 + r]) + tc_align(w, g.scale), E);
+            }
+        }
+        if (Eb == 2047) {  // a line that holds an infinity or a NaN
+#pragma unroll
+            for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(0x7ff8000000000000LL);
+        }
+        if (g.jq_out) {
+            jq_flow_fixed_all(x[it], g.jout);
+        }
+        if constexpr (STRIDED) {
+            const long long o = L / g.inner, i = L - o * g.inner;
+            double* p = g.dst + o * n * g.inner + i;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int k = 8 * c + r;
+                if (k < rows) {
+                    p[(long long)k * g.inner] = x[it][r];
+                    if constexpr (PARTS == 2) p[(long long)(n - 1 - k) * g.inner] = x[it][8 + r];
+                }
+            }
+        } else {
+            double* p = g.dst + L * n;
+            if ((n & 1) == 0 && 8 * c + 8 <= rows) {
+#pragma unroll
+                for (int r = 0; r < 8; r += 2) {
+                    *reinterpret_cast<double2*>(p + 8 * c + r) = make_double2(x[it][r], x[it][r + 1]);
+                    if constexpr (PARTS == 2)
+                        *reinterpret_cast<double2*>(p + n - 2 - 8 * c - r) =
+                            make_double2(x[it][9 + r], x[it][8 + r]);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const int k = 8 * c + r;
+                    if (k < rows) {
+                        p[k] = x[it][r];
+                        if constexpr (PARTS == 2) p[n - 1 - k] = x[it][8 + r];
+                    }
+                }
+            }
+        }
+    }
+    tc_sync<NT>();  // results and smax are rewritten by the next tile
+    return true;
+}
+
+// Sets up a CTA: tensor memory (warp 0), barriers. All threads of the CTA.
+template <int COLS, int STAGES>
+__device__ __forceinline__ uint32_t tc_setup(TcShared& sh) {
+    if (threadIdx.x < 32) tmem_alloc(&sh.tmem, COLS);
+    if (threadIdx.x == 32) {
+        for (int i = 0; i < STAGES; ++i) {
+            mbar_init(&sh.full[i], 1);
+            mbar_init(&sh.empty[i], 1);
+        }
+        mbar_init(&sh.done, 1);
+        mbar_init(&sh.never, 1);
+        sh.abort = 0;
+        fence_mbar_init();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    return sh.tmem;
+}
+
+// A wait of the CTA ran out: before it leaves, its copies and products in flight
+// finish (waits bounded again) and the timeout is recorded. `st` of the producer
+// warp: the last copy of a stage is the one before the stage's next use.
+template <int STAGES>
+__device__ __forceinline__ void tc_drain_copies(TcShared& sh, const TcState& st, long long limit) {
+    for (int i = 0; i < STAGES; ++i)
+        mbar_wait_bounded(&sh.full[i], i < st.stage ? st.parity ^ 1u : st.parity, limit);
+}
+
+}  // namespace sfac
