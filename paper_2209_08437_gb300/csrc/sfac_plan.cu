@@ -177,7 +177,8 @@ sfac_status launch_axis(sfac_plan* P, void* u, int ax, int jq_in, int jq_out, cu
     const int N = P->ax[ax].fft_len;
     cudaError_t err;
     if (P->ax[ax].tc.img) {
-        err = sfac::launch_pass_tc_f64(P->ax[ax].tc, a, st);
+        err = P->p.prec == SFAC_FP64 ? sfac::launch_pass_tc_f64(P->ax[ax].tc, a, st)
+                                     : sfac::launch_pass_tc_f32(P->ax[ax].tc, a, st);
     } else if (P->ax[ax].padded) {
         err = (P->p.prec == SFAC_FP64) ? sfac::launch_pass_padded_f64(N, a, st) : sfac::launch_pass_padded_f32(N, a, st);
     } else if (P->p.prec == SFAC_FP64) {
@@ -270,7 +271,7 @@ sfac_status run_steps(sfac_plan* P, void* u, long long nsteps, cudaStream_t st, 
     const int d = P->p.dim;
     if (!host_in && !host_out && steps_used(P, nsteps)) {
         sfac::TcAxis tc[3];
-        bool all_tc = true;
+        bool all_tc = P->p.prec == SFAC_FP64;
         for (int ax = 0; ax < d; ++ax) {
             tc[ax] = P->ax[ax].tc;
             all_tc = all_tc && tc[ax].img;
@@ -381,13 +382,20 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
                 const int N = padded[l] ? pad[l].L : params->n[l];
                 const int E = sfac::f64_elems_per_thread(N);
                 if (E <= 16) rtw[l] = sfac::ratio_twiddles(N, E);
-                tc[l] = params->n[l] >= sfac::kTcMinN && params->n[l] <= sfac::kTcMaxN;
-                if (tc[l]) sfac::increment_columns(host[l], params->tau, &gcol[l], &hcol[l]);
             }
         } catch (const std::bad_alloc&) {
             delete P;
             return fail(SFAC_ENOMEM, "host allocation failed");
         }
+    }
+    try {
+        for (int l = 0; l < params->dim; ++l) {
+            tc[l] = params->prec == SFAC_FP64 && params->n[l] >= sfac::kTcMinN && params->n[l] <= sfac::kTcLongMaxN;
+            if (tc[l]) sfac::increment_columns(host[l], params->tau, &gcol[l], &hcol[l]);
+        }
+    } catch (const std::bad_alloc&) {
+        delete P;
+        return fail(SFAC_ENOMEM, "host allocation failed");
     }
     // One device block: per axis eC[n], eS[n], twist[2n], twid[2n] reals, the
     // FP64 diagnostic tables, and the ratio twiddles.
@@ -422,11 +430,12 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     total += align256(2 * sizeof(unsigned int));
     // Not part of the upload: the digit images of the tensor-core passes and the
     // builder's scratch (used by one axis after the other).
+    const int slices = params->prec == SFAC_FP64 ? sfac::kTcSlices : sfac::kTcSlices32;
     size_t off_img[3] = {0, 0, 0}, alloc = total, scratch = 0;
     for (int l = 0; l < params->dim; ++l) {
         if (!tc[l]) continue;
         off_img[l] = alloc;
-        alloc += align256(sfac::tc_image_bytes(params->n[l]));
+        alloc += align256(sfac::tc_image_bytes(params->n[l], slices));
         scratch = std::max(scratch, sfac::tc_scratch_bytes(params->n[l]));
     }
     const size_t off_scratch = alloc;
@@ -495,7 +504,8 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     err = cudaMemcpyAsync(P->dev_tables, blob.data(), total, cudaMemcpyHostToDevice, st_);
     for (int l = 0; l < params->dim && err == cudaSuccess; ++l)
         if (tc[l])
-            err = sfac::tc_build(params->n[l], reinterpret_cast<const double*>(base + off[l][9]),
+            err = sfac::tc_build(params->n[l], slices, params->prec == SFAC_FP64 ? sfac::kTcBits : sfac::kTcBits32,
+                                 reinterpret_cast<const double*>(base + off[l][9]),
                                  reinterpret_cast<const double*>(base + off[l][10]), base + off_img[l],
                                  base + off_scratch, report[l], st_);
     if (err == cudaSuccess) err = cudaStreamSynchronize(st_);
@@ -505,7 +515,7 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
         return cuda_fail(err, "table upload");
     }
     for (int l = 0; l < params->dim; ++l)
-        if (tc[l]) sfac::tc_accept(params->n[l], base + off_img[l], report[l], &P->ax[l].tc);
+        if (tc[l]) sfac::tc_accept(params->n[l], slices, base + off_img[l], report[l], &P->ax[l].tc);
     for (int l = 0; l < params->dim; ++l) {
         P->ax[l].eC = base + off[l][0];
         P->ax[l].eS = base + off[l][1];

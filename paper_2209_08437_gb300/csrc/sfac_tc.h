@@ -21,32 +21,38 @@ struct TcAxis {
     int headroom = 0;           // more bits above a line's largest value (0 or 1)
 };
 
-// Digits per operand entry, and their width in bits.
-constexpr int kTcSlices = 6;
-constexpr int kTcBits = 9;
-// Lengths with a tensor-core FP64 pass.
+// Digits per operand entry, and their width in bits: FP64, FP32.
+constexpr int kTcSlices = 6, kTcBits = 9;
+constexpr int kTcSlices32 = 3, kTcBits32 = 10;
+// Lengths with a tensor-core pass.
 constexpr int kTcMinN = 32, kTcMaxN = 256;
+// FP64 lines above kTcMaxN take clusters of CTAs (sfac_tc_long.cu).
+constexpr int kTcLongMaxN = 1024;
 
 // Device bytes of the digit image of an axis of n points, and of the scratch
 // the builder needs (n x n doubles twice, and a few words).
-size_t tc_image_bytes(int n);
+size_t tc_image_bytes(int n, int slices);
 size_t tc_scratch_bytes(int n);
 
 // Builds the image from the first columns g, h (device, n doubles each) of
 // e^{tau/2 C} - I and e^{tau S} - I, on stream s. The host words
-// report[0..6] receive, after the stream is synchronised: the scale exponent,
-// then for each digit place the largest sum of |digit| over a row.
-cudaError_t tc_build(int n, const double* g, const double* h, void* img, void* scratch, int* report_host,
-                     cudaStream_t s);
+// report[0..7] receive, after the stream is synchronised: the scale exponent,
+// then for each of six digit places the largest sum of |digit| over a row's
+// 128 columns, and the largest row sum of |entries| in units of 2^(f - 10).
+cudaError_t tc_build(int n, int slices, int bits, const double* g, const double* h, void* img, void* scratch,
+                     int* report_host, cudaStream_t s);
 
 // Fills *ax from the builder's report; false where the sums could leave the
 // range in which the products are exact (the axis then keeps its FFT pass).
-bool tc_accept(int n, const void* img, const int* report, TcAxis* ax);
+bool tc_accept(int n, int slices, const void* img, const int* report, TcAxis* ax);
 
-// One FP64 axis pass (the arguments of launch_pass_f64) through the tensor cores.
+// One axis pass (the arguments of launch_pass_f64 / _f32) through the tensor cores.
 cudaError_t launch_pass_tc_f64(const TcAxis& ax, const PassArgs& a, cudaStream_t s);
+cudaError_t launch_pass_tc_f32(const TcAxis& ax, const PassArgs& a, cudaStream_t s);
 
-// The same with tiles of 8 lines (few lines: latency bound).
+// FP64 lines of 257 to 1024 points.
+cudaError_t launch_pass_tc_long(const TcAxis& ax, const PassArgs& a, cudaStream_t s);
+// FP64 up to 256 points with tiles of 8 lines (few lines: latency bound).
 cudaError_t launch_pass_tc_small(const TcAxis& ax, const PassArgs& a, cudaStream_t s);
 
 // A whole call on a small grid (as launch_steps) with the operators ax[0..dim-1].

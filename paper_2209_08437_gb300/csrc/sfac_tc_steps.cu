@@ -303,7 +303,7 @@ cudaError_t launch_small(TcStepsArgs& g, const TcAxis* ax, const PassArgs* pa, b
     if (err != cudaSuccess) return err;
     long long grid = 1;
     for (int l = 0; l < g.dim; ++l) {
-        g.ax[l] = tc_pass_of(ax[l], pa[l]);
+        g.ax[l] = tc_pass_of<double>(ax[l], pa[l]);
         g.ax[l].ntiles = (g.ax[l].lines + kLT - 1) / kLT;
         g.img[l] = static_cast<const unsigned char*>(ax[l].img);
         g.parts[l] = ax[l].parts;

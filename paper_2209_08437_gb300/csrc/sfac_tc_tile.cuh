@@ -45,48 +45,55 @@ constexpr int kTcOrders = 6;         // accumulated orders 2..7
 constexpr unsigned kTcBlock = 8192;  // a streamed block: 128 rows x 32 columns of FP16
 constexpr int kTcMaxStages = 24;
 
-template <int PARTS, int LT>
+// S: digit places (6: FP64, 3: FP32).
+template <int PARTS, int LT, int S = kTcSlices>
 struct TcShape {
+    static constexpr int SLICES = S;
     static constexpr int THREADS = LT >= 64 ? 512 : (LT == 32 ? 256 : 128);
     static constexpr int UPT = LT * 16 / THREADS;       // units (line, 8 columns) a thread holds
     // Digits: bytes between 8-column chunks. Core matrices must stay aligned to
     // their 128 bytes.
-    static constexpr int LBO = kTcSlices * LT * 16;
-    static constexpr int PITCH = LT * 8 + 8;            // results: bytes between rows (8 mod 128: banks)
+    static constexpr int LBO = S * LT * 16;
+    static constexpr int PITCH = S == 6 ? LT * 8 + 8 : LT * 4 + 4;  // results: bytes between rows (padded: banks)
     // accumulator columns of a part (LT = 8: a place more, see tc_products)
-    static constexpr int REGION = LT == 8 ? 8 * LT : kTcOrders * LT;
+    static constexpr int REGION = LT == 8 ? (S == 6 ? 8 : 4) * LT : S * LT;
     // A warp of its own for the ring's copies; with 16 computing warps it would
     // cost them a quarter of their registers (128 -> 96), there one of them issues
     // the copies while the others wait for the products.
     static constexpr bool OWN_PRODUCER = THREADS < 512;
     static constexpr int TOTAL = THREADS + (OWN_PRODUCER ? 32 : 0);
     // LT = 64: the accumulators of one part fill tensor memory, the parts run in turn
-    static constexpr bool TWO_PHASES = PARTS == 2 && LT >= 64;
-    static constexpr int COLS = LT >= 64 ? 512 : (PARTS * REGION <= 64 ? 64 : PARTS * REGION <= 128 ? 128
-                                                  : PARTS * REGION <= 256 ? 256 : 512);
+    static constexpr bool TWO_PHASES = PARTS == 2 && S * PARTS * LT > 512;
+    static constexpr int NEED = (TWO_PHASES ? 1 : PARTS) * REGION;
+    static constexpr int COLS = NEED <= 64 ? 64 : NEED <= 128 ? 128 : NEED <= 256 ? 256 : 512;
     __host__ __device__ static constexpr int part_bytes(int kp) { return kp / 8 * LBO; }
     // Ring of operator blocks: what shared memory the digits leave, at most 24.
+    static constexpr int CTAS = S == 6 || LT >= 64 ? 1 : 2;  // resident CTAs an SM
     static constexpr int RING_OFFSET = PARTS * part_bytes(128);
-    static constexpr int FIT = (231000 - RING_OFFSET) / (int)kTcBlock;
+    static constexpr int FIT = (231000 / CTAS - 2000 * (CTAS - 1) - RING_OFFSET) / (int)kTcBlock;
     static constexpr int STAGES = FIT < kTcMaxStages ? FIT : kTcMaxStages;
     static constexpr int SMEM = RING_OFFSET + STAGES * (int)kTcBlock;
 };
 
 // One pass over lines: element k of line L sits at
 // (L / inner) * n * inner + L % inner + k * inner.
-struct TcPass {
-    const double* src;
-    double* dst;
+template <typename R>
+struct TcPassT {
+    const R* src;
+    R* dst;
     long long inner, lines, ntiles;
     int n, rows, kp, scale, headroom;
     int jq_in, jq_out;
     JqFixed jin, jout;
 };
 
-inline TcPass tc_pass_of(const TcAxis& ax, const PassArgs& a) {
-    TcPass p;
-    p.src = static_cast<const double*>(a.u);
-    p.dst = static_cast<double*>(a.u) + a.out_shift;
+using TcPass = TcPassT<double>;
+
+template <typename R>
+inline TcPassT<R> tc_pass_of(const TcAxis& ax, const PassArgs& a) {
+    TcPassT<R> p;
+    p.src = static_cast<const R*>(a.u);
+    p.dst = static_cast<R*>(a.u) + a.out_shift;
     p.inner = a.inner;
     p.lines = a.outer * a.inner;
     p.ntiles = 0;
@@ -265,14 +272,14 @@ __device__ __forceinline__ bool tc_produce(TcShared& sh, TcState& st, unsigned c
 
 // The products of parts [part0, part1), issued by one whole warp; they arrive on
 // sh.done. A block holds one digit place J of D for 32 columns; it meets the
-// places 1 .. 7 - J of x (orders J + 1 .. 7). One compact loop: unrolled over the
+// places 1 .. S + 1 - J of x (orders J + 1 .. S + 1). One compact loop: unrolled over the
 // places, a narrow tile spent most of the time fetching instructions.
-template <int PARTS, int LT, int STAGES>
+template <int PARTS, int LT, int STAGES, int S = kTcSlices>
 __device__ __forceinline__ void tc_products(TcShared& sh, TcState& st, unsigned char* digits, unsigned char* ring,
                                             uint32_t tmem, int part0, int part1, int kp, long long limit) {
-    using Sh = TcShape<PARTS, LT>;
+    using Sh = TcShape<PARTS, LT, S>;
     const uint64_t a0 = tc_desc(smem_u32(ring), 2048, 128), b0 = tc_desc(smem_u32(digits), Sh::LBO, 128);
-    const int blocks = (kp >> 5) * kTcSlices;
+    const int blocks = (kp >> 5) * S;
     bool ok = true;
 #pragma unroll 1
     for (int part = part0; ok && part < part1; ++part) {
@@ -285,21 +292,21 @@ __device__ __forceinline__ void tc_products(TcShared& sh, TcState& st, unsigned 
             ok = tc_wait(&sh.full[st.stage], st.parity, limit, &sh.abort);
             if (!ok) break;
             const uint64_t ad = a0 + (uint32_t)(st.stage * (kTcBlock >> 4));
-            const int m = 6 - j;
+            const int m = S - j;
             // N is a multiple of 16 (LT = 8: an even number of places, whose last may
             // go to an unused order) and at most 256 (LT = 64: 4 places, then the rest)
-            const int w = LT >= 64 ? min(m, 4) : (LT == 8 ? (m + 1) & ~1 : m);
+            const int w = S * LT > 256 ? min(m, 4) : (LT == 8 ? (m + 1) & ~1 : m);
             const uint32_t d = d0 + j * LT;
             const uint32_t idesc = tc_idesc_f16(128, 0) + ((uint32_t)(w * LT) >> 3 << 17);
             // place 1 reaches every order: its first products overwrite them
             const uint32_t acc = j == 0 ? later : 1u;
             if (elect_one()) {
                 tc_mma_f16(d, ad, bd, idesc, acc);
-                if (LT >= 64 && m > 4)
+                if (S * LT > 256 && m > 4)
                     tc_mma_f16(d + 4 * LT, ad, bd + (4 * LT * 16 >> 4),
                                tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), acc);
                 tc_mma_f16(d, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4), idesc, 1u);
-                if (LT >= 64 && m > 4)
+                if (S * LT > 256 && m > 4)
                     tc_mma_f16(d + 4 * LT, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4) + (4 * LT * 16 >> 4),
                                tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), 1u);
                 tc_commit(&sh.empty[st.stage]);
@@ -309,7 +316,7 @@ __device__ __forceinline__ void tc_products(TcShared& sh, TcState& st, unsigned 
                 st.stage = 0;
                 st.parity ^= 1u;
             }
-            if (++j == kTcSlices) {
+            if (++j == S) {
                 j = 0;
                 later = 1;
                 bd += 4 * Sh::LBO >> 4;

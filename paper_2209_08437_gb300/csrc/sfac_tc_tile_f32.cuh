@@ -1,0 +1,234 @@
+// sfac_tc_tile_f32.cuh - FP32 lines as digit products on the tensor cores.
+//
+// As sfac_tc_tile.cuh, in FP32 precision: three digits of 10 bits of x (30 bits
+// of the line's scale) times three of D, orders 2..4 (six products). y = x + D x
+// keeps x in FP32, so only the increment sees the fixed point; the order sums are
+// combined by FP32 multiply-adds, and the nonlinear flow is the increment form
+// of the FP32 passes: y = x0 + (all increments), rounded once.
+#pragma once
+
+#include "sfac_tc_tile.cuh"
+
+namespace sfac {
+
+constexpr unsigned kTcBias32 = (1u << 29) + (1u << 19) + (1u << 9);
+
+// Two biased values -> digit place q as two FP16 integers.
+__device__ __forceinline__ uint32_t tc_digit_pair32(unsigned f0, unsigned f1, int q) {
+    const int sh = kTcBits32 * (kTcSlices32 - 1 - q);
+    const unsigned mask = q == 0 ? 0x7ffu : 0x3ffu;
+    const unsigned h = (((f0 >> sh) & mask) | (((f1 >> sh) & mask) << 16)) + 0x64006400u;  // 1024 + field
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6600)));
+    return *reinterpret_cast<const uint32_t*>(&d);
+}
+
+template <int LT>
+__device__ __forceinline__ void tc_put_digits32(unsigned char* chunk, int line, const unsigned (&F)[8]) {
+#pragma unroll
+    for (int q = 0; q < kTcSlices32; ++q) {
+        const int r = q * LT + line;
+        *reinterpret_cast<uint4*>(chunk + (r >> 3) * 128 + (r & 7) * 16) =
+            make_uint4(tc_digit_pair32(F[0], F[1], q), tc_digit_pair32(F[2], F[3], q),
+                       tc_digit_pair32(F[4], F[5], q), tc_digit_pair32(F[6], F[7], q));
+    }
+}
+
+// One tile of LT lines, by the computing threads: false if a wait ran out.
+template <int PARTS, int LT, bool STRIDED, int STAGES>
+__device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long tile, unsigned char* smem,
+                                            unsigned char* ring, unsigned* smax, TcShared& sh, TcState& st,
+                                            uint32_t tmem, const unsigned char* img, int tid, long long limit) {
+    using Sh = TcShape<PARTS, LT, kTcSlices32>;
+    constexpr int NT = Sh::THREADS, UPT = Sh::UPT, LBO = Sh::LBO;
+    constexpr int VPU = PARTS == 2 ? 16 : 8;
+    static_assert(!Sh::TWO_PHASES, "both parts' accumulators fit");
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int n = g.n, rows = g.rows, kp = g.kp;
+    const int part_bytes = Sh::part_bytes(kp);
+
+    // ---- load: units (line, chunk c of 8 columns, and their mirror images) ----
+    for (int i = tid; i < LT; i += NT) smax[i] = 0;
+    tc_sync<NT>();
+    float x[UPT][VPU], d[UPT][VPU];  // x0 and its increments so far
+    int uline[UPT], uc[UPT];
+    const int nch = kp >> 3;
+    const bool vec = !STRIDED && (n & 3) == 0;
+#pragma unroll
+    for (int it = 0; it < UPT; ++it) {
+        const int u = tid + it * NT;
+        // strided axis: lanes along the lines; contiguous axis: a warp takes
+        // 4 chunks (128 bytes) of 8 lines
+        const int line = STRIDED ? u % LT : (u / 32) % (LT / 8) * 8 + (u & 7);
+        const int c = STRIDED ? u / LT : (u / 32) / (LT / 8) * 4 + ((u >> 3) & 3);
+        const bool in_tile = c < nch;
+        uline[it] = in_tile ? line : -1;
+        uc[it] = c;
+        const long long L = tile * LT + line;
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) x[it][r] = d[it][r] = 0.f;
+        if (in_tile && L < g.lines) {
+            const long long o = STRIDED ? L / g.inner : L, i = STRIDED ? L - o * g.inner : 0;
+            const float* p = g.src + (STRIDED ? o * n * g.inner + i : L * n);
+            const long long stride = STRIDED ? g.inner : 1;
+            if (vec && 8 * c + 8 <= rows) {
+#pragma unroll
+                for (int r = 0; r < 8; r += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(p + 8 * c + r);
+                    x[it][r] = v.x, x[it][r + 1] = v.y, x[it][r + 2] = v.z, x[it][r + 3] = v.w;
+                    if constexpr (PARTS == 2) {
+                        const float4 w = *reinterpret_cast<const float4*>(p + n - 4 - 8 * c - r);
+                        x[it][8 + r] = w.w, x[it][9 + r] = w.z, x[it][10 + r] = w.y, x[it][11 + r] = w.x;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const int k = 8 * c + r;
+                    if (k < rows) {
+                        x[it][r] = p[k * stride];
+                        if constexpr (PARTS == 2) x[it][8 + r] = p[(n - 1 - k) * stride];
+                    }
+                }
+            }
+        }
+        if (g.jq_in) {
+            const float om = (float)g.jin.omE;
+#pragma unroll
+            for (int r = 0; r < VPU; ++r) d[it][r] = jq_increment(x[it][r], om);
+        }
+        unsigned m = 0;
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) m = max(m, __float_as_uint(x[it][r] + d[it][r]) & 0x7fffffffu);
+        if (in_tile) atomicMax(&smax[line], m);
+    }
+    tc_sync<NT>();
+    // ---- digits: x in units of 2^(E - 154) (parts) or 2^(E - 155), sums below 2^29 ----
+    constexpr int Emin = 28;
+#pragma unroll
+    for (int it = 0; it < UPT; ++it) {
+        if (uline[it] < 0) continue;
+        const int E = max((int)(smax[uline[it]] >> 23), Emin);
+        const float m = __uint_as_float((unsigned)((PARTS == 2 ? 281 : 282) - E) << 23);
+        unsigned char* chunk = smem + uc[it] * LBO;
+        int X[VPU];
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) X[r] = __float2int_rn(fmaf(x[it][r], m, d[it][r] * m));
+        unsigned F[8];
+        if constexpr (PARTS == 2) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r) F[r] = kTcBias32 + (unsigned)(X[r] + X[8 + r]);
+            tc_put_digits32<LT>(chunk, uline[it], F);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) F[r] = kTcBias32 + (unsigned)(X[r] - X[8 + r]);
+            tc_put_digits32<LT>(chunk + part_bytes, uline[it], F);
+        } else {
+#pragma unroll
+            for (int r = 0; r < 8; ++r) F[r] = kTcBias32 + (unsigned)X[r];
+            tc_put_digits32<LT>(chunk, uline[it], F);
+        }
+    }
+    fence_proxy_async_smem();
+    tc_sync<NT>();
+    // ---- products: the other warps wait at the barrier, not polling ----
+    bool ok = true;
+    if (warp == 0) {
+        tc_fence_after_sync();
+        tc_products<PARTS, LT, STAGES, kTcSlices32>(sh, st, smem, ring, tmem, 0, PARTS, kp, limit);
+        ok = tc_wait(&sh.done, st.done_parity, limit, &sh.abort);
+    }
+    if (!Sh::OWN_PRODUCER && warp == 1)
+        tc_produce<STAGES>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices32, PARTS * (kp >> 5) * kTcSlices32, limit);
+    st.done_parity ^= 1u;
+    if (!tc_sync_and<NT>(ok && *reinterpret_cast<volatile int*>(&sh.abort) == 0)) return false;
+    tc_fence_after_sync();
+    // ---- the order sums, combined, through shared memory (row, line) ----
+    {
+        constexpr int GROUPS = NT / 128, CPG = LT / GROUPS;
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const int col0 = (warp >> 2) * CPG;
+        // 2^f, the operator's scale
+        const float w2 = __uint_as_float((unsigned)(127 + g.scale) << 23), w3 = w2 * 0x1p-10f, w4 = w2 * 0x1p-20f;
+        float* r0 = reinterpret_cast<float*>(smem + row * Sh::PITCH);
+        float* r1 = reinterpret_cast<float*>(smem + part_bytes + row * Sh::PITCH);
+#pragma unroll 1
+        for (int cc = col0; cc < col0 + CPG; cc += 4) {
+            __syncwarp();
+            uint32_t t[PARTS][kTcSlices32][4];
+#pragma unroll
+            for (int p = 0; p < PARTS; ++p)
+#pragma unroll
+                for (int s = 0; s < kTcSlices32; ++s) tmem_ld4(taddr + p * Sh::REGION + s * LT + cc, t[p][s]);
+            tc_wait_ld();
+            if (row < kp) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float v[PARTS];
+#pragma unroll
+                    for (int p = 0; p < PARTS; ++p)
+                        v[p] = fmaf(__uint_as_float(t[p][2][q]), w4,
+                                    fmaf(__uint_as_float(t[p][1][q]), w3, __uint_as_float(t[p][0][q]) * w2));
+                    if constexpr (PARTS == 2) {
+                        r0[cc + q] = v[0] + v[1];
+                        r1[cc + q] = v[0] - v[1];
+                    } else {
+                        r0[cc + q] = v[0];
+                    }
+                }
+            }
+        }
+    }
+    tc_fence_before_sync();
+    tc_sync<NT>();
+    // ---- y = x0 + increments, the closing flow, store ----
+#pragma unroll
+    for (int it = 0; it < UPT; ++it) {
+        const int line = uline[it], c = uc[it];
+        const long long L = tile * LT + line;
+        if (line < 0 || L >= g.lines) continue;
+        const int Eb = (int)(smax[line] >> 23);
+        // the sums are in units of 2^(E - 145); NaN for a line that holds an infinity or a NaN
+        const float sc = Eb == 255 ? __uint_as_float(0x7fc00000u)
+                                   : __uint_as_float((unsigned)(max(Eb, Emin) - 18) << 23);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int off = (8 * c + r) * Sh::PITCH + line * 4;
+            d[it][r] = fmaf(*reinterpret_cast<const float*>(smem + off), sc, d[it][r]);
+            if constexpr (PARTS == 2)
+                d[it][8 + r] = fmaf(*reinterpret_cast<const float*>(smem + part_bytes + off), sc, d[it][8 + r]);
+        }
+        if (g.jq_out) {
+            const float om = (float)g.jout.omE;
+#pragma unroll
+            for (int r = 0; r < VPU; ++r) d[it][r] += jq_increment(x[it][r] + d[it][r], om);
+        }
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) x[it][r] += d[it][r];
+        const long long o = STRIDED ? L / g.inner : L, i = STRIDED ? L - o * g.inner : 0;
+        float* p = g.dst + (STRIDED ? o * n * g.inner + i : L * n);
+        const long long stride = STRIDED ? g.inner : 1;
+        if (vec && 8 * c + 8 <= rows) {
+#pragma unroll
+            for (int r = 0; r < 8; r += 4) {
+                *reinterpret_cast<float4*>(p + 8 * c + r) =
+                    make_float4(x[it][r], x[it][r + 1], x[it][r + 2], x[it][r + 3]);
+                if constexpr (PARTS == 2)
+                    *reinterpret_cast<float4*>(p + n - 4 - 8 * c - r) =
+                        make_float4(x[it][11 + r], x[it][10 + r], x[it][9 + r], x[it][8 + r]);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int k = 8 * c + r;
+                if (k < rows) {
+                    p[k * stride] = x[it][r];
+                    if constexpr (PARTS == 2) p[(n - 1 - k) * stride] = x[it][8 + r];
+                }
+            }
+        }
+    }
+    tc_sync<NT>();  // results and smax are rewritten by the next tile
+    return true;
+}
+
+}  // namespace sfac

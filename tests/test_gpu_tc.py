@@ -1,7 +1,8 @@
-"""FP64 passes of 32..256 points on the tensor cores (csrc/sfac_tc_pass.cu):
-the edges of their tiles (lengths around the folding limit 128 and the K step
-32, odd lengths, line counts around the tile widths 8..64), the scaling of each
-line, non-finite values, and the bounded wait."""
+"""FP64 passes of 32..1024 points on the tensor cores (csrc/sfac_tc_*.cu):
+the edges of their tiles (lengths around the folding limit 128, the K step 32,
+the cluster limits 256, 512 and 768, odd lengths, line counts around the tile
+widths 8..64), the scaling of each line, non-finite values, and the bounded
+wait."""
 import numpy as np
 import pytest
 
@@ -57,7 +58,45 @@ def test_tile_widths(n):
         assert np.abs(u.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
 
 
-@pytest.mark.parametrize("n", [(64, 16), (256, 16), (16, 256)], ids=str)
+@pytest.mark.parametrize("n", [(257, 33), (33, 258), (300, 31), (511, 3), (512, 32), (16, 513), (769, 9), (1023, 2),
+                               (40, 1024), (3, 1000, 11)], ids=str)
+def test_long_lines(n):
+    """257..1024 points: a cluster of 2, 3 or 4 CTAs per tile of 32 lines (partly
+    filled row blocks, 32-column steps and tiles). Reference: the spectral route
+    (1.1e-15 per application at n = 1024, pinned in test_oracle_pins.py) plus the
+    pass's own 6e-16."""
+    prob = I.Problem(n=n, alpha=(1.3, 1.7, 1.5)[: len(n)], eps=0.05, tau=1e-3)
+    u0 = I.random_field(prob, 76, -1.0, 1.0)
+    ax = int(np.argmax(n))
+    one = I.Problem(n=(n[ax],), alpha=(prob.alpha[ax],), eps=0.05, tau=1e-3)
+    sch = O.Scheme.for_problem(one)
+    got = passes(prob, u0)[ax]
+    lines = np.moveaxis(u0, len(n) - 1 - ax, -1).reshape(-1, n[ax])
+    ref = np.stack([O.apply_axis(v, sch.P[0], 1) for v in lines[:: max(1, len(lines) // 7)]])
+    mine = np.moveaxis(got, len(n) - 1 - ax, -1).reshape(-1, n[ax])[:: max(1, len(lines) // 7)]
+    # (the dense factor's rounding at n = 1024: 1.5e-14, pinned likewise)
+    assert np.abs(mine - ref).max() <= 2e-14 * np.abs(ref).max()
+    if jq_matters(prob):
+        u = torch.tensor(np.ascontiguousarray(u0), device="cuda")
+        with S.Plan.for_problem(prob) as plan:
+            plan.axis_pass(u, ax, 1, 2)
+            plan.check()
+        flowed = O.nonlinear_flow(ref_all(u0, sch, ax, len(n), 0.5 * prob.tau), prob.tau)
+        assert np.abs(u.cpu().numpy() - flowed).max() <= 2e-14 * np.abs(flowed).max()
+
+
+def jq_matters(prob):
+    return prob.points <= 40000
+
+
+def ref_all(u0, sch, ax, dim, s):
+    v = np.moveaxis(O.nonlinear_flow(u0, s), dim - 1 - ax, -1)
+    shape = v.shape
+    out = np.stack([O.apply_axis(w, sch.P[0], 1) for w in v.reshape(-1, shape[-1])]).reshape(shape)
+    return np.moveaxis(out, -1, dim - 1 - ax)
+
+
+@pytest.mark.parametrize("n", [(64, 16), (256, 16), (16, 256), (600, 16), (16, 600)], ids=str)
 def test_lines_scale_exactly(n):
     """A line times a power of two gives its result times that power, bit for
     bit: each line is scaled by its own largest value."""
@@ -85,7 +124,21 @@ def test_zero_and_non_finite_lines():
     assert np.array_equal(got[rest], want[rest])
 
 
-@pytest.mark.parametrize("n", [(256, 96), (64, 96)], ids=str)
+def test_non_finite_long_lines():
+    prob = I.Problem(n=(600, 40), alpha=(1.4, 1.6), eps=0.1, tau=0.01)
+    u0 = I.random_field(prob, 77, -1.0, 1.0)
+    want = passes(prob, u0, (1, 1))[0]
+    u0[3] = 0.0
+    u0[5, 17] = np.inf
+    u0[39, 400] = np.nan
+    got = passes(prob, u0, (1, 1))[0]
+    assert np.array_equal(got[3], np.zeros(600))
+    assert np.isnan(got[5]).all() and np.isnan(got[39]).all()
+    rest = [i for i in range(40) if i not in (3, 5, 39)]
+    assert np.array_equal(got[rest], want[rest])
+
+
+@pytest.mark.parametrize("n", [(256, 96), (64, 96), (600, 96), (64, 3000 // 2)], ids=str)
 def test_wait_runs_out_and_the_plan_stays_usable(n):
     prob = I.Problem(n=n, alpha=(1.4, 1.6), eps=0.1, tau=1e-2)
     u0 = I.random_field(prob, 75)
