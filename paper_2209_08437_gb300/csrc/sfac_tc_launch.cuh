@@ -35,12 +35,12 @@ tc_pass_kernel(const TcArgs<R> g) {
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     TcState st;
     const int producer = Sh::OWN_PRODUCER ? NT / 32 : 1;
-    const int tile_chunks = PARTS * (g.pass.kp >> 5) * kSlicesOf<R>;
+    const int stages = PARTS * (g.pass.kp >> 5) * kSlicesOf<R> / Sh::G;  // of the operator
     if (warp == producer) {
         st.parity = 1;
-        st.left = (g.pass.ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x * tile_chunks;
-        tc_produce<Sh::STAGES>(sh, st, ring, g.img, tile_chunks, Sh::OWN_PRODUCER ? st.left : Sh::STAGES,
-                               g.wait_cycles);
+        st.left = (g.pass.ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x * stages;
+        tc_produce<Sh::STAGES, Sh::G>(sh, st, ring, g.img, stages, Sh::OWN_PRODUCER ? st.left : Sh::STAGES,
+                                      g.wait_cycles);
     }
     if (warp < NT / 32) {
         // the test hook: a barrier that nothing completes

@@ -30,10 +30,10 @@ constexpr int kThreads = kNT + 64;
 constexpr int kStepBytes = Shape::part_bytes(32);  // digits of 32 columns of one part
 constexpr int kBuffers = 2;
 constexpr int kRing = kBuffers * 2 * kStepBytes;
-constexpr int kStages = 21;
-constexpr int kSmem = kRing + kStages * (int)kTcBlock;
+constexpr int kG = 3, kStages = 7;    // a stage: kG blocks of the operator
+constexpr int kSmem = kRing + kStages * kG * (int)kTcBlock;
 constexpr int kPitch = kLT * 8 + 8;  // results, in the ring's place: bytes between rows
-static_assert(kSmem <= 231000 && kStages <= kTcMaxStages && 2 * 128 * kPitch <= kStages * (int)kTcBlock, "smem");
+static_assert(kSmem <= 231000 && kStages <= kTcMaxStages && 2 * 128 * kPitch <= kStages * kG * (int)kTcBlock, "smem");
 
 struct TcLongArgs {
     TcPass pass;
@@ -87,9 +87,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
     if (warp == kNT / 32) {
         // ---- the copies ----
         st.parity = 1;
-        st.left = (long long)nkc * 2 * kTcSlices;
+        st.left = nkc * 2 * kTcSlices / kG;
         const unsigned char* img = g.img + (size_t)rank * nkc * 2 * kTcSlices * kTcBlock;
-        tc_produce<kStages>(sh, st, smem + kRing, img, nkc * 2 * kTcSlices, st.left, limit);
+        tc_produce<kStages, kG>(sh, st, smem + kRing, img, nkc * 2 * kTcSlices / kG, st.left, limit);
     } else if (warp == kNT / 32 + 1) {
         // ---- the products ----
         if (g.hold) alive = tc_wait(&sh.never, 0, limit, &sh.abort);  // the test hook
@@ -105,26 +105,29 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
             int j = 0;
             uint32_t d0 = tmem;
 #pragma unroll 1
-            for (int b = 0; alive && b < 2 * kTcSlices; ++b) {
+            for (int b = 0; alive && b < 2 * kTcSlices / kG; ++b) {
                 alive = tc_wait(&sh.full[st.stage], st.parity, limit, &sh.abort);
                 if (!alive) break;
-                const uint64_t ad = a0 + (uint32_t)(st.stage * (kTcBlock >> 4));
-                const uint32_t idesc = tc_idesc_f16(128, 0) + ((uint32_t)((kTcSlices - j) * kLT) >> 3 << 17);
-                const uint32_t acc = j == 0 && (kc & 3) == 0 ? 0u : 1u;
-                if (elect_one()) {
-                    tc_mma_f16(d0 + j * kLT, ad, bd, idesc, acc);
-                    tc_mma_f16(d0 + j * kLT, ad + (4096 >> 4), bd + (2 * Shape::LBO >> 4), idesc, 1u);
-                    tc_commit(&sh.empty[st.stage]);
+                uint64_t ad = a0 + (uint32_t)(st.stage * (kG * kTcBlock >> 4));
+#pragma unroll 1
+                for (int q = 0; q < kG; ++q, ad += kTcBlock >> 4) {
+                    const uint32_t idesc = tc_idesc_f16(128, 0) + ((uint32_t)((kTcSlices - j) * kLT) >> 3 << 17);
+                    const uint32_t acc = j == 0 && (kc & 3) == 0 ? 0u : 1u;
+                    if (elect_one()) {
+                        tc_mma_f16(d0 + j * kLT, ad, bd, idesc, acc);
+                        tc_mma_f16(d0 + j * kLT, ad + (4096 >> 4), bd + (2 * Shape::LBO >> 4), idesc, 1u);
+                        if (q == kG - 1) tc_commit(&sh.empty[st.stage]);
+                    }
+                    __syncwarp();
+                    if (++j == kTcSlices) {
+                        j = 0;
+                        d0 += Shape::REGION;
+                        bd += kStepBytes >> 4;
+                    }
                 }
-                __syncwarp();
                 if (++st.stage == kStages) {
                     st.stage = 0;
                     st.parity ^= 1u;
-                }
-                if (++j == kTcSlices) {
-                    j = 0;
-                    d0 += Shape::REGION;
-                    bd += kStepBytes >> 4;
                 }
             }
             if (elect_one()) {

@@ -11,7 +11,7 @@
 // Whole calls: as in sfac_steps.cu a cooperative launch runs every step of the
 // call and the CTAs meet at a grid-wide barrier between axis passes. The
 // operators do not depend on the field, so the warp that streams them runs
-// ahead, through the barriers, by up to 192 KB: the products of a pass find
+// ahead, through the barriers, by up to 168 KB: the products of a pass find
 // their operator in shared memory.
 #include <cuda_runtime.h>
 
@@ -28,8 +28,8 @@ constexpr int kNT = 256;  // computing threads; one more warp issues the copies
 // Shared memory: digits (then results), the lines' values, the ring.
 constexpr int kXArea = Shape2::RING_OFFSET;                  // 2 parts x 64 pairs x 8 lines x 16 bytes
 constexpr int kRing = kXArea + 2 * 64 * 128;
-constexpr int kStages = 23;
-constexpr int kSmem = kRing + kStages * (int)kTcBlock;
+constexpr int kG = 3, kStages = 7;  // a stage: kG blocks
+constexpr int kSmem = kRing + kStages * kG * (int)kTcBlock;
 static_assert(kStages <= kTcMaxStages && kSmem <= 231000, "shared memory");
 
 struct TcStepsArgs {
@@ -153,7 +153,7 @@ __device__ __forceinline__ bool tc_small_tile(const TcPass& g, long long tile, u
     bool ok = true;
     if (warp == 0) {
         tc_fence_after_sync();
-        tc_products<PARTS, kLT, kStages>(sh, st, smem, smem + kRing, tmem, 0, PARTS, kp, limit);
+        tc_products<PARTS, kLT, kStages, kG>(sh, st, smem, smem + kRing, tmem, 0, PARTS, kp, limit);
         ok = tc_wait(&sh.done, st.done_parity, limit, &sh.abort);
     }
     st.done_parity ^= 1u;
@@ -242,10 +242,10 @@ __global__ void __launch_bounds__(kNT + 32, 1) tc_steps_kernel(const TcStepsArgs
         st.parity = 1;
         for (long long s = 0; alive && s < g.nsteps; ++s)
             for (int ax = 0; alive && ax < g.dim; ++ax) {
-                const int chunks = g.parts[ax] * (g.ax[ax].kp >> 5) * kTcSlices;
+                const int stages = g.parts[ax] * (g.ax[ax].kp >> 5) * kTcSlices / kG;
                 for (long long tile = blockIdx.x; alive && tile < g.ax[ax].ntiles; tile += gridDim.x) {
-                    st.left = chunks;
-                    alive = tc_produce<kStages>(sh, st, smem + kRing, g.img[ax], chunks, chunks, g.wait_cycles);
+                    st.left = stages;
+                    alive = tc_produce<kStages, kG>(sh, st, smem + kRing, g.img[ax], stages, stages, g.wait_cycles);
                 }
             }
     } else {

@@ -67,12 +67,15 @@ struct TcShape {
     static constexpr int NEED = (TWO_PHASES ? 1 : PARTS) * REGION;
     static constexpr int COLS = NEED <= 64 ? 64 : NEED <= 128 ? 128 : NEED <= 256 ? 256 : 512;
     __host__ __device__ static constexpr int part_bytes(int kp) { return kp / 8 * LBO; }
-    // Ring of operator blocks: what shared memory the digits leave, at most 24.
+    // Ring of operator blocks: what shared memory the digits leave, at most 24
+    // blocks. Where it is deep enough a stage is three blocks: the waits of either
+    // side cost about 200 cycles a stage, more than one block's products.
     static constexpr int CTAS = S == 6 || LT >= 64 ? 1 : 2;  // resident CTAs an SM
     static constexpr int RING_OFFSET = PARTS * part_bytes(128);
     static constexpr int FIT = (231000 / CTAS - 2000 * (CTAS - 1) - RING_OFFSET) / (int)kTcBlock;
-    static constexpr int STAGES = FIT < kTcMaxStages ? FIT : kTcMaxStages;
-    static constexpr int SMEM = RING_OFFSET + STAGES * (int)kTcBlock;
+    static constexpr int G = FIT >= 9 ? 3 : 1;  // blocks of a stage
+    static constexpr int STAGES = (FIT < kTcMaxStages ? FIT : kTcMaxStages) / G;
+    static constexpr int SMEM = RING_OFFSET + STAGES * G * (int)kTcBlock;
 };
 
 // One pass over lines: element k of line L sits at
@@ -83,6 +86,7 @@ struct TcPassT {
     R* dst;
     long long inner, lines, ntiles;
     int n, rows, kp, scale, headroom;
+    int prefetch;  // lines in device memory: later tiles may be prefetched
     int jq_in, jq_out;
     JqFixed jin, jout;
 };
@@ -102,6 +106,7 @@ inline TcPassT<R> tc_pass_of(const TcAxis& ax, const PassArgs& a) {
     p.kp = ax.kp;
     p.scale = ax.scale;
     p.headroom = ax.headroom;
+    p.prefetch = !a.host_io;
     p.jq_in = a.jq_in;
     p.jq_out = a.jq_out;
     p.jin = make_jq_fixed(a.jq_in_E, a.jq_in_1mE);
@@ -118,7 +123,7 @@ struct TcShared {
 
 // Ring and barrier positions of a CTA's warps; every lane of a warp holds the
 // same values. The warp that issues the copies keeps its own ring position, the
-// next block of the image, and how many blocks are still to come.
+// next stage of the image, and how many stages are still to come.
 struct TcState {
     int stage = 0;
     unsigned parity = 0;       // consumer: of full; producer: of empty (starts at 1)
@@ -247,21 +252,81 @@ __device__ __forceinline__ T tc_ld(const T* p) {
     else return *p;
 }
 
-// The producer: up to `count` more blocks of an image of tile_chunks blocks.
-template <int STAGES>
+// Eight consecutive values at p, which need not be 16-byte aligned (lines of odd
+// length): aligned 16-byte loads of the values around them, then a shift.
+// Scalar loads, one value of each lane's sectors at a time, missed the small L1
+// beside the tile (n = 255: 350 against 300 us a pass of 255^3). `inside`: the
+// 16 bytes that hold p[7] may reach past p[7].
+template <bool CG>
+__device__ __forceinline__ void tc_load8(const double* p, bool inside, double (&v)[8]) {
+    const bool odd = (reinterpret_cast<uintptr_t>(p) & 8) != 0;
+    if (odd && !inside) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = tc_ld<CG>(p + r);
+        return;
+    }
+    const double2* q = reinterpret_cast<const double2*>(p - (odd ? 1 : 0));
+    double t[10];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        double2 w = make_double2(0.0, 0.0);
+        if (i < 4 || odd) w = tc_ld<CG>(q + i);
+        t[2 * i] = w.x;
+        t[2 * i + 1] = w.y;
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = odd ? t[r + 1] : t[r];
+}
+__device__ __forceinline__ void tc_store8(double* p, const double (&v)[8]) {
+    if ((reinterpret_cast<uintptr_t>(p) & 8) != 0) {
+        p[0] = v[0];
+#pragma unroll
+        for (int r = 1; r < 7; r += 2) *reinterpret_cast<double2*>(p + r) = make_double2(v[r], v[r + 1]);
+        p[7] = v[7];
+    } else {
+#pragma unroll
+        for (int r = 0; r < 8; r += 2) *reinterpret_cast<double2*>(p + r) = make_double2(v[r], v[r + 1]);
+    }
+}
+
+// Asks L2 for the lines of a later tile, 128 bytes a lane (threads `me` of
+// `many`): their loads then wait for L2 and not for memory.
+template <int LT, bool STRIDED, typename R>
+__device__ __forceinline__ void tc_prefetch(const TcPassT<R>& g, long long tile, int me, int many) {
+    constexpr int PER = 128 / (int)sizeof(R);  // values of 128 bytes
+    if (!g.prefetch || tile >= g.ntiles) return;
+    if constexpr (STRIDED) {
+        constexpr int PIECES = LT / PER > 0 ? LT / PER : 1;
+        const long long L = tile * LT + me % PIECES * PER;
+        if (L >= g.lines) return;
+        const long long o = L / g.inner;
+        const R* p = g.src + o * g.n * g.inner + (L - o * g.inner);
+        for (int k = me / PIECES; k < g.n; k += many / PIECES)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p + k * g.inner));
+    } else {
+        const long long first = tile * LT * g.n, last = min((tile + 1) * LT, g.lines) * g.n;
+        for (long long i = first + me * PER; i < last; i += many * PER)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(g.src + i));
+    }
+}
+
+// The producer: up to `count` more stages of an image of `stages` of them (st.left
+// counts stages too).
+template <int STAGES, int G>
 __device__ __forceinline__ bool tc_produce(TcShared& sh, TcState& st, unsigned char* ring, const unsigned char* img,
-                                           int tile_chunks, long long count, long long limit) {
+                                           int stages, long long count, long long limit) {
+    constexpr unsigned BYTES = G * kTcBlock;
     if (count > st.left) count = st.left;
 #pragma unroll 1
     for (long long c = 0; c < count; ++c) {
         if (!tc_wait<true>(&sh.empty[st.stage], st.parity, limit, &sh.abort)) return false;
         if (elect_one()) {
-            mbar_expect_tx(&sh.full[st.stage], kTcBlock);
-            bulk_load(ring + st.stage * kTcBlock, img + (size_t)st.block * kTcBlock, kTcBlock, &sh.full[st.stage]);
+            mbar_expect_tx(&sh.full[st.stage], BYTES);
+            bulk_load(ring + st.stage * BYTES, img + (size_t)st.block * BYTES, BYTES, &sh.full[st.stage]);
         }
         __syncwarp();
         --st.left;
-        if (++st.block == tile_chunks) st.block = 0;
+        if (++st.block == stages) st.block = 0;
         if (++st.stage == STAGES) {
             st.stage = 0;
             st.parity ^= 1u;
@@ -274,12 +339,12 @@ __device__ __forceinline__ bool tc_produce(TcShared& sh, TcState& st, unsigned c
 // sh.done. A block holds one digit place J of D for 32 columns; it meets the
 // places 1 .. S + 1 - J of x (orders J + 1 .. S + 1). One compact loop: unrolled over the
 // places, a narrow tile spent most of the time fetching instructions.
-template <int PARTS, int LT, int STAGES, int S = kTcSlices>
+template <int PARTS, int LT, int STAGES, int G, int S = kTcSlices>
 __device__ __forceinline__ void tc_products(TcShared& sh, TcState& st, unsigned char* digits, unsigned char* ring,
                                             uint32_t tmem, int part0, int part1, int kp, long long limit) {
     using Sh = TcShape<PARTS, LT, S>;
     const uint64_t a0 = tc_desc(smem_u32(ring), 2048, 128), b0 = tc_desc(smem_u32(digits), Sh::LBO, 128);
-    const int blocks = (kp >> 5) * S;
+    const int stages = (kp >> 5) * S / G;
     bool ok = true;
 #pragma unroll 1
     for (int part = part0; ok && part < part1; ++part) {
@@ -288,38 +353,41 @@ __device__ __forceinline__ void tc_products(TcShared& sh, TcState& st, unsigned 
         int j = 0;  // J - 1
         uint32_t later = 0;
 #pragma unroll 1
-        for (int b = 0; b < blocks; ++b) {
+        for (int b = 0; b < stages; ++b) {
             ok = tc_wait(&sh.full[st.stage], st.parity, limit, &sh.abort);
             if (!ok) break;
-            const uint64_t ad = a0 + (uint32_t)(st.stage * (kTcBlock >> 4));
-            const int m = S - j;
-            // N is a multiple of 16 (LT = 8: an even number of places, whose last may
-            // go to an unused order) and at most 256 (LT = 64: 4 places, then the rest)
-            const int w = S * LT > 256 ? min(m, 4) : (LT == 8 ? (m + 1) & ~1 : m);
-            const uint32_t d = d0 + j * LT;
-            const uint32_t idesc = tc_idesc_f16(128, 0) + ((uint32_t)(w * LT) >> 3 << 17);
-            // place 1 reaches every order: its first products overwrite them
-            const uint32_t acc = j == 0 ? later : 1u;
-            if (elect_one()) {
-                tc_mma_f16(d, ad, bd, idesc, acc);
-                if (S * LT > 256 && m > 4)
-                    tc_mma_f16(d + 4 * LT, ad, bd + (4 * LT * 16 >> 4),
-                               tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), acc);
-                tc_mma_f16(d, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4), idesc, 1u);
-                if (S * LT > 256 && m > 4)
-                    tc_mma_f16(d + 4 * LT, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4) + (4 * LT * 16 >> 4),
-                               tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), 1u);
-                tc_commit(&sh.empty[st.stage]);
+            uint64_t ad = a0 + (uint32_t)(st.stage * (G * kTcBlock >> 4));
+#pragma unroll 1
+            for (int q = 0; q < G; ++q, ad += kTcBlock >> 4) {
+                const int m = S - j;
+                // N is a multiple of 16 (LT = 8: an even number of places, whose last may
+                // go to an unused order) and at most 256 (LT = 64: 4 places, then the rest)
+                const int w = S * LT > 256 ? min(m, 4) : (LT == 8 ? (m + 1) & ~1 : m);
+                const uint32_t d = d0 + j * LT;
+                const uint32_t idesc = tc_idesc_f16(128, 0) + ((uint32_t)(w * LT) >> 3 << 17);
+                // place 1 reaches every order: its first products overwrite them
+                const uint32_t acc = j == 0 ? later : 1u;
+                if (elect_one()) {
+                    tc_mma_f16(d, ad, bd, idesc, acc);
+                    if (S * LT > 256 && m > 4)
+                        tc_mma_f16(d + 4 * LT, ad, bd + (4 * LT * 16 >> 4),
+                                   tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), acc);
+                    tc_mma_f16(d, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4), idesc, 1u);
+                    if (S * LT > 256 && m > 4)
+                        tc_mma_f16(d + 4 * LT, ad + (4096 >> 4), bd + (2 * Sh::LBO >> 4) + (4 * LT * 16 >> 4),
+                                   tc_idesc_f16(128, 0) + ((uint32_t)((m - 4) * LT) >> 3 << 17), 1u);
+                    if (q == G - 1) tc_commit(&sh.empty[st.stage]);
+                }
+                __syncwarp();
+                if (++j == S) {
+                    j = 0;
+                    later = 1;
+                    bd += 4 * Sh::LBO >> 4;
+                }
             }
-            __syncwarp();
             if (++st.stage == STAGES) {
                 st.stage = 0;
                 st.parity ^= 1u;
-            }
-            if (++j == S) {
-                j = 0;
-                later = 1;
-                bd += 4 * Sh::LBO >> 4;
             }
         }
     }
@@ -375,17 +443,15 @@ __device__ __forceinline__ bool tc_tile(const TcPass& g, long long tile, unsigne
                 }
             } else {
                 const double* p = g.src + L * n;
-                if ((n & 1) == 0 && 8 * c + 8 <= rows) {
+                if (8 * c + 8 <= rows) {
+                    double v[8];
+                    tc_load8<CG>(p + 8 * c, true, v);
 #pragma unroll
-                    for (int r = 0; r < 8; r += 2) {
-                        const double2 v = tc_ld<CG>(reinterpret_cast<const double2*>(p + 8 * c + r));
-                        x[it][r] = v.x;
-                        x[it][r + 1] = v.y;
-                        if constexpr (PARTS == 2) {
-                            const double2 w = tc_ld<CG>(reinterpret_cast<const double2*>(p + n - 2 - 8 * c - r));
-                            x[it][8 + r] = w.y;
-                            x[it][9 + r] = w.x;
-                        }
+                    for (int r = 0; r < 8; ++r) x[it][r] = v[r];
+                    if constexpr (PARTS == 2) {
+                        tc_load8<CG>(p + n - 8 - 8 * c, c > 0 || L + 1 < g.lines, v);
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) x[it][8 + r] = v[7 - r];
                     }
                 } else {
 #pragma unroll
@@ -446,13 +512,14 @@ __device__ __forceinline__ bool tc_tile(const TcPass& g, long long tile, unsigne
         bool ok = true;
         if (warp == 0) {
             tc_fence_after_sync();
-            tc_products<PARTS, LT, STAGES>(sh, st, smem, ring, tmem, TWO_PHASES ? ph : 0, TWO_PHASES ? ph + 1 : PARTS,
+            tc_products<PARTS, LT, STAGES, Sh::G>(sh, st, smem, ring, tmem, TWO_PHASES ? ph : 0, TWO_PHASES ? ph + 1 : PARTS,
                                            kp, limit);
             ok = tc_wait(&sh.done, st.done_parity, limit, &sh.abort);
         }
+        if (ph == 0 && warp >= 2) tc_prefetch<LT, STRIDED>(g, tile + gridDim.x, tid - 64, NT - 64);
         if (!Sh::OWN_PRODUCER && warp == 1)
-            tc_produce<STAGES>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices,
-                               (TWO_PHASES ? 1 : PARTS) * (kp >> 5) * kTcSlices, limit);
+            tc_produce<STAGES, Sh::G>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices / Sh::G,
+                                      (TWO_PHASES ? 1 : PARTS) * (kp >> 5) * kTcSlices / Sh::G, limit);
         st.done_parity ^= 1u;
         if (!tc_sync_and<NT>(ok && *reinterpret_cast<volatile int*>(&sh.abort) == 0)) return false;
         tc_fence_after_sync();
@@ -557,13 +624,15 @@ __device__ __forceinline__ bool tc_tile(const TcPass& g, long long tile, unsigne
             }
         } else {
             double* p = g.dst + L * n;
-            if ((n & 1) == 0 && 8 * c + 8 <= rows) {
+            if (8 * c + 8 <= rows) {
+                double v[8];
 #pragma unroll
-                for (int r = 0; r < 8; r += 2) {
-                    *reinterpret_cast<double2*>(p + 8 * c + r) = make_double2(x[it][r], x[it][r + 1]);
-                    if constexpr (PARTS == 2)
-                        *reinterpret_cast<double2*>(p + n - 2 - 8 * c - r) =
-                            make_double2(x[it][9 + r], x[it][8 + r]);
+                for (int r = 0; r < 8; ++r) v[r] = x[it][r];
+                tc_store8(p + 8 * c, v);
+                if constexpr (PARTS == 2) {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) v[r] = x[it][15 - r];
+                    tc_store8(p + n - 8 - 8 * c, v);
                 }
             } else {
 #pragma unroll

@@ -33,6 +33,38 @@ __device__ __forceinline__ void tc_put_digits32(unsigned char* chunk, int line, 
     }
 }
 
+// Eight consecutive values at any 4-byte aligned p, as tc_load8.
+__device__ __forceinline__ void tc_load8(const float* p, bool inside, float (&v)[8]) {
+    const unsigned s = (unsigned)(reinterpret_cast<uintptr_t>(p) >> 2) & 3u;
+    if (s != 0 && !inside) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = p[r];
+        return;
+    }
+    const float4* q = reinterpret_cast<const float4*>(p - s);
+    float t[12], h[11];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < 2 || s != 0) w = q[i];
+        t[4 * i] = w.x, t[4 * i + 1] = w.y, t[4 * i + 2] = w.z, t[4 * i + 3] = w.w;
+    }
+#pragma unroll
+    for (int r = 0; r < 11; ++r) h[r] = s & 1u ? t[r + 1] : t[r];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = s & 2u ? h[r + 2] : h[r];
+}
+__device__ __forceinline__ void tc_store8(float* p, const float (&v)[8]) {
+    auto two = [&](int i) { *reinterpret_cast<float2*>(p + i) = make_float2(v[i], v[i + 1]); };
+    auto four = [&](int i) { *reinterpret_cast<float4*>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]); };
+    switch ((unsigned)(reinterpret_cast<uintptr_t>(p) >> 2) & 3u) {
+        case 0: four(0), four(4); break;
+        case 1: p[0] = v[0], two(1), four(3), p[7] = v[7]; break;
+        case 2: two(0), four(2), two(6); break;
+        default: p[0] = v[0], four(1), two(5), p[7] = v[7]; break;
+    }
+}
+
 // One tile of LT lines, by the computing threads: false if a wait ran out.
 template <int PARTS, int LT, bool STRIDED, int STAGES>
 __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long tile, unsigned char* smem,
@@ -52,7 +84,6 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
     float x[UPT][VPU], d[UPT][VPU];  // x0 and its increments so far
     int uline[UPT], uc[UPT];
     const int nch = kp >> 3;
-    const bool vec = !STRIDED && (n & 3) == 0;
 #pragma unroll
     for (int it = 0; it < UPT; ++it) {
         const int u = tid + it * NT;
@@ -70,15 +101,16 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
             const long long o = STRIDED ? L / g.inner : L, i = STRIDED ? L - o * g.inner : 0;
             const float* p = g.src + (STRIDED ? o * n * g.inner + i : L * n);
             const long long stride = STRIDED ? g.inner : 1;
-            if (vec && 8 * c + 8 <= rows) {
+            if (!STRIDED && 8 * c + 8 <= rows) {
+                float v[8];
+                tc_load8(p + 8 * c, true, v);
 #pragma unroll
-                for (int r = 0; r < 8; r += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(p + 8 * c + r);
-                    x[it][r] = v.x, x[it][r + 1] = v.y, x[it][r + 2] = v.z, x[it][r + 3] = v.w;
-                    if constexpr (PARTS == 2) {
-                        const float4 w = *reinterpret_cast<const float4*>(p + n - 4 - 8 * c - r);
-                        x[it][8 + r] = w.w, x[it][9 + r] = w.z, x[it][10 + r] = w.y, x[it][11 + r] = w.x;
-                    }
+                for (int r = 0; r < 8; ++r) x[it][r] = v[r];
+                if constexpr (PARTS == 2) {
+                    // (the 16 bytes around the line's last value may reach two values further)
+                    tc_load8(p + n - 8 - 8 * c, c > 0 || L + 1 < g.lines, v);
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) x[it][8 + r] = v[7 - r];
                 }
             } else {
 #pragma unroll
@@ -133,11 +165,13 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
     bool ok = true;
     if (warp == 0) {
         tc_fence_after_sync();
-        tc_products<PARTS, LT, STAGES, kTcSlices32>(sh, st, smem, ring, tmem, 0, PARTS, kp, limit);
+        tc_products<PARTS, LT, STAGES, Sh::G, kTcSlices32>(sh, st, smem, ring, tmem, 0, PARTS, kp, limit);
         ok = tc_wait(&sh.done, st.done_parity, limit, &sh.abort);
     }
+    if (warp >= 2) tc_prefetch<LT, STRIDED>(g, tile + gridDim.x, tid - 64, NT - 64);
     if (!Sh::OWN_PRODUCER && warp == 1)
-        tc_produce<STAGES>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices32, PARTS * (kp >> 5) * kTcSlices32, limit);
+        tc_produce<STAGES, Sh::G>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices32 / Sh::G,
+                                  PARTS * (kp >> 5) * kTcSlices32 / Sh::G, limit);
     st.done_parity ^= 1u;
     if (!tc_sync_and<NT>(ok && *reinterpret_cast<volatile int*>(&sh.abort) == 0)) return false;
     tc_fence_after_sync();
@@ -207,14 +241,15 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
         const long long o = STRIDED ? L / g.inner : L, i = STRIDED ? L - o * g.inner : 0;
         float* p = g.dst + (STRIDED ? o * n * g.inner + i : L * n);
         const long long stride = STRIDED ? g.inner : 1;
-        if (vec && 8 * c + 8 <= rows) {
+        if (!STRIDED && 8 * c + 8 <= rows) {
+            float v[8];
 #pragma unroll
-            for (int r = 0; r < 8; r += 4) {
-                *reinterpret_cast<float4*>(p + 8 * c + r) =
-                    make_float4(x[it][r], x[it][r + 1], x[it][r + 2], x[it][r + 3]);
-                if constexpr (PARTS == 2)
-                    *reinterpret_cast<float4*>(p + n - 4 - 8 * c - r) =
-                        make_float4(x[it][11 + r], x[it][10 + r], x[it][9 + r], x[it][8 + r]);
+            for (int r = 0; r < 8; ++r) v[r] = x[it][r];
+            tc_store8(p + 8 * c, v);
+            if constexpr (PARTS == 2) {
+#pragma unroll
+                for (int r = 0; r < 8; ++r) v[r] = x[it][15 - r];
+                tc_store8(p + n - 8 - 8 * c, v);
             }
         } else {
 #pragma unroll

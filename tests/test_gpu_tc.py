@@ -155,3 +155,28 @@ def test_wait_runs_out_and_the_plan_stays_usable(n):
         plan.axis_pass(a, 0, 1, 2)
         plan.check()
     assert np.array_equal(a.cpu().numpy(), passes(prob, u0, (1, 2))[0])
+
+
+@pytest.mark.parametrize("n", [(65, 70), (100, 4866), (127, 9730), (129, 66), (255, 2433), (255, 9730), (200, 130)], ids=str)
+def test_fp32_padded_lengths(n):
+    """FP32 zero-padded axes of 65..256 points: tiles of 16, 32 and 64 lines
+    (16, 32, 64 times 152 SMs), odd lines that start at every 4-byte offset, both
+    kinds of axis, with and without the flow. Bar: the rounding of y (6e-8 at
+    |y| <= 1), the increment (3e-8) and the flow's increments (2 x 3e-8)."""
+    m = n[1] // 14 if n[1] > 256 else n[1]
+    rest = (m, n[1] // m) if n[1] > 256 else (m,)
+    for shape, ax in (((n[0],) + rest, 0), (rest + (n[0],), len(rest))):
+        prob = I.Problem(n=shape, alpha=(1.3, 1.7, 1.5)[: len(shape)], eps=0.05, tau=2e-3)
+        u0 = I.random_field(prob, 78, -1.0, 1.0).astype(np.float32)
+        P = O.Scheme.for_problem(I.Problem(n=(n[0],), alpha=(prob.alpha[ax],), eps=0.05, tau=2e-3)).P[0]
+        with S.Plan.for_problem(prob, S.SFAC_FP32) as plan:
+            assert S.sfac_plan_info(plan.handle, ax)[1]          # zero-padded
+            for jq in ((0, 0), (1, 2)):
+                u = torch.tensor(np.ascontiguousarray(u0), device="cuda")
+                plan.axis_pass(u, ax, *jq)
+                plan.check()
+                ref = u0.astype(np.float64)
+                ref = O.nonlinear_flow(ref, 0.5 * prob.tau) if jq[0] else ref
+                ref = O.apply_axis(ref, P, ax + 1)
+                ref = O.nonlinear_flow(ref, prob.tau) if jq[1] else ref
+                assert np.abs(u.double().cpu().numpy() - ref).max() <= 1.8e-7
