@@ -129,6 +129,18 @@ void increment_columns(const AxisHost& T, double tau, std::vector<double>* g, st
     }
 }
 
+std::vector<double> increment_spectra(const AxisHost& T, double tau) {
+    const int n = T.n;
+    std::vector<double> out(4 * (size_t)n);
+    for (int j = 0; j < n; ++j) {
+        out[j] = std::expm1(0.5 * tau * T.lambda[j]);
+        out[n + j] = std::expm1(tau * T.mu[j]);
+    }
+    double s;
+    for (int m = 0; m < 2 * n; ++m) sincospi_frac(m, n, &out[2 * (size_t)n + m], &s);
+    return out;
+}
+
 void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P) {
     const int n = T.n;
     const int L = padded_length(n);

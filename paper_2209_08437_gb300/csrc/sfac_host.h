@@ -34,6 +34,10 @@ int padded_length(int n);
 // values each) of the axis in T.
 void increment_columns(const AxisHost& T, double tau, std::vector<double>* g, std::vector<double>* h);
 
+// The n expm1 values of each spectrum (e^{tau/2 C} - I, then e^{tau S} - I) and
+// cos(pi m / n) for m = 0 .. 2n - 1, from which the columns are summed.
+std::vector<double> increment_spectra(const AxisHost& T, double tau);
+
 // Padded tables of one axis (needs the spectra of compute_axis in T).
 void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P);
 

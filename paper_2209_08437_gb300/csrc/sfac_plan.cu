@@ -372,9 +372,9 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
         delete P;
         return cuda_fail(err, "cudaGetDevice");
     }
-    // FP64 ratio twiddles of each axis's FFT length; first columns of the
-    // exponentials' increments for axes with a tensor-core pass.
-    std::vector<double> rtw[3], gcol[3], hcol[3];
+    // FP64 ratio twiddles of each axis's FFT length; the spectra from which the
+    // operators of axes with a tensor-core pass are built.
+    std::vector<double> rtw[3], spectra[3];
     bool tc[3] = {false, false, false};
     if (params->prec == SFAC_FP64) {
         try {
@@ -397,7 +397,7 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
             // lines of up to 64 points (63^3: 8.9 against 9.4 us).
             tc[l] = params->prec == SFAC_FP64 ? params->n[l] >= sfac::kTcMinN && params->n[l] <= sfac::kTcLongMaxN
                                               : padded[l] && params->n[l] > 64 && params->n[l] <= sfac::kTcMaxN;
-            if (tc[l]) sfac::increment_columns(host[l], params->tau, &gcol[l], &hcol[l]);
+            if (tc[l]) spectra[l] = sfac::increment_spectra(host[l], params->tau);
         }
     } catch (const std::bad_alloc&) {
         delete P;
@@ -406,17 +406,17 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     // One device block: per axis eC[n], eS[n], twist[2n], twid[2n] reals, the
     // FP64 diagnostic tables, and the ratio twiddles.
     const size_t rs = real_size(P);
-    size_t off[3][11], total = 0;
+    size_t off[3][10], total = 0;
     long long max_partials = 1;
     {
         long long inner = 1;
         for (int l = 0; l < params->dim; ++l) {
             const size_t n = padded[l] ? (size_t)pad[l].L : (size_t)params->n[l];
-            const size_t sz[11] = {n * rs, n * rs, padded[l] ? 0 : 2 * n * rs, 2 * n * rs,
+            const size_t sz[10] = {n * rs, n * rs, padded[l] ? 0 : 2 * n * rs, 2 * n * rs,
                                   n * 8,  padded[l] ? 0 : n * 8, padded[l] ? 0 : 2 * n * 8, 2 * n * 8,
                                   rtw[l].size() * sizeof(double),
-                                  gcol[l].size() * sizeof(double), hcol[l].size() * sizeof(double)};
-            for (int q = 0; q < 11; ++q) {
+                                  spectra[l].size() * sizeof(double)};
+            for (int q = 0; q < 10; ++q) {
                 off[l][q] = total;
                 total += align256(sz[q]);
             }
@@ -483,10 +483,7 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
                 std::memcpy(blob.data() + off[l][4 + q], dsrc[q]->data(), dsrc[q]->size() * sizeof(double));
         if (!rtw[l].empty())
             std::memcpy(blob.data() + off[l][8], rtw[l].data(), rtw[l].size() * sizeof(double));
-        if (tc[l]) {
-            std::memcpy(blob.data() + off[l][9], gcol[l].data(), gcol[l].size() * sizeof(double));
-            std::memcpy(blob.data() + off[l][10], hcol[l].data(), hcol[l].size() * sizeof(double));
-        }
+        if (tc[l]) std::memcpy(blob.data() + off[l][9], spectra[l].data(), spectra[l].size() * sizeof(double));
         for (int q = 0; q < 4; ++q) {
             unsigned char* dst = blob.data() + off[l][q];
             const std::vector<double>& v = *src[q];
@@ -511,8 +508,7 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     for (int l = 0; l < params->dim && err == cudaSuccess; ++l)
         if (tc[l])
             err = sfac::tc_build(params->n[l], slices, params->prec == SFAC_FP64 ? sfac::kTcBits : sfac::kTcBits32,
-                                 reinterpret_cast<const double*>(base + off[l][9]),
-                                 reinterpret_cast<const double*>(base + off[l][10]), base + off_img[l],
+                                 reinterpret_cast<const double*>(base + off[l][9]), base + off_img[l],
                                  base + off_scratch, report[l], st_);
     if (err == cudaSuccess) err = cudaStreamSynchronize(st_);
     if (err != cudaSuccess) {

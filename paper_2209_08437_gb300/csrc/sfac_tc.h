@@ -30,17 +30,16 @@ constexpr int kTcMinN = 32, kTcMaxN = 256;
 constexpr int kTcLongMaxN = 1024;
 
 // Device bytes of the digit image of an axis of n points, and of the scratch
-// the builder needs (n x n doubles twice, and a few words).
+// the builder needs.
 size_t tc_image_bytes(int n, int slices);
 size_t tc_scratch_bytes(int n);
 
-// Builds the image from the first columns g, h (device, n doubles each) of
-// e^{tau/2 C} - I and e^{tau S} - I, on stream s. The host words
-// report[0..7] receive, after the stream is synchronised: the scale exponent,
-// then for each of six digit places the largest sum of |digit| over a row's
-// 128 columns, and the largest row sum of |entries| in units of 2^(f - 10).
-cudaError_t tc_build(int n, int slices, int bits, const double* g, const double* h, void* img, void* scratch,
-                     int* report_host, cudaStream_t s);
+// Builds the image from increment_spectra's 4n values (device), on stream s. The
+// host words report[0..7] receive, after the stream is synchronised: the scale
+// exponent, then for each of six digit places the largest sum of |digit| over a
+// row's 128 columns, and the largest row sum of |entries| in units of 2^(f - 10).
+cudaError_t tc_build(int n, int slices, int bits, const double* spectra, void* img, void* scratch, int* report_host,
+                     cudaStream_t s);
 
 // Fills *ax from the builder's report; false where the sums could leave the
 // range in which the products are exact (the axis then keeps its FFT pass).

@@ -19,6 +19,38 @@ int parts_of(int n) { return n <= 128 ? 1 : 2; }
 int rows_of(int n) { return n <= 128 ? n : (n + 1) / 2; }
 int kp_of(int n) { return (rows_of(n) + 31) / 32 * 32; }
 
+// First columns g, h from the expm1 values xc, xs of the spectra and cs[m] =
+// cos(pi m / n):  g_d = (1/n) sum_j xc_j cos(2 pi j d / n),
+// h_d = (1/n) sum_j xs_j cos(pi d (2j - 1) / n). One CTA per d; each thread sums
+// with compensation (Neumaier), the partial sums are added in a fixed order.
+__global__ void __launch_bounds__(128) tc_columns(int n, const double* __restrict__ spectra, double* __restrict__ g,
+                                                  double* __restrict__ h) {
+    const int d = blockIdx.x, skew = blockIdx.y, two_n = 2 * n;
+    const double* x = spectra + skew * n;
+    const double* cs = spectra + two_n;
+    __shared__ double part[2][128];
+    double s = 0.0, c = 0.0;
+    auto add = [&](double v) {
+        const double t = __dadd_rn(s, v);
+        c += fabs(s) >= fabs(v) ? __dadd_rn(__dadd_rn(s, -t), v) : __dadd_rn(__dadd_rn(v, -t), s);
+        s = t;
+    };
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int m = (int)((skew ? (long long)d * (2 * j - 1) + two_n * (long long)n : 2LL * d * j) % two_n);
+        add(__dmul_rn(x[j], cs[m]));
+    }
+    part[0][threadIdx.x] = s;
+    part[1][threadIdx.x] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int t = 1; t < blockDim.x; ++t) {
+            add(part[0][t]);
+            c += part[1][t];
+        }
+        (skew ? h : g)[d] = (s + c) / n;
+    }
+}
+
 // out = X + Y + X Y with X[i][p] = x[|i - p|]; Y = y[|p - j|] (first product) or
 // the stored matrix Ym. All of them are centrosymmetric (M[i][j] =
 // M[n-1-i][n-1-j]): only the first ceil(n/2) rows are formed and stored.
@@ -119,18 +151,21 @@ __global__ void __launch_bounds__(128) tc_digits(int n, int parts, int rows, int
 }  // namespace
 
 size_t tc_image_bytes(int n, int slices) { return (size_t)parts_of(n) * ((rows_of(n) + 127) / 128) * (kp_of(n) / 32) * slices * 8192; }
-size_t tc_scratch_bytes(int n) { return 2 * sizeof(double) * (size_t)((n + 1) / 2) * n + 64; }
+size_t tc_scratch_bytes(int n) { return 2 * sizeof(double) * ((size_t)((n + 1) / 2) * n + n) + 64; }
 
-cudaError_t tc_build(int n, int slices, int bits, const double* g, const double* h, void* img, void* scratch, int* report_host,
+cudaError_t tc_build(int n, int slices, int bits, const double* spectra, void* img, void* scratch, int* report_host,
                      cudaStream_t s) {
     const int parts = parts_of(n), rows = rows_of(n), kp = kp_of(n);
     double* W = static_cast<double*>(scratch);
     double* D = W + (size_t)((n + 1) / 2) * n;
-    unsigned long long* mx = reinterpret_cast<unsigned long long*>(D + (size_t)((n + 1) / 2) * n);
+    double* g = D + (size_t)((n + 1) / 2) * n;
+    double* h = g + n;
+    unsigned long long* mx = reinterpret_cast<unsigned long long*>(h + n);
     int* report = reinterpret_cast<int*>(mx + 1);
     cudaError_t err = cudaMemsetAsync(mx, 0, 64, s);
     if (err != cudaSuccess) return err;
     const dim3 grid((n + 31) / 32, ((n + 1) / 2 + 7) / 8), block(32, 8);
+    tc_columns<<<dim3(n, 2), 128, 0, s>>>(n, spectra, g, h);
     tc_product<<<grid, block, 0, s>>>(n, h, g, nullptr, W);
     tc_product<<<grid, block, 0, s>>>(n, g, nullptr, W, D);
     tc_max<<<std::max(1, std::min(64, n / 4)), 256, 0, s>>>(n, parts, rows, D, mx);
