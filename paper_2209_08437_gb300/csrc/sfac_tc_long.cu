@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
         };
         // the line's largest value
         unsigned m = 0;
-#pragma unroll 2
+#pragma unroll 4
         for (int kc = 0; kc < nkc; ++kc) {
             double v[8];
             load(kc, v);
@@ -255,25 +255,50 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
             r1[q] = sum[0][q] - sum[1][q];
         }
         tc_sync<kNT>();
+        // four values and their mirror images at a time, so that their loads overlap
+        constexpr int B = 4;
 #pragma unroll 1
-        for (int u = tid; u < 128 * kLT; u += kNT) {
-            const int rr = STRIDED ? u / kLT : u % 128, l = STRIDED ? u % kLT : u / 128;
-            const int k = (int)rank * 128 + rr;
-            const long long b = sbase[l];
-            if (k >= rows || b < 0) continue;
-            const int Eb = (int)(smax[l] >> 20);
-            const int E = max(Eb, Emin) + ps.headroom;
-            const long long at[2] = {b + k * inner, b + (n - 1 - k) * inner};
-            double v[2] = {ps.src[at[0]], ps.src[at[1]]};
+        for (int u0 = tid; u0 < 128 * kLT; u0 += B * kNT) {
+            double v[2 * B];
+            auto where = [&](int i, int* rr, int* l) {
+                const int u = u0 + i * kNT;
+                *rr = STRIDED ? u / kLT : u % 128;
+                *l = STRIDED ? u % kLT : u / 128;
+                return (int)rank * 128 + *rr < rows ? sbase[*l] : -1;
+            };
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const long long d = *reinterpret_cast<const long long*>(smem + kRing + (h * 128 + rr) * kPitch + l * 8);
-                v[h] = tc_to_double(tc_fixed(v[h], E) + tc_align(d, ps.scale), E);
-                if (Eb == 2047) v[h] = __longlong_as_double(0x7ff8000000000000LL);
+            for (int i = 0; i < B; ++i) {
+                int rr, l;
+                const long long b = where(i, &rr, &l);
+                const int k = (int)rank * 128 + rr;
+                v[i] = b < 0 ? 0.0 : ps.src[b + k * inner];
+                v[B + i] = b < 0 ? 0.0 : ps.src[b + (n - 1 - k) * inner];
+            }
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                int rr, l;
+                where(i, &rr, &l);
+                const int Eb = (int)(smax[l] >> 20);
+                const int E = max(Eb, Emin) + ps.headroom;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    double& w = v[h * B + i];
+                    const long long d =
+                        *reinterpret_cast<const long long*>(smem + kRing + (h * 128 + rr) * kPitch + l * 8);
+                    w = tc_to_double(tc_fixed(w, E) + tc_align(d, ps.scale), E);
+                    if (Eb == 2047) w = __longlong_as_double(0x7ff8000000000000LL);
+                }
             }
             if (ps.jq_out) jq_flow_fixed_all(v, ps.jout);
-            ps.dst[at[0]] = v[0];
-            ps.dst[at[1]] = v[1];
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                int rr, l;
+                const long long b = where(i, &rr, &l);
+                const int k = (int)rank * 128 + rr;
+                if (b < 0) continue;
+                ps.dst[b + k * inner] = v[i];
+                ps.dst[b + (n - 1 - k) * inner] = v[B + i];
+            }
         }
     }
     __syncthreads();
