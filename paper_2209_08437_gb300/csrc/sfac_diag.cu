@@ -137,6 +137,96 @@ diag_reduce_kernel(const double3* __restrict__ partial, long long n, double* __r
     }
 }
 
+// Small grids. The FFT passes above are latency bound there (2D 127^2: about 35 us
+// an axis for 64 line pairs, four launches, whatever the arithmetic): n^2 / 2
+// multiply-adds a line, spread over a CTA, take less up to a few hundred points.
+// Side by side on one GB300: a 127^2 FP64 step with diagnostics 101 -> 57 us. The
+// FP64 pipes do 304 multiply-adds a clock, so kDiagDirectMost of them take 42 us,
+// where the FFT passes are no slower.
+template <typename Rin>
+__global__ void __launch_bounds__(DIAG_THREADS) diag_direct_kernel(const DiagDirect g) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[3][DIAG_THREADS];
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    long long line = blockIdx.x;
+    int ax = 0;
+    while (line >= g.lines[ax]) line -= g.lines[ax++];
+    const int n = g.n[ax];
+    const long long inner = g.inner[ax], o = line / inner;
+    const Rin* p = static_cast<const Rin*>(g.u) + o * n * inner + (line - o * inner);
+    double* x = reinterpret_cast<double*>(smem_raw);
+    double* b = x + n;
+    double dot = 0.0, pot = 0.0, mx = 0.0;
+    const double b0 = g.b[ax][0];
+    for (int i = tid; i < n; i += DIAG_THREADS) {
+        const double v = (double)p[i * inner];
+        x[i] = v;
+        b[i] = g.b[ax][i];
+        dot += b0 * v * v;
+        if (ax == 0) {
+            const double w = v * v - 1.0;
+            pot += w * w;
+            mx = fmax(mx, fabs(v));
+        }
+    }
+    __syncthreads();
+    // offsets d and n - d together have n terms; two threads take half each
+    for (int d1 = 1 + (tid >> 1); 2 * d1 <= n; d1 += DIAG_THREADS / 2) {
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const int d = h ? n - d1 : d1;
+            if (h && d == d1) break;
+            const int len = n - d, mid = len / 2;
+            const int i1 = (tid & 1) ? len : mid;
+            double s[4] = {0, 0, 0, 0};
+            int i = (tid & 1) ? mid : 0;
+            for (; i + 4 <= i1; i += 4)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s[q] = fma(x[i + q], x[i + q + d], s[q]);
+            for (; i < i1; ++i) s[0] = fma(x[i], x[i + d], s[0]);
+            dot = fma(2.0 * b[d], (s[0] + s[1]) + (s[2] + s[3]), dot);
+        }
+    }
+    auto reduce = [&]() {
+        red[0][tid] = dot;
+        red[1][tid] = pot;
+        red[2][tid] = mx;
+        __syncthreads();
+        for (int w = DIAG_THREADS / 2; w > 0; w >>= 1) {
+            if (tid < w) {
+                red[0][tid] += red[0][tid + w];
+                red[1][tid] += red[1][tid + w];
+                red[2][tid] = fmax(red[2][tid], red[2][tid + w]);
+            }
+            __syncthreads();
+        }
+    };
+    reduce();
+    if (tid == 0) {
+        g.partial[blockIdx.x] = make_double3(red[0][0], red[1][0], red[2][0]);
+        __threadfence();
+        last = atomicAdd(g.counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    dot = pot = mx = 0.0;
+    for (unsigned i = tid; i < gridDim.x; i += DIAG_THREADS) {
+        const volatile double* v = reinterpret_cast<const volatile double*>(g.partial + i);
+        dot += v[0];
+        pot += v[1];
+        mx = fmax(mx, v[2]);
+    }
+    reduce();
+    if (tid == 0) {
+        g.out[0] = red[0][0];
+        g.out[1] = red[1][0];
+        g.out[2] = red[2][0];
+        *g.counter = 0;
+    }
+}
+
 template <typename Rin, int N, bool STRIDED, bool PADDED>
 cudaError_t launch_diag_cfg(const PassArgs& a, const double* mA, const double* mB, int first_axis,
                             double3* partial, long long* nblocks, cudaStream_t s) {
@@ -185,6 +275,19 @@ cudaError_t launch_diag_any(int N, const PassArgs& a, const double* mA, const do
 }
 
 }  // namespace
+
+cudaError_t launch_diag_direct(bool f64_field, const DiagDirect& d, cudaStream_t s) {
+    long long blocks = 0;
+    int nmax = 0;
+    for (int ax = 0; ax < d.dim; ++ax) {
+        blocks += d.lines[ax];
+        nmax = d.n[ax] > nmax ? d.n[ax] : nmax;
+    }
+    const size_t smem = 2 * sizeof(double) * (size_t)nmax;  // n <= 2048: 32 KB
+    if (f64_field) diag_direct_kernel<double><<<(unsigned)blocks, DIAG_THREADS, smem, s>>>(d);
+    else diag_direct_kernel<float><<<(unsigned)blocks, DIAG_THREADS, smem, s>>>(d);
+    return cudaGetLastError();
+}
 
 long long diag_partials_needed(long long clines, int N) {
     const int E = N < DIAG_E ? N : DIAG_E;

@@ -21,4 +21,21 @@ long long diag_partials_needed(long long clines, int N);
 cudaError_t launch_diag_axis(bool f64_field, bool padded, int N, const PassArgs& a, const double* mA,
                              const double* mB, int first_axis, double3* partial, double* out, cudaStream_t s);
 
+// Small grids: every line of every axis by one CTA of one launch, x . B x as the
+// Toeplitz sum b_0 sum x_i^2 + 2 sum_d b_d sum_i x_i x_{i+d}, and the final sum by
+// the CTA that finishes last (fixed order).
+struct DiagDirect {
+    const void* u;
+    int dim;
+    int n[3];
+    long long inner[3], lines[3];
+    const double* b[3];     // first column of B_axis
+    double3* partial;       // one entry per line of all axes
+    unsigned int* counter;  // 0 before and after
+    double* out;            // out[0..2] as launch_diag_axis
+};
+// Most multiply-adds (sum over lines of n^2 / 2) of a grid that takes this route.
+constexpr double kDiagDirectMost = 2.4e7;
+cudaError_t launch_diag_direct(bool f64_field, const DiagDirect& d, cudaStream_t s);
+
 }  // namespace sfac

@@ -107,10 +107,13 @@ struct sfac_plan {
         const double* dB;
         const void* dtwist;
         const void* dtwid;
+        const double* dcol;  // first column of B_axis
         sfac::TcAxis tc;  // FP64 lines with a tensor-core pass (tc.img != NULL)
     } ax[3] = {};
     double3* diag_partial = nullptr;
     double* diag_out = nullptr;
+    unsigned int* diag_counter = nullptr;
+    bool diag_direct = false;  // small grid: sfac_diagnostics in one launch
     unsigned int* status = nullptr;       // SFAC_PASS_TIMEOUT bits set by the passes (device)
     unsigned int* bar = nullptr;          // grid barrier of the whole-call launch (device, 2 words)
     unsigned int* status_host = nullptr;  // pinned host copy of it
@@ -406,26 +409,33 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     // One device block: per axis eC[n], eS[n], twist[2n], twid[2n] reals, the
     // FP64 diagnostic tables, and the ratio twiddles.
     const size_t rs = real_size(P);
-    size_t off[3][10], total = 0;
-    long long max_partials = 1;
+    size_t off[3][11], total = 0;
+    long long max_partials = 1, direct_lines = 0;
+    double direct_work = 0.0;
+    int direct_n = 0;
     {
         long long inner = 1;
         for (int l = 0; l < params->dim; ++l) {
             const size_t n = padded[l] ? (size_t)pad[l].L : (size_t)params->n[l];
-            const size_t sz[10] = {n * rs, n * rs, padded[l] ? 0 : 2 * n * rs, 2 * n * rs,
+            const size_t sz[11] = {n * rs, n * rs, padded[l] ? 0 : 2 * n * rs, 2 * n * rs,
                                   n * 8,  padded[l] ? 0 : n * 8, padded[l] ? 0 : 2 * n * 8, 2 * n * 8,
                                   rtw[l].size() * sizeof(double),
-                                  spectra[l].size() * sizeof(double)};
-            for (int q = 0; q < 10; ++q) {
+                                  spectra[l].size() * sizeof(double), (size_t)params->n[l] * sizeof(double)};
+            for (int q = 0; q < 11; ++q) {
                 off[l][q] = total;
                 total += align256(sz[q]);
             }
             const long long outer = P->npts / ((long long)params->n[l] * inner);
             const long long clines = l == 0 ? (outer + 1) / 2 : outer * ((inner + 1) / 2);
             max_partials = std::max(max_partials, sfac::diag_partials_needed(clines, (int)n));
+            direct_lines += outer * inner;
+            direct_work += 0.5 * (double)(outer * inner) * params->n[l] * params->n[l];
+            direct_n = std::max(direct_n, params->n[l]);
             inner *= params->n[l];
         }
     }
+    P->diag_direct = direct_work <= sfac::kDiagDirectMost && direct_n <= 2048;
+    if (P->diag_direct) max_partials = std::max(max_partials, direct_lines);
     const size_t off_partial = total;
     total += align256(sizeof(double3) * (size_t)max_partials);
     const size_t off_out = total;
@@ -484,6 +494,7 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
         if (!rtw[l].empty())
             std::memcpy(blob.data() + off[l][8], rtw[l].data(), rtw[l].size() * sizeof(double));
         if (tc[l]) std::memcpy(blob.data() + off[l][9], spectra[l].data(), spectra[l].size() * sizeof(double));
+        std::memcpy(blob.data() + off[l][10], host[l].bcol.data(), host[l].bcol.size() * sizeof(double));
         for (int q = 0; q < 4; ++q) {
             unsigned char* dst = blob.data() + off[l][q];
             const std::vector<double>& v = *src[q];
@@ -530,9 +541,11 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
         P->ax[l].dB = padded[l] ? nullptr : reinterpret_cast<const double*>(base + off[l][5]);
         P->ax[l].dtwist = padded[l] ? nullptr : base + off[l][6];
         P->ax[l].dtwid = base + off[l][7];
+        P->ax[l].dcol = reinterpret_cast<const double*>(base + off[l][10]);
     }
     P->diag_partial = reinterpret_cast<double3*>(base + off_partial);
     P->diag_out = reinterpret_cast<double*>(base + off_out);
+    P->diag_counter = reinterpret_cast<unsigned int*>(base + off_out + 3 * sizeof(double));
     P->status = reinterpret_cast<unsigned int*>(base + off_status);
     P->bar = reinterpret_cast<unsigned int*>(base + off_bar);
     err = cudaMallocHost(reinterpret_cast<void**>(&P->status_host), sizeof(unsigned int));
@@ -683,12 +696,34 @@ sfac_status sfac_diagnostics(sfac_plan* plan, const void* u_dev, double* out, vo
     DeviceGuard g(plan->device);
     if (!g.ok) return fail(SFAC_ECUDA, "cannot select the plan's device");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t err = cudaMemsetAsync(plan->diag_out, 0, 3 * sizeof(double), st);
-    if (err != cudaSuccess) return cuda_fail(err, "diagnostics reset");
+    cudaError_t err = cudaSuccess;
+    if (plan->diag_direct) {
+        sfac::DiagDirect d{};
+        d.u = u_dev;
+        d.dim = plan->p.dim;
+        long long in = 1;
+        for (int ax = 0; ax < d.dim; ++ax) {
+            d.n[ax] = plan->p.n[ax];
+            d.inner[ax] = in;
+            d.lines[ax] = plan->npts / d.n[ax];
+            d.b[ax] = plan->ax[ax].dcol;
+            in *= d.n[ax];
+        }
+        d.partial = plan->diag_partial;
+        d.counter = plan->diag_counter;
+        d.out = plan->diag_out;
+        err = sfac::launch_diag_direct(plan->p.prec == SFAC_FP64, d, st);
+        if (err != cudaSuccess) return cuda_fail(err, "diagnostics launch");
+    } else {
+        err = cudaMemsetAsync(plan->diag_out, 0, 3 * sizeof(double), st);
+        if (err != cudaSuccess) return cuda_fail(err, "diagnostics reset");
+    }
     long long inner = 1;
     double hprod = 1.0;
     for (int ax = 0; ax < plan->p.dim; ++ax) {
         const int n = plan->p.n[ax];
+        hprod *= (plan->p.b - plan->p.a) / (double)(n + 1);
+        if (plan->diag_direct) continue;
         sfac::PassArgs a;
         a.u = const_cast<void*>(u_dev);
         a.inner = inner;
@@ -705,7 +740,6 @@ sfac_status sfac_diagnostics(sfac_plan* plan, const void* u_dev, double* out, vo
                                      plan->diag_out, st);
         if (err != cudaSuccess) return cuda_fail(err, "diagnostics launch");
         inner *= n;
-        hprod *= (plan->p.b - plan->p.a) / (double)(n + 1);
     }
     double host[3];
     err = cudaMemcpyAsync(host, plan->diag_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, st);
