@@ -121,7 +121,9 @@ axis_pass_staged_kernel(const __grid_constant__ CUtensorMap tmap, const PassArgs
         fence_mbar_init();
     }
     PassArgs a = a0;
+    pass_next_may_start();
     SmemTables<float, N, E, false>::load(a, tabs);  // ends with __syncthreads
+    pass_wait_for_previous();
 
     const long long first = blockIdx.x, step = gridDim.x;
     const long long mine = first < ntiles ? (ntiles - 1 - first) / step + 1 : 0;
@@ -249,8 +251,7 @@ cudaError_t launch_staged(const PassArgs& a, cudaStream_t s) {
     const long long ntiles = a.outer * tiles_per_outer;
     if (ntiles <= 0) return cudaSuccess;
     const long long grid = ntiles < resident ? ntiles : resident;
-    kern<<<(unsigned)grid, Sh::WPB * 32, Sh::SMEM, s>>>(map, a, tiles_per_outer, ntiles);
-    return cudaGetLastError();
+    return launch_overlapped(kern, (unsigned)grid, Sh::WPB * 32, Sh::SMEM, s, map, a, tiles_per_outer, ntiles);
 }
 
 // SMs of the current device (cached per device).

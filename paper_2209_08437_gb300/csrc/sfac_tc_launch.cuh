@@ -31,7 +31,7 @@ tc_pass_kernel(const TcArgs<R> g) {
     __shared__ TcShared sh;
     __shared__ unsigned smax[LT];
     unsigned char* ring = smem + Sh::RING_OFFSET;
-    tc_next_may_start();
+    pass_next_may_start();
     const uint32_t tmem = tc_setup<Sh::COLS, Sh::STAGES>(sh);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     TcState st;
@@ -44,7 +44,7 @@ tc_pass_kernel(const TcArgs<R> g) {
                                       g.wait_cycles);
     }
     if (warp < NT / 32) {
-        tc_wait_for_previous();
+        pass_wait_for_previous();
         // the test hook: a barrier that nothing completes
         if (g.hold && warp == 0) tc_wait(&sh.never, 0, g.wait_cycles, &sh.abort);
         bool alive = true;
@@ -87,15 +87,7 @@ cudaError_t launch_tc(const TcAxis& ax, const PassArgs& a, long long lines, cuda
     g.hold = a.hold;
     if (g.pass.ntiles <= 0) return cudaSuccess;
     const long long grid = g.pass.ntiles < resident ? g.pass.ntiles : resident;
-    cudaLaunchAttribute attr[1] = {tc_overlap_attribute()};
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(Sh::TOTAL);
-    cfg.dynamicSmemBytes = Sh::SMEM;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, g);
+    return launch_overlapped(kern, (unsigned)grid, Sh::TOTAL, Sh::SMEM, s, g);
 }
 
 template <typename R, int PARTS, int LT>

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
     const TcPass& ps = g.pass;
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    tc_next_may_start();
+    pass_next_may_start();
     unsigned rank;
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     const long long tile = blockIdx.x / ((ps.rows + 127) / 128);
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
     const int Emin = max(1, 64 - ps.scale);
     long long sum[2][16];  // row (warp & 3) * 32 + lane, lines (warp >> 2) * 16 ..
     if (warp < kNT / 32) {
-        tc_wait_for_previous();
+        pass_wait_for_previous();
         const long long base = sbase[line];
         const double* p = ps.src + (base < 0 ? 0 : base);
         auto load = [&](int kc, double (&v)[8]) {
@@ -323,8 +323,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
 // CTA of the cluster and the closing update would each apply it again (2D
 // 1024^2: 96 us a pass, against 62 us without the flow).
 __global__ void __launch_bounds__(256) tc_flow_kernel(const double* src, double* dst, long long npts, JqFixed q) {
-    tc_next_may_start();
-    tc_wait_for_previous();
+    pass_next_may_start();
+    pass_wait_for_previous();
     constexpr int V = 4;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < npts; i += V * stride) {
@@ -356,14 +356,8 @@ cudaError_t launch_long(const TcAxis& ax, const PassArgs& a, cudaStream_t s) {
     if (g.pass.ntiles > 0x7fffffffLL / cluster) return cudaErrorInvalidValue;
     if (a.jq_in) {
         const long long npts = g.pass.lines * ax.n, want = (npts + 1023) / 1024, most = 16LL * current_device_sms();
-        cudaLaunchAttribute overlap[1] = {tc_overlap_attribute()};
-        cudaLaunchConfig_t flow = {};
-        flow.gridDim = dim3((unsigned)(want < most || most <= 0 ? want : most));
-        flow.blockDim = dim3(256);
-        flow.stream = s;
-        flow.attrs = overlap;
-        flow.numAttrs = 1;
-        err = cudaLaunchKernelEx(&flow, tc_flow_kernel, g.pass.src, g.pass.dst, npts, g.pass.jin);
+        err = launch_overlapped(tc_flow_kernel, (unsigned)(want < most || most <= 0 ? want : most), 256, 0, s,
+                                g.pass.src, g.pass.dst, npts, g.pass.jin);
         if (err != cudaSuccess) return err;
         g.pass.src = g.pass.dst;
     }
@@ -375,7 +369,7 @@ cudaError_t launch_long(const TcAxis& ax, const PassArgs& a, cudaStream_t s) {
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim = {(unsigned)cluster, 1, 1};
-    attr[1] = tc_overlap_attribute();
+    attr[1] = pass_overlap_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, tc_long_kernel<STRIDED>, g);

@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kNT + 32, 1) tc_steps_kernel(const TcStepsArgs
     __shared__ unsigned smax[kLT];
     __shared__ long long base[kLT];
     __shared__ TcPass pass;
-    if (g.single) tc_next_may_start();
+    if (g.single) pass_next_may_start();
     const uint32_t tmem = tc_setup<Shape2::COLS, kStages>(sh);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     TcState st;
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kNT + 32, 1) tc_steps_kernel(const TcStepsArgs
                 }
             }
     } else {
-        if (g.single) tc_wait_for_previous();
+        if (g.single) pass_wait_for_previous();
         if (g.single && g.hold && warp == 0) tc_wait(&sh.never, 0, g.wait_cycles, &sh.abort);  // the test hook
         unsigned target = 0;
         for (long long s = 0; alive && s < g.nsteps; ++s) {
@@ -321,7 +321,7 @@ cudaError_t launch_small(TcStepsArgs& g, const TcAxis* ax, const PassArgs* pa, b
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
     } else {
-        attr[0] = tc_overlap_attribute();
+        attr[0] = pass_overlap_attribute();
     }
     cfg.attrs = attr;
     cfg.numAttrs = 1;

@@ -650,20 +650,6 @@ __device__ __forceinline__ bool tc_tile(const TcPass& g, long long tile, unsigne
     return true;
 }
 
-// Passes of one call follow each other on a stream: the next launch may start
-// while this one runs (programmatic dependent launch) and then waits, before it
-// touches the field, until this one is complete and its stores are visible. Its
-// set-up and the first copies of the operator, which no launch writes, overlap
-// this one's tail.
-__device__ __forceinline__ void tc_next_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void tc_wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-inline cudaLaunchAttribute tc_overlap_attribute() {
-    cudaLaunchAttribute a{};
-    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a.val.programmaticStreamSerializationAllowed = 1;
-    return a;
-}
-
 // Sets up a CTA: tensor memory (warp 0), barriers. All threads of the CTA.
 template <int COLS, int STAGES>
 __device__ __forceinline__ uint32_t tc_setup(TcShared& sh) {
