@@ -25,7 +25,7 @@ struct TcAxis {
 constexpr int kTcSlices = 6, kTcBits = 9;
 constexpr int kTcSlices32 = 3, kTcBits32 = 10;
 // Lengths with a tensor-core pass.
-constexpr int kTcMinN = 32, kTcMaxN = 256;
+constexpr int kTcMinN = 17, kTcMaxN = 256;
 // FP64 lines above kTcMaxN take clusters of CTAs (sfac_tc_long.cu).
 constexpr int kTcLongMaxN = 1024;
 

@@ -8,9 +8,10 @@ template <int PARTS>
 cudaError_t launch_tc_parts32(const TcAxis& ax, const PassArgs& a, cudaStream_t s) {
     const long long lines = a.outer * a.inner;
     const int sms = current_device_sms();
-    if (lines >= 64LL * sms) return launch_tc_axis<float, PARTS, 64>(ax, a, lines, s);
-    if (lines >= 32LL * sms) return launch_tc_axis<float, PARTS, 32>(ax, a, lines, s);
-    return launch_tc_axis<float, PARTS, 16>(ax, a, lines, s);
+    // the narrowest tile with which every SM gets one at most
+    if (lines <= 16LL * sms) return launch_tc_axis<float, PARTS, 16>(ax, a, lines, s);
+    if (lines <= 32LL * sms) return launch_tc_axis<float, PARTS, 32>(ax, a, lines, s);
+    return launch_tc_axis<float, PARTS, 64>(ax, a, lines, s);
 }
 
 }  // namespace

@@ -1,4 +1,4 @@
-"""FP64 passes of 32..1024 points on the tensor cores (csrc/sfac_tc_*.cu):
+"""FP64 passes of 17..1024 points on the tensor cores (csrc/sfac_tc_*.cu):
 the edges of their tiles (lengths around the folding limit 128, the K step 32,
 the cluster limits 256, 512 and 768, odd lengths, line counts around the tile
 widths 8..64), the scaling of each line, non-finite values, and the bounded
@@ -30,7 +30,7 @@ def passes(prob, u0, jq=(0, 0)):
     return out
 
 
-@pytest.mark.parametrize("n", [(32, 33), (63, 64), (65, 96), (127, 128), (129, 130), (255, 256), (7, 256), (256, 9),
+@pytest.mark.parametrize("n", [(17, 31), (32, 33), (63, 64), (65, 96), (127, 128), (129, 130), (255, 256), (7, 256), (256, 9),
                                (160, 200), (32, 8, 33), (129, 3, 5)], ids=str)
 def test_lengths_around_the_tile_edges(n):
     prob = I.Problem(n=n, alpha=(1.2, 1.8, 1.5)[: len(n)], eps=0.08, tau=0.01)
@@ -43,9 +43,9 @@ def test_lengths_around_the_tile_edges(n):
 
 @pytest.mark.parametrize("n", [(64, 13, 187), (48, 5, 973), (256, 3, 811), (33, 23, 423), (130, 10, 973)], ids=str)
 def test_tile_widths(n):
-    """Line counts just below and above 16, 32 and 64 times the device's 152
-    SMs, where the tile widens to 16, 32 and 64 lines, with a partly filled last
-    tile; the contiguous axis and the last one."""
+    """Line counts around 16, 32 and 64 times the device's 152 SMs: tiles of 16
+    lines (2431), 32 (2433) and 64 (4865; 9729 and 9730: a second round), with a
+    partly filled last tile; the contiguous axis and the last one."""
     for m, ax in ((n, 0), ((n[1], n[2], n[0]), 2)):
         prob = I.Problem(n=m, alpha=(1.3, 1.7, 1.5), eps=0.08, tau=0.01)
         u0 = I.random_field(prob, 72, -1.0, 1.0)
@@ -159,8 +159,7 @@ def test_wait_runs_out_and_the_plan_stays_usable(n):
 
 @pytest.mark.parametrize("n", [(65, 70), (100, 4866), (127, 9730), (129, 66), (255, 2433), (255, 9730), (200, 130)], ids=str)
 def test_fp32_padded_lengths(n):
-    """FP32 zero-padded axes of 65..256 points: tiles of 16, 32 and 64 lines
-    (16, 32, 64 times 152 SMs), odd lines that start at every 4-byte offset, both
+    """FP32 zero-padded axes of 65..256 points: tiles of 16, 32 and 64 lines, odd lines that start at every 4-byte offset, both
     kinds of axis, with and without the flow. Bar: the rounding of y (6e-8 at
     |y| <= 1), the increment (3e-8) and the flow's increments (2 x 3e-8)."""
     m = n[1] // 14 if n[1] > 256 else n[1]
