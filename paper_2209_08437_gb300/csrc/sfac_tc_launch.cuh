@@ -47,14 +47,15 @@ tc_pass_kernel(const TcArgs<R> g) {
         pass_wait_for_previous();
         // the test hook: a barrier that nothing completes
         if (g.hold && warp == 0) tc_wait(&sh.never, 0, g.wait_cycles, &sh.abort);
-        bool alive = true;
-        for (long long tile = blockIdx.x; alive && tile < g.pass.ntiles; tile += gridDim.x)
-            if constexpr (sizeof(R) == 8)
-                alive = tc_tile<PARTS, LT, STRIDED, false, Sh::STAGES>(g.pass, tile, smem, ring, smax, sh, st, tmem,
-                                                                       g.img, threadIdx.x, g.wait_cycles);
-            else
+        if constexpr (sizeof(R) == 8) {
+            tc_tiles<PARTS, LT, STRIDED, Sh::STAGES>(g.pass, smem, ring, smax, sh, st, tmem, g.img, threadIdx.x,
+                                                     g.wait_cycles);
+        } else {
+            bool alive = true;
+            for (long long tile = blockIdx.x; alive && tile < g.pass.ntiles; tile += gridDim.x)
                 alive = tc_tile_f32<PARTS, LT, STRIDED, Sh::STAGES>(g.pass, tile, smem, ring, smax, sh, st, tmem,
                                                                     g.img, threadIdx.x, g.wait_cycles);
+        }
     }
     __syncthreads();
     if (sh.abort) {

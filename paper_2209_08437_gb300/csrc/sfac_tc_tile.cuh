@@ -232,6 +232,11 @@ __device__ __forceinline__ void tc_put_digits(unsigned char* chunk, int line, co
 // A sum in units of 2^(E - 1082 + f) in units of 2^(E - 1082), rounded.
 __device__ __forceinline__ long long tc_align(long long v, int f) {
     if (f >= 0) return v << f;
+    if (f > -32) {  // a funnel shift; f is the same for the whole launch
+        const unsigned long long t = (unsigned long long)(v + (1LL << (-f - 1)));
+        return (long long)(((unsigned long long)(unsigned)((int)(t >> 32) >> -f) << 32) |
+                           __funnelshift_r((unsigned)t, (unsigned)(t >> 32), (unsigned)-f));
+    }
     const int right = min(-f, 62);
     return (v + (1LL << (right - 1))) >> right;
 }
@@ -246,46 +251,60 @@ __device__ __forceinline__ long long tc_combine(const float (&a)[kTcOrders]) {
     return (hi << 24) + lo;
 }
 
-template <bool CG, typename T>
-__device__ __forceinline__ T tc_ld(const T* p) {
-    if constexpr (CG) return __ldcg(p);
-    else return *p;
+// 32 aligned bytes, one sector of L2, a lane.
+__device__ __forceinline__ void ld_sector(const double* p, double (&v)[4]) {
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void st_sector(double* p, double a, double b, double c, double d) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
 }
 
-// Eight consecutive values at p, which need not be 16-byte aligned (lines of odd
-// length): aligned 16-byte loads of the values around them, then a shift.
-// Scalar loads, one value of each lane's sectors at a time, missed the small L1
-// beside the tile (n = 255: 350 against 300 us a pass of 255^3). `inside`: the
-// 16 bytes that hold p[7] may reach past p[7].
-template <bool CG>
+// Eight consecutive values at any 8-byte aligned p: the aligned sectors around
+// them, then a shift. Narrower loads, each lane in sectors of its own, come back to a
+// sector that has left the small L1 beside the tile (16-byte loads: a contiguous
+// pass of 256^3 took 227 us, a strided one 208). `inside`: the sector that holds
+// p[7] may reach past it.
 __device__ __forceinline__ void tc_load8(const double* p, bool inside, double (&v)[8]) {
-    const bool odd = (reinterpret_cast<uintptr_t>(p) & 8) != 0;
-    if (odd && !inside) {
+    const unsigned s = (unsigned)(reinterpret_cast<uintptr_t>(p) >> 3) & 3u;
+    if (s == 0) {
+        double t[4];
+        ld_sector(p, t);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) v[r] = tc_ld<CG>(p + r);
+        for (int r = 0; r < 4; ++r) v[r] = t[r];
+        ld_sector(p + 4, t);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[4 + r] = t[r];
         return;
     }
-    const double2* q = reinterpret_cast<const double2*>(p - (odd ? 1 : 0));
-    double t[10];
+    if (!inside) {
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        double2 w = make_double2(0.0, 0.0);
-        if (i < 4 || odd) w = tc_ld<CG>(q + i);
-        t[2 * i] = w.x;
-        t[2 * i + 1] = w.y;
+        for (int r = 0; r < 8; ++r) v[r] = p[r];
+        return;
+    }
+    double t[12], h[11];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double w[4];
+        ld_sector(p - s + 4 * i, w);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) t[4 * i + r] = w[r];
     }
 #pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = odd ? t[r + 1] : t[r];
+    for (int r = 0; r < 11; ++r) h[r] = s & 1u ? t[r + 1] : t[r];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = s & 2u ? h[r + 2] : h[r];
 }
 __device__ __forceinline__ void tc_store8(double* p, const double (&v)[8]) {
-    if ((reinterpret_cast<uintptr_t>(p) & 8) != 0) {
-        p[0] = v[0];
-#pragma unroll
-        for (int r = 1; r < 7; r += 2) *reinterpret_cast<double2*>(p + r) = make_double2(v[r], v[r + 1]);
-        p[7] = v[7];
-    } else {
-#pragma unroll
-        for (int r = 0; r < 8; r += 2) *reinterpret_cast<double2*>(p + r) = make_double2(v[r], v[r + 1]);
+    auto two = [&](int i) { *reinterpret_cast<double2*>(p + i) = make_double2(v[i], v[i + 1]); };
+    auto four = [&](int i) { st_sector(p + i, v[i], v[i + 1], v[i + 2], v[i + 3]); };
+    switch ((unsigned)(reinterpret_cast<uintptr_t>(p) >> 3) & 3u) {
+        case 0: four(0), four(4); break;
+        case 1: p[0] = v[0], two(1), four(3), p[7] = v[7]; break;
+        case 2: two(0), four(2), two(6); break;
+        default: p[0] = v[0], four(1), two(5), p[7] = v[7]; break;
     }
 }
 
@@ -395,258 +414,254 @@ __device__ __forceinline__ void tc_products(TcShared& sh, TcState& st, unsigned 
     __syncwarp();
 }
 
-// One tile of LT lines, by the computing threads: false if a wait ran out.
+// Line L's first element (an index), with a 32-bit division where it suffices.
+__device__ __forceinline__ long long tc_line_base(long long L, long long inner, int n) {
+    if (((L | inner) >> 32) == 0) {
+        const unsigned o = (unsigned)L / (unsigned)inner;
+        return (long long)o * n * inner + ((unsigned)L - o * (unsigned)inner);
+    }
+    const long long o = L / inner;
+    return o * n * inner + (L - o * inner);
+}
+
+// The CTA's tiles of LT lines, by the computing threads: false if a wait ran out.
 // smem: the digits (then the results); smax: LT words.
-template <int PARTS, int LT, bool STRIDED, bool CG, int STAGES>
-__device__ __forceinline__ bool tc_tile(const TcPass& g, long long tile, unsigned char* smem, unsigned char* ring,
-                                        unsigned* smax, TcShared& sh, TcState& st, uint32_t tmem,
-                                        const unsigned char* img, int tid, long long limit) {
+//
+// What a tile's 58,000 cycles (n = 256, 64 lines) were spent on, one after the
+// other: load 8,500, digits 9,500, products 9,000 and 9,000, sums 4,500 and
+// 4,500, update and store 12,500. Two of these overlap others: the digits of the
+// odd part are written while the even part's products run, and a unit's next
+// values are loaded into its registers as soon as it is stored.
+template <int PARTS, int LT, bool STRIDED, int STAGES>
+__device__ __forceinline__ bool tc_tiles(const TcPass& g, unsigned char* smem, unsigned char* ring, unsigned* smax,
+                                         TcShared& sh, TcState& st, uint32_t tmem, const unsigned char* img, int tid,
+                                         long long limit) {
     using Sh = TcShape<PARTS, LT>;
     constexpr int NT = Sh::THREADS, UPT = Sh::UPT, LBO = Sh::LBO;
     constexpr int VPU = PARTS == 2 ? 16 : 8;  // values of a unit
     constexpr bool TWO_PHASES = Sh::TWO_PHASES;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    const int n = g.n, rows = g.rows, kp = g.kp;
+    const int n = g.n, rows = g.rows, kp = g.kp, nch = kp >> 3;
     const int part_bytes = Sh::part_bytes(kp);
+    const int Emin = max(1, 64 - g.scale);
 
-    // ---- load: units (line, chunk c of 8 columns, and their mirror images) ----
-    for (int i = tid; i < LT; i += NT) smax[i] = 0;
-    tc_sync<NT>();
+    // Units (line, chunk c of 8 columns, and their mirror images). Strided axis:
+    // lanes along the lines; contiguous axis: a warp takes 4 chunks (256 bytes) of
+    // 8 lines.
     double x[UPT][VPU];  // then, as integers, the fixed-point values
-    int uline[UPT], uc[UPT];
-    const int nch = kp >> 3;
+    int uline[UPT] = {}, uc[UPT] = {};
+    auto load = [&](int it, long long tile) {
+        const int c = uc[it];
+        const long long L = tile * LT + uline[it];
+#pragma unroll
+        for (int r = 0; r < VPU; ++r) x[it][r] = 0.0;
+        if (uline[it] < 0 || L >= g.lines) return;
+        const double* p = g.src + (STRIDED ? tc_line_base(L, g.inner, n) : L * n);
+        if (!STRIDED && 8 * c + 8 <= rows) {
+            double v[8];
+            tc_load8(p + 8 * c, true, v);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) x[it][r] = v[r];
+            if constexpr (PARTS == 2) {
+                tc_load8(p + n - 8 - 8 * c, c > 0 || L + 1 < g.lines, v);
+#pragma unroll
+                for (int r = 0; r < 8; ++r) x[it][8 + r] = v[7 - r];
+            }
+            return;
+        }
+        const long long stride = STRIDED ? g.inner : 1;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int k = 8 * c + r;
+            if (k < rows) {
+                x[it][r] = p[k * stride];
+                if constexpr (PARTS == 2) x[it][8 + r] = p[(n - 1 - k) * stride];
+            }
+        }
+    };
+    // digits of one part of a unit: sums and differences in units of 2^(E - 1075),
+    // values themselves in units of 2^(E - 1076): at most 2^54 in size, rounded
+    auto digits = [&](int it, int part) {
+        constexpr int SB = PARTS == 2 ? 7 : 6;
+        constexpr unsigned long long bias = (kTcBias << SB) + (1ULL << (SB - 1));
+        if (uline[it] < 0) return;
+        unsigned long long F[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            F[r] = bias + __double_as_longlong(x[it][r]);
+            if constexpr (PARTS == 2) {
+                const long long y = __double_as_longlong(x[it][8 + r]);
+                F[r] += part == 0 ? y : -y;
+            }
+        }
+        tc_put_digits<LT, SB>(smem + part * part_bytes + uc[it] * LBO, uline[it], F);
+    };
 #pragma unroll
     for (int it = 0; it < UPT; ++it) {
         const int u = tid + it * NT;
-        // strided axis: lanes along the lines; contiguous axis: a warp takes
-        // 4 chunks (256 bytes) of 8 lines
-        const int line = STRIDED ? u % LT : (u / 32) % (LT / 8) * 8 + (u & 7);
-        const int c = STRIDED ? u / LT : (u / 32) / (LT / 8) * 4 + ((u >> 3) & 3);
-        uline[it] = line;
-        uc[it] = c;
-        const bool in_tile = c < nch;
-        if (!in_tile) uline[it] = -1;
-        const long long L = tile * LT + line;
-#pragma unroll
-        for (int r = 0; r < VPU; ++r) x[it][r] = 0.0;
-        if (in_tile && L < g.lines) {
-            if constexpr (STRIDED) {
-                const long long o = L / g.inner, i = L - o * g.inner;
-                const double* p = g.src + o * n * g.inner + i;
-#pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    const int k = 8 * c + r;
-                    if (k < rows) {
-                        x[it][r] = tc_ld<CG>(p + (long long)k * g.inner);
-                        if constexpr (PARTS == 2) x[it][8 + r] = tc_ld<CG>(p + (long long)(n - 1 - k) * g.inner);
-                    }
-                }
-            } else {
-                const double* p = g.src + L * n;
-                if (8 * c + 8 <= rows) {
-                    double v[8];
-                    tc_load8<CG>(p + 8 * c, true, v);
-#pragma unroll
-                    for (int r = 0; r < 8; ++r) x[it][r] = v[r];
-                    if constexpr (PARTS == 2) {
-                        tc_load8<CG>(p + n - 8 - 8 * c, c > 0 || L + 1 < g.lines, v);
-#pragma unroll
-                        for (int r = 0; r < 8; ++r) x[it][8 + r] = v[7 - r];
-                    }
-                } else {
-#pragma unroll
-                    for (int r = 0; r < 8; ++r) {
-                        const int k = 8 * c + r;
-                        if (k < rows) {
-                            x[it][r] = tc_ld<CG>(p + k);
-                            if constexpr (PARTS == 2) x[it][8 + r] = tc_ld<CG>(p + n - 1 - k);
-                        }
-                    }
-                }
-            }
-        }
-        if (g.jq_in) {
-            jq_flow_fixed_all(x[it], g.jin);
-        }
-        unsigned m = 0;
-#pragma unroll
-        for (int r = 0; r < VPU; ++r) m = max(m, (unsigned)__double2hiint(x[it][r]) & 0x7fffffffu);
-        if (in_tile) atomicMax(&smax[line], m);
+        uc[it] = STRIDED ? u / LT : (u / 32) / (LT / 8) * 4 + ((u >> 3) & 3);
+        uline[it] = uc[it] >= nch ? -1 : STRIDED ? u % LT : (u / 32) % (LT / 8) * 8 + (u & 7);
+        load(it, blockIdx.x);
     }
-    tc_sync<NT>();
-    // ---- digits ----
-    const int Emin = max(1, 64 - g.scale);
-#pragma unroll
-    for (int it = 0; it < UPT; ++it) {
-        if (uline[it] < 0) continue;
-        const int E = max((int)(smax[uline[it]] >> 20), Emin) + g.headroom;
-        unsigned char* chunk = smem + uc[it] * LBO;
-#pragma unroll
-        for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(tc_fixed(x[it][r], E));
-        // sums and differences in units of 2^(E - 1075), values themselves in
-        // units of 2^(E - 1076): at most 2^54 in size, rounded
-        constexpr int SB = PARTS == 2 ? 7 : 6;
-        constexpr unsigned long long bias = (kTcBias << SB) + (1ULL << (SB - 1));
-        unsigned long long F[8];
-        if constexpr (PARTS == 2) {
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-                F[r] = bias + __double_as_longlong(x[it][r]) + __double_as_longlong(x[it][8 + r]);
-            tc_put_digits<LT, SB>(chunk, uline[it], F);
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-                F[r] = bias + __double_as_longlong(x[it][r]) - __double_as_longlong(x[it][8 + r]);
-            tc_put_digits<LT, SB>(chunk + part_bytes, uline[it], F);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 8; ++r) F[r] = bias + __double_as_longlong(x[it][r]);
-            tc_put_digits<LT, SB>(chunk, uline[it], F);
-        }
-    }
-    fence_proxy_async_smem();
-    tc_sync<NT>();
 
 #pragma unroll 1
-    for (int ph = 0; ph < (TWO_PHASES ? 2 : 1); ++ph) {
-        // ---- products: the other warps wait at the barrier, not polling ----
-        bool ok = true;
-        if (warp == 0) {
-            tc_fence_after_sync();
-            tc_products<PARTS, LT, STAGES, Sh::G>(sh, st, smem, ring, tmem, TWO_PHASES ? ph : 0, TWO_PHASES ? ph + 1 : PARTS,
-                                           kp, limit);
-            ok = tc_wait(&sh.done, st.done_parity, limit, &sh.abort);
+    for (long long tile = blockIdx.x; tile < g.ntiles; tile += gridDim.x) {
+        for (int i = tid; i < LT; i += NT) smax[i] = 0;
+        tc_sync<NT>();
+#pragma unroll
+        for (int it = 0; it < UPT; ++it) {
+            if (g.jq_in) jq_flow_fixed_all(x[it], g.jin);
+            unsigned m = 0;
+#pragma unroll
+            for (int r = 0; r < VPU; ++r) m = max(m, (unsigned)__double2hiint(x[it][r]) & 0x7fffffffu);
+            if (uline[it] >= 0) atomicMax(&smax[uline[it]], m);
         }
-        if (ph == 0 && warp >= 2) tc_prefetch<LT, STRIDED>(g, tile + gridDim.x, tid - 64, NT - 64);
-        if (!Sh::OWN_PRODUCER && warp == 1)
-            tc_produce<STAGES, Sh::G>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices / Sh::G,
-                                      (TWO_PHASES ? 1 : PARTS) * (kp >> 5) * kTcSlices / Sh::G, limit);
-        st.done_parity ^= 1u;
-        if (!tc_sync_and<NT>(ok && *reinterpret_cast<volatile int*>(&sh.abort) == 0)) return false;
-        tc_fence_after_sync();
-        // ---- the order sums -> integers, through shared memory (row, line) ----
-        {
-            constexpr int GROUPS = NT / 128, CPG = LT / GROUPS < 4 ? 4 : LT / GROUPS;
-            const int row = (warp & 3) * 32 + lane;
-            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-            const int col0 = (warp >> 2) * CPG;
-            unsigned char* r0 = smem + row * Sh::PITCH;
-            unsigned char* r1 = smem + part_bytes + row * Sh::PITCH;
+        tc_sync<NT>();
+        // ---- digits (two phases: the odd part's by the issuing warps only, see below) ----
+        const bool issues = warp < 2;
+#pragma unroll
+        for (int it = 0; it < UPT; ++it) {
+            const int E = max((int)(smax[max(uline[it], 0)] >> 20), Emin) + g.headroom;
+#pragma unroll
+            for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(tc_fixed(x[it][r], E));
+            digits(it, 0);
+            if (PARTS == 2 && (!TWO_PHASES || issues)) digits(it, 1);
+        }
+        fence_proxy_async_smem();
+        tc_sync<NT>();
 #pragma unroll 1
-            for (int cc = col0; cc < col0 + CPG; cc += 4) {
-                __syncwarp();
-                uint32_t t[kTcOrders][4];
+        for (int ph = 0; ph < (TWO_PHASES ? 2 : 1); ++ph) {
+            // ---- products: the other warps wait at the barrier, not polling ----
+            bool ok = true;
+            if (warp == 0) {
+                tc_fence_after_sync();
+                tc_products<PARTS, LT, STAGES, Sh::G>(sh, st, smem, ring, tmem, TWO_PHASES ? ph : 0, TWO_PHASES ? ph + 1 : PARTS,
+                                               kp, limit);
+                ok = tc_wait(&sh.done, st.done_parity, limit, &sh.abort);
+            }
+            if (ph == 0 && !issues) {
+                if constexpr (TWO_PHASES) {
 #pragma unroll
-                for (int s = 0; s < kTcOrders; ++s) tmem_ld4(taddr + s * LT + cc, t[s]);
-                tc_wait_ld();
-                long long v[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float f[kTcOrders];
-#pragma unroll
-                    for (int s = 0; s < kTcOrders; ++s) f[s] = __uint_as_float(t[s][q]);
-                    v[q] = tc_combine(f);
+                    for (int it = 0; it < UPT; ++it) digits(it, 1);
+                    fence_proxy_async_smem();
                 }
-                long long w[4];
-                if constexpr (PARTS == 2 && !TWO_PHASES) {
+                tc_prefetch<LT, STRIDED>(g, tile + gridDim.x, tid - 64, NT - 64);
+            }
+            if (!Sh::OWN_PRODUCER && warp == 1)
+                tc_produce<STAGES, Sh::G>(sh, st, ring, img, PARTS * (kp >> 5) * kTcSlices / Sh::G,
+                                          (TWO_PHASES ? 1 : PARTS) * (kp >> 5) * kTcSlices / Sh::G, limit);
+            st.done_parity ^= 1u;
+            if (!tc_sync_and<NT>(ok && *reinterpret_cast<volatile int*>(&sh.abort) == 0)) return false;
+            tc_fence_after_sync();
+            // ---- the order sums -> integers, through shared memory (row, line) ----
+            {
+                constexpr int GROUPS = NT / 128, CPG = LT / GROUPS < 4 ? 4 : LT / GROUPS;
+                const int row = (warp & 3) * 32 + lane;
+                const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+                const int col0 = (warp >> 2) * CPG;
+                unsigned char* r0 = smem + row * Sh::PITCH;
+                unsigned char* r1 = smem + part_bytes + row * Sh::PITCH;
+#pragma unroll 1
+                for (int cc = col0; cc < col0 + CPG; cc += 4) {
+                    __syncwarp();
+                    uint32_t t[kTcOrders][4];
 #pragma unroll
-                    for (int s = 0; s < kTcOrders; ++s) tmem_ld4(taddr + Sh::REGION + s * LT + cc, t[s]);
+                    for (int s = 0; s < kTcOrders; ++s) tmem_ld4(taddr + s * LT + cc, t[s]);
                     tc_wait_ld();
+                    long long v[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         float f[kTcOrders];
 #pragma unroll
                         for (int s = 0; s < kTcOrders; ++s) f[s] = __uint_as_float(t[s][q]);
-                        w[q] = tc_combine(f);
+                        v[q] = tc_combine(f);
                     }
-                }
-                if (row < kp) {
+                    long long w[4];
+                    if constexpr (PARTS == 2 && !TWO_PHASES) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int off = (cc + q) * 8;
-                        long long* p0 = reinterpret_cast<long long*>(r0 + off);
-                        long long* p1 = reinterpret_cast<long long*>(r1 + off);
-                        if constexpr (PARTS == 1) {
-                            *p0 = v[q];
-                        } else if constexpr (TWO_PHASES) {
-                            if (ph == 0) {
+                        for (int s = 0; s < kTcOrders; ++s) tmem_ld4(taddr + Sh::REGION + s * LT + cc, t[s]);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            float f[kTcOrders];
+#pragma unroll
+                            for (int s = 0; s < kTcOrders; ++s) f[s] = __uint_as_float(t[s][q]);
+                            w[q] = tc_combine(f);
+                        }
+                    }
+                    if (row < kp) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int off = (cc + q) * 8;
+                            long long* p0 = reinterpret_cast<long long*>(r0 + off);
+                            long long* p1 = reinterpret_cast<long long*>(r1 + off);
+                            if constexpr (PARTS == 1) {
                                 *p0 = v[q];
+                            } else if constexpr (TWO_PHASES) {
+                                if (ph == 0) {
+                                    *p0 = v[q];
+                                } else {
+                                    const long long e = *p0;
+                                    *p0 = e + v[q];
+                                    *p1 = e - v[q];
+                                }
                             } else {
-                                const long long e = *p0;
-                                *p0 = e + v[q];
-                                *p1 = e - v[q];
+                                *p0 = v[q] + w[q];
+                                *p1 = v[q] - w[q];
                             }
-                        } else {
-                            *p0 = v[q] + w[q];
-                            *p1 = v[q] - w[q];
                         }
                     }
                 }
             }
+            tc_fence_before_sync();
+            tc_sync<NT>();
         }
-        tc_fence_before_sync();
-        tc_sync<NT>();
-    }
-    // ---- y = x + D x, the closing flow, store ----
+        // ---- y = x + D x, the closing flow, store; load the unit's next values ----
 #pragma unroll
-    for (int it = 0; it < UPT; ++it) {
-        const int line = uline[it], c = uc[it];
-        const long long L = tile * LT + line;
-        if (line < 0 || L >= g.lines) continue;
-        const int Eb = (int)(smax[line] >> 20);
-        const int E = max(Eb, Emin) + g.headroom;
+        for (int it = 0; it < UPT; ++it) {
+            const int line = uline[it], c = uc[it];
+            const long long L = tile * LT + line;
+            if (line >= 0 && L < g.lines) {
+                const int Eb = (int)(smax[line] >> 20);
+                const int E = max(Eb, Emin) + g.headroom;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const int off = (8 * c + r) * Sh::PITCH + line * 8;
-            const long long v = *reinterpret_cast<const long long*>(smem + off);
-            x[it][r] = tc_to_double(__double_as_longlong(x[it][r]) + tc_align(v, g.scale), E);
-            if constexpr (PARTS == 2) {
-                const long long w = *reinterpret_cast<const long long*>(smem + part_bytes + off);
-                x[it][8 + r] = tc_to_double(__double_as_longlong(x[it][8 + r]) + tc_align(w, g.scale), E);
-            }
-        }
-        if (Eb == 2047) {  // a line that holds an infinity or a NaN
-#pragma unroll
-            for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(0x7ff8000000000000LL);
-        }
-        if (g.jq_out) {
-            jq_flow_fixed_all(x[it], g.jout);
-        }
-        if constexpr (STRIDED) {
-            const long long o = L / g.inner, i = L - o * g.inner;
-            double* p = g.dst + o * n * g.inner + i;
-#pragma unroll
-            for (int r = 0; r < 8; ++r) {
-                const int k = 8 * c + r;
-                if (k < rows) {
-                    p[(long long)k * g.inner] = x[it][r];
-                    if constexpr (PARTS == 2) p[(long long)(n - 1 - k) * g.inner] = x[it][8 + r];
+                for (int r = 0; r < VPU; ++r) {
+                    const int off = (8 * c + (r & 7)) * Sh::PITCH + line * 8 + (r >> 3) * part_bytes;
+                    const long long v = *reinterpret_cast<const long long*>(smem + off);
+                    x[it][r] = tc_to_double(__double_as_longlong(x[it][r]) + tc_align(v, g.scale), E);
                 }
-            }
-        } else {
-            double* p = g.dst + L * n;
-            if (8 * c + 8 <= rows) {
-                double v[8];
+                if (Eb == 2047) {  // a line that holds an infinity or a NaN
 #pragma unroll
-                for (int r = 0; r < 8; ++r) v[r] = x[it][r];
-                tc_store8(p + 8 * c, v);
-                if constexpr (PARTS == 2) {
-#pragma unroll
-                    for (int r = 0; r < 8; ++r) v[r] = x[it][15 - r];
-                    tc_store8(p + n - 8 - 8 * c, v);
+                    for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(0x7ff8000000000000LL);
                 }
-            } else {
+                if (g.jq_out) jq_flow_fixed_all(x[it], g.jout);
+                double* p = g.dst + (STRIDED ? tc_line_base(L, g.inner, n) : L * n);
+                if (!STRIDED && 8 * c + 8 <= rows) {
+                    double v[8];
 #pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    const int k = 8 * c + r;
-                    if (k < rows) {
-                        p[k] = x[it][r];
-                        if constexpr (PARTS == 2) p[n - 1 - k] = x[it][8 + r];
+                    for (int r = 0; r < 8; ++r) v[r] = x[it][r];
+                    tc_store8(p + 8 * c, v);
+                    if constexpr (PARTS == 2) {
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) v[r] = x[it][15 - r];
+                        tc_store8(p + n - 8 - 8 * c, v);
+                    }
+                } else {
+                    const long long stride = STRIDED ? g.inner : 1;
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) {
+                        const int k = 8 * c + r;
+                        if (k < rows) {
+                            p[k * stride] = x[it][r];
+                            if constexpr (PARTS == 2) p[(n - 1 - k) * stride] = x[it][8 + r];
+                        }
                     }
                 }
             }
+            if (tile + gridDim.x < g.ntiles) load(it, tile + gridDim.x);
         }
+        tc_sync<NT>();  // results and smax are rewritten by the next tile
     }
-    tc_sync<NT>();  // results and smax are rewritten by the next tile
     return true;
 }
 

@@ -35,6 +35,13 @@ __device__ __forceinline__ void tc_put_digits32(unsigned char* chunk, int line, 
 
 // Eight consecutive values at any 4-byte aligned p, as tc_load8.
 __device__ __forceinline__ void tc_load8(const float* p, bool inside, float (&v)[8]) {
+    if ((reinterpret_cast<uintptr_t>(p) & 31) == 0) {  // a sector
+        asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "l"(p)
+                     : "memory");
+        return;
+    }
     const unsigned s = (unsigned)(reinterpret_cast<uintptr_t>(p) >> 2) & 3u;
     if (s != 0 && !inside) {
 #pragma unroll
@@ -55,6 +62,12 @@ __device__ __forceinline__ void tc_load8(const float* p, bool inside, float (&v)
     for (int r = 0; r < 8; ++r) v[r] = s & 2u ? h[r + 2] : h[r];
 }
 __device__ __forceinline__ void tc_store8(float* p, const float (&v)[8]) {
+    if ((reinterpret_cast<uintptr_t>(p) & 31) == 0) {
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                     "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                     : "memory");
+        return;
+    }
     auto two = [&](int i) { *reinterpret_cast<float2*>(p + i) = make_float2(v[i], v[i + 1]); };
     auto four = [&](int i) { *reinterpret_cast<float4*>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]); };
     switch ((unsigned)(reinterpret_cast<uintptr_t>(p) >> 2) & 3u) {
