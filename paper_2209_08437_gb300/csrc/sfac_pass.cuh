@@ -761,6 +761,100 @@ axis_pass_cta_rows_kernel(const PassArgs a0, long long ngroups) {
     }
 }
 
+// The same lines on a strided axis whose columns come in whole sectors (32 bytes:
+// four line pairs). axis_pass_cta_rows_kernel reads and writes 8 LPC bytes of a row
+// a CTA, a quarter of each sector at 4096 points, and waits for those loads most
+// of the time. Here the CL = 4 / LPC CTAs that share the sectors form a cluster: each
+// loads N / CL rows of all four pairs, hands every pair to the CTA that transforms
+// it through distributed shared memory (into its exchange region), and the results
+// go back the same way. Same lines, same arithmetic, same bits.
+template <int N, int LPC>
+__global__ void __launch_bounds__(LPC * (N / 16), 1) axis_pass_cluster_rows_kernel(const PassArgs a0,
+                                                                                  long long ngroups) {
+    constexpr int E = 16, T = N / E, NT = LPC * T, CL = 4 / LPC, RPT = N / CL / NT;  // rows a thread moves
+    static_assert(RPT * 8 == 2 * E, "as many values moved as transformed");
+    using Ex = PadExchange<float, N, LPC, true>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PassArgs a = a0;
+    pass_next_may_start();
+    SmemTables<float, N, E, false>::load(a, smem_raw);
+    pass_wait_for_previous();
+    const int tid = threadIdx.x, j = tid % LPC, t = tid / LPC;
+    unsigned rank;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    float2* land = reinterpret_cast<float2*>(smem_raw + SmemTables<float, N, E, false>::BYTES);  // [pair][row]
+    const Ex ex{reinterpret_cast<C2<float>*>(land), j};
+    uint32_t peer[CL];  // the landing areas of the cluster's CTAs
+#pragma unroll
+    for (int q = 0; q < CL; ++q) {
+        const uint32_t mine = static_cast<uint32_t>(__cvta_generic_to_shared(land));
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer[q]) : "r"(mine), "r"(q));
+    }
+    auto cluster_sync = []() {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    };
+    const int row0 = (int)rank * (N / CL) + tid;
+    const long long octets = a.inner >> 3;
+    auto at = [&](long long g, int i) {
+        const long long o = g / octets;
+        return o * N * a.inner + 8 * (g - o * octets) + (long long)(row0 + i * NT) * a.inner;
+    };
+    float xn[RPT][8];
+    auto load = [&](long long g) {
+        const float* u = static_cast<const float*>(a.u);
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+            asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=f"(xn[i][0]), "=f"(xn[i][1]), "=f"(xn[i][2]), "=f"(xn[i][3]), "=f"(xn[i][4]),
+                           "=f"(xn[i][5]), "=f"(xn[i][6]), "=f"(xn[i][7])
+                         : "l"(u + at(g, i))
+                         : "memory");
+    };
+    const long long step = gridDim.x / CL;
+    long long g = blockIdx.x / CL;
+    if (g < ngroups) load(g);
+    for (; g < ngroups; g += step) {
+        cluster_sync();  // every CTA has left its exchange region
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(
+                                 peer[q / LPC] + 8u * (unsigned)(q % LPC * N + row0 + i * NT)),
+                             "f"(xn[i][2 * q]), "f"(xn[i][2 * q + 1])
+                             : "memory");
+        cluster_sync();
+        C2<float> x[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const float2 v = land[j * N + t + e * T];
+            x[e] = {v.x, v.y};
+        }
+        if (g + step < ngroups) load(g + step);  // in flight during the transforms
+        __syncthreads();
+        fused_pass<float, N, E, false, false, true>(x, t, a, ex);
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) land[j * N + t + e * T] = make_float2(x[e].x, x[e].y);
+        cluster_sync();
+        float* d = static_cast<float*>(a.u) + a.out_shift;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            float y[8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+                             : "=f"(y[2 * q]), "=f"(y[2 * q + 1])
+                             : "r"(peer[q / LPC] + 8u * (unsigned)(q % LPC * N + row0 + i * NT))
+                             : "memory");
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + at(g, i)), "f"(y[0]),
+                         "f"(y[1]), "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]), "f"(y[7])
+                         : "memory");
+        }
+    }
+    cluster_sync();  // no CTA leaves while another reads its shared memory
+}
+
 // ---------------------------------------------------------------------------
 // Launch configuration
 // ---------------------------------------------------------------------------
@@ -868,6 +962,48 @@ cudaError_t launch_cta_rows(const PassArgs& a, cudaStream_t s) {
     return launch_overlapped(kern, (unsigned)grid, LPC * (N / E), smem, s, a, ngroups);
 }
 
+// Whether axis_pass_cluster_rows_kernel takes the pass: whole 32-byte sectors of
+// every row, in device memory.
+inline bool cluster_rows_eligible(const PassArgs& a) {
+    return a.inner > 1 && a.inner % 8 == 0 && !a.host_io && a.nmem > 0 &&
+           reinterpret_cast<unsigned long long>(a.u) % 32 == 0 && a.out_shift % 8 == 0;
+}
+
+template <int N, int LPC>
+cudaError_t launch_cluster_rows(const PassArgs& a, cudaStream_t s) {
+    constexpr int CL = 4 / LPC, NT = LPC * (N / 16);
+    using Ex = PadExchange<float, N, LPC, true>;
+    const size_t smem = SmemTables<float, N, 16, false>::BYTES + sizeof(C2<float>) * (size_t)Ex::elems();
+    auto kern = axis_pass_cluster_rows_kernel<N, LPC>;
+    static LaunchSetup setup;
+    int dev = 0;
+    cudaError_t err = set_smem(kern, smem, setup, &dev);
+    if (err != cudaSuccess) return err;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {CL, 1, 1};
+    attr[1] = pass_overlap_attribute();
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    int clusters = setup.resident[dev].load();  // resident at once, asked once per device
+    if (clusters == 0) {
+        cfg.gridDim = dim3(CL);
+        cfg.numAttrs = 1;
+        err = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+        if (err != cudaSuccess) return err;
+        clusters = clusters < 1 ? 1 : clusters;
+        setup.resident[dev].store(clusters);
+    }
+    const long long ngroups = a.outer * (a.inner / 8);
+    if (ngroups <= 0) return cudaSuccess;
+    cfg.gridDim = dim3((unsigned)(CL * (ngroups < clusters ? ngroups : clusters)));
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, a, ngroups);
+}
+
 // SMs of the current device (cached per device; 0 if unknown).
 inline int current_device_sms() {
     static std::atomic<int> cache[LaunchSetup::kMaxDevices] = {};
@@ -938,6 +1074,8 @@ cudaError_t launch_n(const PassArgs& a, cudaStream_t s) {
         // 0.437 ms, 2048^2 0.140 -> 0.107 ms). At 1024 points the grid is
         // latency bound and the per-CTA table build cost more (0.036 -> 0.046 ms).
         if constexpr (N >= 2048) {
+            if constexpr (!PADDED)
+                if (cluster_rows_eligible(a)) return launch_cluster_rows<N, LPC_S>(a, s);
             if (a.inner > 1) return launch_cta_rows<R, N, 16, LPC_S, true, PADDED>(a, s);
             return launch_cta_rows<R, N, 16, 1, false, PADDED>(a, s);
         }
