@@ -82,6 +82,10 @@ FP32_PEAK_TFLOPS = 128 * 152 * 2 * SM_CLOCK_GHZ / 1e3
 PEAK_SOURCE = {"f64": "derived: 2 FP64 fma/clk/SM x 152 SMs x 2 flops x 2.07 GHz",
                "f32": "derived: 128 FP32 lanes x 152 SMs x 2 flops x 2.07 GHz"}
 
+# FP64 axes of these lengths run on the tensor cores: 21 products of FP16 digits, over
+# n^2 (n <= 128) or n^2 / 2 (folded) multiply-adds a line.
+TC_MIN_N, TC_MAX_N = 17, 1024
+
 # DRAM bytes (read + write) per launch from ncu, keyed by (workload, precision,
 # axis): the mean of dram__bytes_read.sum + dram__bytes_write.sum over the
 # captured launches of each pass, from
@@ -91,14 +95,11 @@ PEAK_SOURCE = {"f64": "derived: 2 FP64 fma/clk/SM x 152 SMs x 2 flops x 2.07 GHz
 # (-c 28 for 2d1024 and 2d4096, -c 42 for 3d256, -s 15 -c 15 for 3d512). An entry is
 # removed when its kernel changes.
 NCU_TRAFFIC = {
-    ("2d1024", "f64", 0): 8570000, ("2d1024", "f64", 1): 8585714,
     ("2d1024", "f32", 0): 4281429, ("2d1024", "f32", 1): 4291429,
-    ("3d256", "f64", 0): 203777143, ("3d256", "f64", 1): 209997143, ("3d256", "f64", 2): 209608571,
     ("3d256", "f32", 0): 72635714, ("3d256", "f32", 1): 75765714, ("3d256", "f32", 2): 75717143,
-    ("3d512", "f64", 0): 2085800000, ("3d512", "f64", 1): 2090875000, ("3d512", "f64", 2): 2091510000,
     ("3d512", "f32", 0): 1008836667, ("3d512", "f32", 1): 1014696667, ("3d512", "f32", 2): 1014876667,
     ("2d4096", "f64", 0): 205950000, ("2d4096", "f64", 1): 213458571,
-    ("2d4096", "f32", 0): 71625714, ("2d4096", "f32", 1): 78167143,
+    ("2d4096", "f32", 0): 71625714,
 }
 
 
@@ -285,6 +286,24 @@ def roofline(workload, problem, res, prec_name, peaks_live):
     tflops = flops / t / 1e12
     gbs = bytes_ / t / 1e9
     hbm = measured_peaks().get("hbm_gbs", 6800.0)
+    if prec_name == "f64" and TC_MIN_N <= problem.n[ax] <= TC_MAX_N:
+        # tensor-core pass: the FP64 pipe bounds nothing; what it cannot do without is
+        # the field's traffic and the digit products
+        n = problem.n[ax]
+        tensor = (42.0 if n <= 128 else 21.0) * n * pts / t / 1e12
+        peak = measured_peaks().get("bf16_tflops", 1900.0)
+        if gbs / hbm >= tensor / peak:
+            out = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
+                   "peak_source": "measured copy bandwidth (MEASURED_PEAKS.json)"}
+        else:
+            out = {"bound": "tensor", "achieved": tensor, "peak": peak, "unit": "TFLOP/s", "frac": tensor / peak,
+                   "peak_source": "measured cuBLAS bf16 rate (MEASURED_PEAKS.json); FP16 digit products"}
+        out.update({"traffic": NCU_TRAFFIC.get((workload, prec_name, ax)),
+                    "kernel": f"tensor-core pass axis {ax + 1} (n={n})", "kernel_ms": axis_avg[ax],
+                    "per_axis_ms": axis_avg, "algorithmic_bytes": bytes_, "algorithmic_flops": flops,
+                    "fft_equivalent_tflops": tflops, "hbm_gbs": gbs, "hbm_frac_of_measured": gbs / hbm,
+                    "tensor_tflops": tensor, "tensor_frac_of_measured": tensor / peak})
+        return out
     peak = FP64_PEAK_TFLOPS if prec_name == "f64" else FP32_PEAK_TFLOPS
     frac_alu, frac_hbm = tflops / peak, gbs / hbm
     if frac_alu >= frac_hbm:

@@ -80,8 +80,12 @@ typedef struct sfac_plan sfac_plan;
  * and any 2 <= n[l] <= 2048 otherwise: then e^{tau/2 C} and e^{tau S}, both
  * symmetric Toeplitz matrices, are applied as linear convolutions with their
  * first columns, zero-padded to a power of two L >= 2n - 1 (real multipliers,
- * no twist); an axis whose stride is odd takes that path too. Other lengths
- * return SFAC_EUNSUPPORTED. The plan owns its device tables and
+ * no twist); an axis whose stride is odd takes that path too. FP64 axes of 17 to
+ * 1024 points, and zero-padded FP32 axes of 65 to 256, apply the same factor as
+ * a dense operator on the tensor cores (exact sums of fixed-point digit products;
+ * the plan keeps the operator's digits, up to 6.3 MB an axis at 1024 points, and
+ * an axis whose operator would not keep them exact stays with the FFTs). Other
+ * lengths return SFAC_EUNSUPPORTED. The plan owns its device tables and
  * any staging buffer; free it with sfac_plan_destroy. On success *out is set;
  * on failure *out is NULL. The call synchronises `stream` once (upload). */
 sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan** out);
@@ -96,6 +100,8 @@ sfac_status sfac_plan_info(const sfac_plan* plan, int axis, int* fft_len, int* p
 #define SFAC_KERNEL_CTA 0    /* lines spread over a CTA, CTA-wide exchanges (FP64; FP32 N >= 1024, persistent CTAs from 2048) */
 #define SFAC_KERNEL_WARP 1   /* FP32, 32 <= N <= 512: lines held inside one warp, persistent CTAs */
 #define SFAC_KERNEL_STAGED 2 /* the warp kernel fed by TMA tile copies (FP32 strided axes) */
+/* A pass on the tensor cores reports the kind of the FFT pass it replaces: CTA
+ * for FP64, WARP for zero-padded FP32 axes. */
 
 /* Which kernel a pass of axis `axis` would use for the field at u_dev: *kind
  * receives one of SFAC_KERNEL_*. The staged kernel needs an FP32 plan, a
@@ -116,7 +122,7 @@ sfac_status sfac_plan_kernel(const sfac_plan* plan, int axis, const void* u_dev,
  * call in one cooperative launch: two steps or more, every axis a spectral
  * (not zero-padded) pass of 32..256 points, at most 65536 unknowns, and every
  * line's warp resident at once on the device (one 32-thread CTA per line pair,
- * N/32 values per thread). The CTAs meet at a grid-wide barrier between passes;
+ * N/32 values per thread; FP64: tiles of 8 lines on the tensor cores). The CTAs meet at a grid-wide barrier between passes;
  * each wait on it is bounded by the plan's wait limit (sfac_plan_set_wait_limit,
  * whose hold hook makes the first wait of every CTA run out), and a wait that
  * runs out is reported by sfac_plan_check. Otherwise SFAC_STEP_PASSES: one
@@ -126,15 +132,15 @@ sfac_status sfac_plan_step_kernel(const sfac_plan* plan, long long nsteps, int* 
 /* Synchronise `stream`, then report whether an axis pass of this plan gave up
  * on one of its bounded waits since the last check: SFAC_ETIMEOUT if so (the
  * field written by that pass is not valid; the flag is cleared), SFAC_OK
- * otherwise. The staged kernel waits on its tile copies and the whole-call
- * launch of small grids on its grid barrier (about two seconds at most per
- * wait); sfac_step_host checks automatically. The paper has no counterpart. */
+ * otherwise. The staged kernel waits on its tile copies, a tensor-core pass on
+ * its operator's copies and its products, and the whole-call launch of small grids
+ * on its grid barrier (about two seconds at most per wait); sfac_step_host checks automatically. The paper has no counterpart. */
 sfac_status sfac_plan_check(sfac_plan* plan, void* stream);
 
 /* Limit of each bounded wait of the plan's passes, in SM clock cycles
  * (default 2^32, about two seconds at 2.07 GHz; must be >= 1). hold != 0 is a
- * test hook: the first wait of every CTA of a staged pass then waits for a
- * barrier that nothing completes, so it runs out after wait_cycles, the pass
+ * test hook: the first wait of every CTA of a staged or tensor-core pass then
+ * waits for a barrier that nothing completes, so it runs out after wait_cycles, the pass
  * records the timeout (see sfac_plan_check) and leaves the field partly
  * updated. Host-only. The paper has no counterpart. */
 sfac_status sfac_plan_set_wait_limit(sfac_plan* plan, long long wait_cycles, int hold);
@@ -146,7 +152,8 @@ sfac_status sfac_plan_destroy(sfac_plan* plan);
 /* Advance the device field u_dev (layout above, plan precision) by `nsteps`
  * complete steps of eq. (finalstrang) on `stream`; nsteps = 0 is a no-op.
  * Each axis is one fused pass over the field (load, J^Q if first, six FFTs
- * with the eigenvalue multiplies and the twist, J^Q if last, store); inside one
+ * with the eigenvalue multiplies and the twist, or their product as one dense
+ * operator on the tensor cores, J^Q if last, store); inside one
  * call the closing J^Q_{tau/2} of a step and the opening J^Q_{tau/2} of the
  * next are applied together as J^Q_{tau} (exact: J^Q is a flow). u_dev is
  * updated in place and must not be accessed by other streams until the work
@@ -165,7 +172,9 @@ sfac_status sfac_solve(sfac_plan* plan, void* u_dev, double T, void* stream);
  * load / store: 0 none, 1 J^Q_{tau/2}, 2 J^Q_{tau} (eq. (nonlinear_operator)).
  * sfac_step(plan, u, 1) launches exactly axis_pass(0, 1, 0), axis_pass(1, 0, 0),
  * ..., axis_pass(dim-1, 0, 1) (for dim = 1: axis_pass(0, 1, 1)); this entry point
- * exposes one such launch so that callers can time or test it alone.
+ * exposes one such pass so that callers can time or test it alone (one launch;
+ * two for an FP64 axis of 257 to 1024 points with jq_in, whose flow is a launch
+ * of its own).
  * SFAC_EINVAL for a bad axis, mode or pointer. */
 sfac_status sfac_axis_pass(sfac_plan* plan, void* u_dev, int axis, int jq_in, int jq_out, void* stream);
 
@@ -174,7 +183,8 @@ sfac_status sfac_axis_pass(sfac_plan* plan, void* u_dev, int axis, int jq_in, in
  * - (1/2) u^T A u ), h^d the product of the axes' h, A u = sum_l B_l along axis l.
  * u^T A u is accumulated line by line as x . B_l x with B_l x formed through the
  * spectra of C_l and S_l (zero-padded axes: one linear convolution with B_l's
- * column); FP64 arithmetic for both precisions; partial sums are added in a
+ * column), or on small grids (sum over all lines of n^2/2 up to 2.4e7) as a
+ * direct Toeplitz sum; FP64 arithmetic for both precisions; partial sums are added in a
  * fixed order (deterministic). u_dev is read only. Synchronises `stream`. */
 sfac_status sfac_diagnostics(sfac_plan* plan, const void* u_dev, double* out, void* stream);
 
@@ -411,9 +421,10 @@ sfac_status sfac_probe_fma(int kind, int blocks, long long iters, void* out_dev,
 
 /* The nonlinear flow J^Q_s(v) = v / sqrt(E + (1 - E) v^2), E = e^{-2s} (the
  * exact solution of u' = u - u^3 over time s, Sec. 2.2), evaluated on n values
- * by the very device code the passes use: v times the double reciprocal
- * square root of E + (1 - E) v^2 in the FP64 passes, v plus the increment of
- * the FP32 passes (which use 1 - E only). It lets a test measure that code's error value by value; the paper
+ * by the very device code the passes use: the 64-bit fixed-point form of the
+ * FP64 tensor-core passes (v times the double reciprocal square root of
+ * E + (1 - E) v^2, the FP64 FFT passes' form, outside its range: |v| >= 4 or
+ * E < 1/4), v plus the increment of the FP32 passes (which use 1 - E only). It lets a test measure that code's error value by value; the paper
  * has no counterpart. prec SFAC_FP64 / SFAC_FP32 sets the element type of
  * v_dev and out_dev (n elements each, device memory, may be the same buffer);
  * E in (0, 1] and one_minus_E = 1 - E as the plans compute them. Enqueued on

@@ -665,7 +665,7 @@ static sfac_status status_after_sync(sfac_plan* plan, cudaStream_t st) {
     cudaError_t err = cudaMemsetAsync(plan->status, 0, sizeof(unsigned int), st);
     if (err == cudaSuccess) err = cudaStreamSynchronize(st);
     if (err != cudaSuccess) return cuda_fail(err, "status reset");
-    return fail(SFAC_ETIMEOUT, "an axis pass gave up waiting for a staged tile copy; the field is not valid");
+    return fail(SFAC_ETIMEOUT, "an axis pass gave up one of its bounded waits; the field is not valid");
 }
 
 sfac_status sfac_plan_set_wait_limit(sfac_plan* plan, long long wait_cycles, int hold) try {

@@ -4,7 +4,8 @@
 // symmetric Toeplitz with first columns g, h) the linear factor of an axis is
 //   P = (I + G)(I + H)(I + G) = I + D,  D = G + W + G W,  W = H + G + H G.
 // D is formed in FP64 from the increments, so its rounding is relative to D
-// itself. It runs once per plan (n = 256: 34 M multiply-adds).
+// itself. It runs once per plan (n = 256: 17 M multiply-adds an axis; plan creation for
+// 3D 256^3 0.7 -> 1.3 ms, for 2D 1024^2 4.6 -> 9.0 ms).
 #include <cuda_fp16.h>
 
 #include <algorithm>

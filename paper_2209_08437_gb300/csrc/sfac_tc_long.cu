@@ -13,7 +13,10 @@
 // barrier separates the last load of the lines from the first store.
 //
 // Eight warps convert, drain and store; one more issues the copies and one the
-// products.
+// products. Measured on 2D 1024^2 (side by side, passes without the flow): 205 us a
+// pass by FFTs on the FP64 pipe (90% busy), 62 us contiguous and 54 us strided here;
+// 512^2 37 and 33 us. The loads' latency and the conversion bound it (long-scoreboard
+// stalls 4-5 per issue, ALU 25-31%, tensor pipe 18%).
 #include <cuda_runtime.h>
 
 #include <atomic>

@@ -1,7 +1,7 @@
 // sfac_tc_steps.cu - FP64 tensor-core passes with few lines: tiles of 8 lines, and a
 // whole sfac_step call on a small grid in one launch.
 //
-// With fewer than 16 lines an SM the latency of one tile bounds a pass: load,
+// With at most 8 lines an SM the latency of one tile bounds a pass: load,
 // digits, products, sums, store. The arithmetic is that of sfac_tc_tile.cuh; what
 // differs is the code: a thread works on pairs of columns in rolled loops and
 // the lines' values stay in shared memory, so that the whole pass is a few KB

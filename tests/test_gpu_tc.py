@@ -179,3 +179,56 @@ def test_fp32_padded_lengths(n):
                 ref = O.apply_axis(ref, P, ax + 1)
                 ref = O.nonlinear_flow(ref, prob.tau) if jq[1] else ref
                 assert np.abs(u.double().cpu().numpy() - ref).max() <= 1.8e-7
+
+
+ROUTES = [((255, 63), S.SFAC_FP64), ((300, 40), S.SFAC_FP64), ((128, 96, 100), S.SFAC_FP64), ((127, 250), S.SFAC_FP32),
+          ((1024, 64), S.SFAC_FP32), ((32, 256, 80), S.SFAC_FP32), ((16, 2048), S.SFAC_FP32)]
+
+
+def field(prob, prec, seed):
+    dt = torch.float64 if prec == S.SFAC_FP64 else torch.float32
+    return torch.tensor(np.ascontiguousarray(I.random_field(prob, seed)), dtype=dt, device="cuda")
+
+
+@pytest.mark.parametrize("n,prec", ROUTES, ids=str)
+def test_steps_in_a_cuda_graph(n, prec):
+    """The overlapped launches of a call's passes can be captured and replayed:
+    same bits as the direct calls."""
+    prob = I.Problem(n=n, alpha=(1.3, 1.7, 1.5)[: len(n)], eps=0.06, tau=2e-3)
+    with S.Plan.for_problem(prob, prec) as plan:
+        u, ref = field(prob, prec, 79), field(prob, prec, 79)
+        for _ in range(3):
+            plan.step(ref, 1)
+        torch.cuda.synchronize()
+        side = torch.cuda.Stream()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(side):
+            with torch.cuda.graph(g, stream=side):
+                plan.step(u, 1, stream=side.cuda_stream)
+        u.copy_(field(prob, prec, 79))
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        plan.check()
+    assert torch.equal(u, ref)
+
+
+@pytest.mark.parametrize("n,prec", ROUTES, ids=str)
+def test_one_plan_on_two_streams(n, prec):
+    """The passes keep nothing in the plan: two fields advance on two streams at
+    the same time with the bits of one after the other."""
+    prob = I.Problem(n=n, alpha=(1.3, 1.7, 1.5)[: len(n)], eps=0.06, tau=2e-3)
+    with S.Plan.for_problem(prob, prec) as plan:
+        want = [field(prob, prec, 90 + i) for i in range(2)]
+        for u in want:
+            for _ in range(6):
+                plan.step(u, 1)
+        got = [field(prob, prec, 90 + i) for i in range(2)]
+        torch.cuda.synchronize()
+        streams = [torch.cuda.Stream() for _ in range(2)]
+        for _ in range(6):
+            for u, s in zip(got, streams):
+                plan.step(u, 1, stream=s.cuda_stream)
+        torch.cuda.synchronize()
+        plan.check()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
