@@ -15,16 +15,19 @@
 //
 // Kernel shapes that share that chain:
 //  - axis_pass_kernel: a line's T = N/E threads may span several warps, so the
-//    exchanges synchronise the CTA (FP64 at every N; FP32 below 32 and at
-//    1024 points);
+//    exchanges synchronise the CTA (FP64; FP32 below 32 and at 1024 points);
 //  - axis_pass_cta_rows_kernel: the same lines in persistent CTAs that keep
 //    the tables and twiddle rows in shared memory (FP32, 2048 and 4096 points);
+//  - axis_pass_cluster_rows_kernel: 4096-point lines on strided axes, in clusters
+//    that share whole sectors of the rows;
 //  - axis_pass_warp_kernel: 16 values per thread, so a line of N <= 512 points
 //    lives inside one warp (with 32/T lines per warp); the exchanges need only
 //    warp-level synchronisation; persistent CTAs keep the tables in shared
 //    memory (FP32, 32 <= N <= 512);
 //  - the TMA-staged kernel of sfac_pass_staged_f32.cu (FP32 strided axes) and
 //    the batch kernel of sfac_batch.cuh run the same warp-local lines.
+// FP64 axes of 17..1024 points and zero-padded FP32 axes of 65..256 do not come
+// here: they run on the tensor cores (sfac_tc_tile.cuh).
 // The FP32 chain is the increment form, rolled for N <= SFAC_ROLLED_MAX_N.
 // The FP64 CTA kernel runs its FFTs on ratio twiddles (FftPassRatio in
 // sfac_fft.cuh, records in PassArgs::rtwid); the batch kernel uses the complex
@@ -768,6 +771,8 @@ axis_pass_cta_rows_kernel(const PassArgs a0, long long ngroups) {
 // loads N / CL rows of all four pairs, hands every pair to the CTA that transforms
 // it through distributed shared memory (into its exchange region), and the results
 // go back the same way. Same lines, same arithmetic, same bits.
+// Bound by the loads' latency and the two cluster barriers a group. Side by side on
+// GB300: 2D 4096^2 strided pass 241 -> 203 us, 64 x 4096 33 -> 17 us.
 template <int N, int LPC>
 __global__ void __launch_bounds__(LPC * (N / 16), 1) axis_pass_cluster_rows_kernel(const PassArgs a0,
                                                                                   long long ngroups) {
@@ -872,6 +877,7 @@ struct LaunchSetup {
     static constexpr int kMaxDevices = 64;
     std::atomic<unsigned long long> configured{0};  // bit d: attribute set on device d
     std::atomic<int> resident[kMaxDevices] = {};
+    std::atomic<int> most[kMaxDevices] = {};      // launch_spread: the dynamic shared memory of a CTA alone on an SM
 };
 
 template <class K>
@@ -901,6 +907,64 @@ cudaError_t resident_grid(K kern, int threads, size_t smem, LaunchSetup& ls, int
     }
     *grid = r;
     return cudaSuccess;
+}
+
+// SMs of the current device (cached per device; 0 if unknown).
+inline int current_device_sms() {
+    static std::atomic<int> cache[LaunchSetup::kMaxDevices] = {};
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= LaunchSetup::kMaxDevices) {
+        cudaGetLastError();
+        return 0;
+    }
+    if ((sms = cache[dev].load()) != 0) return sms;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    cache[dev].store(sms);
+    return sms;
+}
+
+// Set-up of a kernel for launch_spread, in place of set_smem (once per device).
+constexpr int kSmShared = 228 * 1024, kCtaReserved = 1024;  // bytes of an SM, and of it a CTA's system share
+template <class K>
+cudaError_t set_smem_spread(K kern, LaunchSetup& ls, int* dev_out) {
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    if (dev < 0 || dev >= LaunchSetup::kMaxDevices) return cudaErrorInvalidDevice;
+    *dev_out = dev;
+    if (ls.most[dev].load() != 0) return cudaSuccess;
+    cudaFuncAttributes fa;
+    err = cudaFuncGetAttributes(&fa, kern);
+    if (err != cudaSuccess) return err;
+    const int most = (kSmShared - kCtaReserved - (int)fa.sharedSizeBytes) & ~127;
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (err == cudaSuccess) ls.most[dev].store(most);
+    return err;
+}
+
+// An overlapped launch whose CTAs are spread over the SMs. CTAs placed while the
+// previous pass runs go to whichever SMs it leaves free, several on one, and a pass
+// that had one CTA for every SM then ran on a part of them. So each CTA asks for
+// shared memory (`smem` is what it uses) that leaves room on an SM for its even share
+// of the grid, or for four warps, one a scheduler, where that is more. FP32 steps side
+// by side on GB300, plain / overlapped / spread: 1024 x 256 20.9 / 26.2 / 18.6 us,
+// 64 x 128 x 64 25.1 / 28.7 / 17.5, 64 x 128 x 128 31.2 / 29.2 / 21.9, 256 x 256 22.2 /
+// 10.9 / 10.6 (17.9 without the four warps, which keep room beside the previous
+// pass's CTAs). axis_pass_kernel stays as it is: 1024 x 1024 31.2 / 26.8 / 29.0.
+template <typename... P, typename... A>
+cudaError_t launch_spread(void (*kern)(P...), long long grid, unsigned block, size_t smem, const LaunchSetup& ls,
+                          int dev, cudaStream_t s, const A&... args) {
+    const int sms = current_device_sms();
+    if (sms > 0 && grid < ls.resident[dev].load()) {  // a full grid has no room to pile up
+        const long long even = (grid + sms - 1) / sms, free_warps = 4 / (block / 32);
+        const long long share = kSmShared / (even > free_warps ? even : free_warps);
+        const long long room = (share - (kSmShared - ls.most[dev].load())) & ~127LL;
+        if (room > (long long)smem) smem = (size_t)room;
+    }
+    return launch_overlapped(kern, (unsigned)grid, block, smem, s, args...);
 }
 
 template <typename R, int N, int E, int LPC, bool STRIDED, bool PADDED>
@@ -936,14 +1000,14 @@ cudaError_t launch_warp(const PassArgs& a, cudaStream_t s) {
     auto kern = axis_pass_warp_kernel<R, N, E, WPB, STRIDED, PADDED>;
     static LaunchSetup setup;
     int dev = 0, resident = 0;
-    cudaError_t err = set_smem(kern, smem, setup, &dev);
+    cudaError_t err = set_smem_spread(kern, setup, &dev);
     if (err == cudaSuccess) err = resident_grid(kern, WPB * 32, smem, setup, dev, &resident);
     if (err != cudaSuccess) return err;
     const long long ngroups = (a.clines + LPW - 1) / LPW;
     if (ngroups <= 0) return cudaSuccess;
     const long long want = (ngroups + WPB - 1) / WPB;
     const long long grid = want < resident ? want : resident;
-    return launch_overlapped(kern, (unsigned)grid, WPB * 32, smem, s, a, ngroups);
+    return launch_spread(kern, grid, WPB * 32, smem, setup, dev, s, a, ngroups);
 }
 
 template <typename R, int N, int E, int LPC, bool STRIDED, bool PADDED>
@@ -1004,23 +1068,6 @@ cudaError_t launch_cluster_rows(const PassArgs& a, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, kern, a, ngroups);
 }
 
-// SMs of the current device (cached per device; 0 if unknown).
-inline int current_device_sms() {
-    static std::atomic<int> cache[LaunchSetup::kMaxDevices] = {};
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= LaunchSetup::kMaxDevices) {
-        cudaGetLastError();
-        return 0;
-    }
-    if ((sms = cache[dev].load()) != 0) return sms;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    cache[dev].store(sms);
-    return sms;
-}
-
 // Values per thread that give a line 32 threads (at least 2 values): the
 // shape of the small-grid passes below.
 template <int N>
@@ -1074,7 +1121,11 @@ cudaError_t launch_n(const PassArgs& a, cudaStream_t s) {
         // 0.437 ms, 2048^2 0.140 -> 0.107 ms). At 1024 points the grid is
         // latency bound and the per-CTA table build cost more (0.036 -> 0.046 ms).
         if constexpr (N >= 2048) {
-            if constexpr (!PADDED)
+            // Strided axes of 4096 points go to the cluster kernel wherever the sectors are
+            // whole: 241 -> 203 us on 4096^2, 33 -> 17 us on 64 x 4096. A 2048-point CTA
+            // holds two pairs, half a sector, and its cluster barriers cost more than the
+            // other half (2048^2 41 -> 47 us, 64 x 2048 11.6 -> 13.2 us).
+            if constexpr (!PADDED && N == 4096)
                 if (cluster_rows_eligible(a)) return launch_cluster_rows<N, LPC_S>(a, s);
             if (a.inner > 1) return launch_cta_rows<R, N, 16, LPC_S, true, PADDED>(a, s);
             return launch_cta_rows<R, N, 16, 1, false, PADDED>(a, s);

@@ -244,14 +244,14 @@ cudaError_t launch_staged(const PassArgs& a, cudaStream_t s) {
     auto kern = axis_pass_staged_kernel<N>;
     static LaunchSetup setup;
     int dev = 0, resident = 0;
-    cudaError_t err = set_smem(kern, Sh::SMEM, setup, &dev);
+    cudaError_t err = set_smem_spread(kern, setup, &dev);
     if (err == cudaSuccess) err = resident_grid(kern, Sh::WPB * 32, Sh::SMEM, setup, dev, &resident);
     if (err != cudaSuccess) return err;
     const long long tiles_per_outer = (a.inner + Sh::BW - 1) / Sh::BW;
     const long long ntiles = a.outer * tiles_per_outer;
     if (ntiles <= 0) return cudaSuccess;
     const long long grid = ntiles < resident ? ntiles : resident;
-    return launch_overlapped(kern, (unsigned)grid, Sh::WPB * 32, Sh::SMEM, s, map, a, tiles_per_outer, ntiles);
+    return launch_spread(kern, grid, Sh::WPB * 32, Sh::SMEM, setup, dev, s, map, a, tiles_per_outer, ntiles);
 }
 
 // SMs of the current device (cached per device).

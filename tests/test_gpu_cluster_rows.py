@@ -1,5 +1,5 @@
-"""FP32 strided passes of 2048 and 4096 points whose columns come in whole 32-byte
-sectors run in clusters that exchange the rows through distributed shared memory
+"""FP32 strided passes of 4096 points whose columns come in whole 32-byte sectors run
+in clusters that exchange the rows through distributed shared memory
 (axis_pass_cluster_rows_kernel). The lines and their arithmetic are those of the
 persistent CTA kernel, which a field that starts 16 bytes into a sector, or a
 stride that is not a multiple of 8, still takes: same bits."""
@@ -13,7 +13,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [(8, 4096), (24, 2048), (1224, 4096), (16, 2048, 3)], ids=str)
+@pytest.mark.parametrize("n", [(8, 4096), (24, 2048), (1224, 4096), (16, 4096, 3)], ids=str)
 @pytest.mark.parametrize("jq", [(0, 0), (1, 2)], ids=str)
 def test_same_bits_as_the_cta_kernel(n, jq):
     prob = I.Problem(n=n, alpha=(1.4, 1.6, 1.5)[: len(n)], eps=0.06, tau=1e-3)
