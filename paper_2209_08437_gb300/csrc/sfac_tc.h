@@ -29,6 +29,13 @@ constexpr int kTcMinN = 17, kTcMaxN = 256;
 // FP64 lines above kTcMaxN take clusters of CTAs (sfac_tc_long.cu).
 constexpr int kTcLongMaxN = 1024;
 
+// Whether the passes may load the eight values from index i of a field of `total`
+// values as whole aligned groups of four (32-byte sectors of FP64, 16 bytes of
+// FP32). Where the values start inside a group, three groups hold them: up to
+// three values before and three after are read too, which at the field's ends
+// are somebody else's memory.
+__host__ __device__ constexpr bool tc_groups_inside(long long i, long long total) { return i >= 3 && i + 11 <= total; }
+
 // Device bytes of the digit image of an axis of n points, and of the scratch
 // the builder needs.
 size_t tc_image_bytes(int n, int slices);

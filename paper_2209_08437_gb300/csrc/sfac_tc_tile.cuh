@@ -272,8 +272,8 @@ __device__ __forceinline__ void st_sector(double* p, double a, double b, double 
 // Eight consecutive values at any 8-byte aligned p: the aligned sectors around
 // them, then a shift. Narrower loads, each lane in sectors of its own, come back to a
 // sector that has left the small L1 beside the tile (16-byte loads: a contiguous
-// pass of 256^3 took 227 us, a strided one 208). `inside`: the sector that holds
-// p[7] may reach past it.
+// pass of 256^3 took 227 us, a strided one 208). `inside`: the sectors around the
+// values lie in the field (tc_groups_inside).
 __device__ __forceinline__ void tc_load8(const double* p, bool inside, double (&v)[8]) {
     const unsigned s = (unsigned)(reinterpret_cast<uintptr_t>(p) >> 3) & 3u;
     if (s == 0) {
@@ -466,11 +466,11 @@ __device__ __forceinline__ bool tc_tiles(const TcPass& g, unsigned char* smem, u
         const double* p = g.src + (STRIDED ? tc_line_base(L, g.inner, n) : L * n);
         if (!STRIDED && 8 * c + 8 <= rows) {
             double v[8];
-            tc_load8(p + 8 * c, true, v);
+            tc_load8(p + 8 * c, tc_groups_inside(L * n + 8 * c, g.lines * n), v);
 #pragma unroll
             for (int r = 0; r < 8; ++r) x[it][r] = v[r];
             if constexpr (PARTS == 2) {
-                tc_load8(p + n - 8 - 8 * c, c > 0 || L + 1 < g.lines, v);
+                tc_load8(p + n - 8 - 8 * c, tc_groups_inside(L * n + n - 8 - 8 * c, g.lines * n), v);
 #pragma unroll
                 for (int r = 0; r < 8; ++r) x[it][8 + r] = v[7 - r];
             }

@@ -116,12 +116,11 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
             const long long stride = STRIDED ? g.inner : 1;
             if (!STRIDED && 8 * c + 8 <= rows) {
                 float v[8];
-                tc_load8(p + 8 * c, true, v);
+                tc_load8(p + 8 * c, tc_groups_inside(L * n + 8 * c, g.lines * n), v);
 #pragma unroll
                 for (int r = 0; r < 8; ++r) x[it][r] = v[r];
                 if constexpr (PARTS == 2) {
-                    // (the 16 bytes around the line's last value may reach two values further)
-                    tc_load8(p + n - 8 - 8 * c, c > 0 || L + 1 < g.lines, v);
+                    tc_load8(p + n - 8 - 8 * c, tc_groups_inside(L * n + n - 8 - 8 * c, g.lines * n), v);
 #pragma unroll
                     for (int r = 0; r < 8; ++r) x[it][8 + r] = v[7 - r];
                 }

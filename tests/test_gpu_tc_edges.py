@@ -1,0 +1,36 @@
+"""Tensor-core passes at the ends of the field and of the number range."""
+import numpy as np
+import pytest
+
+import paper_2209_08437_gb300 as S
+import sfac_inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,prec", [((33, 1218), S.SFAC_FP64), ((17, 1242), S.SFAC_FP64), ((64, 1300), S.SFAC_FP64),
+                                    ((129, 1300), S.SFAC_FP64), ((256, 1218), S.SFAC_FP64), ((65, 70), S.SFAC_FP32),
+                                    ((73, 131), S.SFAC_FP32), ((129, 70), S.SFAC_FP32)], ids=str)
+@pytest.mark.parametrize("start", [0, 16], ids=["aligned", "mid-sector"])
+def test_field_ends_and_mid_sector_starts(n, prec, start):
+    """The first and the last lines of a field that begins at a sector or 16 bytes
+    into one, with lengths whose last values leave a part of a sector: the bits
+    of each line in the middle of a field, and nothing outside is written."""
+    dt = torch.float64 if prec == S.SFAC_FP64 else torch.float32
+    w, pts = dt.itemsize, n[0] * n[1]
+    prob = I.Problem(n=n, alpha=(1.4, 1.6), eps=0.08, tau=0.01)
+    u0 = torch.tensor(I.random_field(prob, 83), dtype=dt, device="cuda")
+    roll = n[1] // 2
+    with S.Plan.for_problem(prob, prec) as plan:
+        want = torch.roll(u0, roll, 0).contiguous()      # the ends' lines, in the middle
+        plan.axis_pass(want, 0, 1, 0)
+        flat = torch.full((pts + 64 // w,), 7.0, dtype=dt, device="cuda")
+        lo = start // w
+        u = flat[lo:lo + pts].view(u0.shape)
+        assert u.data_ptr() % 32 == start
+        u.copy_(u0)
+        plan.axis_pass(u, 0, 1, 0)
+        plan.check()
+    assert torch.equal(u, torch.roll(want, -roll, 0))
+    assert bool((flat[:lo] == 7.0).all()) and bool((flat[lo + pts:] == 7.0).all())
