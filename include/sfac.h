@@ -185,7 +185,9 @@ sfac_status sfac_axis_pass(sfac_plan* plan, void* u_dev, int axis, int jq_in, in
  * spectra of C_l and S_l (zero-padded axes: one linear convolution with B_l's
  * column), or on small grids (sum over all lines of n^2/2 up to 2.4e7) as a
  * direct Toeplitz sum; FP64 arithmetic for both precisions; partial sums are added in a
- * fixed order (deterministic). u_dev is read only. Synchronises `stream`. */
+ * fixed order (deterministic). u_dev is read only. Synchronises `stream`. The
+ * partial sums are the plan's: calls on one plan must not overlap (on several
+ * streams or threads); calls after such ones are not affected. */
 sfac_status sfac_diagnostics(sfac_plan* plan, const void* u_dev, double* out, void* stream);
 
 /* End-to-end variant on HOST memory: advance u_host (plan precision, layout

@@ -206,7 +206,9 @@ __global__ void __launch_bounds__(DIAG_THREADS) diag_direct_kernel(const DiagDir
     if (tid == 0) {
         g.partial[blockIdx.x] = make_double3(red[0][0], red[1][0], red[2][0]);
         __threadfence();
-        last = atomicAdd(g.counter, 1u) == gridDim.x - 1;
+        // the counter wraps to 0 with the last arrival: whatever calls on one plan
+        // overlapped, it is 0 again once they have finished
+        last = atomicInc(g.counter, gridDim.x - 1) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
@@ -223,7 +225,6 @@ __global__ void __launch_bounds__(DIAG_THREADS) diag_direct_kernel(const DiagDir
         g.out[0] = red[0][0];
         g.out[1] = red[1][0];
         g.out[2] = red[2][0];
-        *g.counter = 0;
     }
 }
 

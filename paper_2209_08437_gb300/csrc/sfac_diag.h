@@ -31,7 +31,7 @@ struct DiagDirect {
     long long inner[3], lines[3];
     const double* b[3];     // first column of B_axis
     double3* partial;       // one entry per line of all axes
-    unsigned int* counter;  // 0 before and after
+    unsigned int* counter;  // arrivals, modulo the CTAs of a launch: 0 before and after
     double* out;            // out[0..2] as launch_diag_axis
 };
 // Most multiply-adds (sum over lines of n^2 / 2) of a grid that takes this route.
