@@ -183,7 +183,7 @@ sfac_status sfac_axis_pass(sfac_plan* plan, void* u_dev, int axis, int jq_in, in
  * - (1/2) u^T A u ), h^d the product of the axes' h, A u = sum_l B_l along axis l.
  * u^T A u is accumulated line by line as x . B_l x with B_l x formed through the
  * spectra of C_l and S_l (zero-padded axes: one linear convolution with B_l's
- * column), or on small grids (sum over all lines of n^2/2 up to 2.4e7) as a
+ * column), or on grids with few short lines, where that is no slower, as a
  * direct Toeplitz sum; FP64 arithmetic for both precisions; partial sums are added in a
  * fixed order (deterministic). u_dev is read only. Synchronises `stream`. The
  * partial sums are the plan's: calls on one plan must not overlap (on several

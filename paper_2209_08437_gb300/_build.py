@@ -24,7 +24,7 @@ SOURCES = ["sfac_plan.cu", "sfac_host.cu", "sfac_pass_f64.cu", "sfac_pass_f32.cu
            "sfac_tc_build.cu", "sfac_tc_pass.cu", "sfac_tc_pass_f32.cu",
            "sfac_tc_steps.cu", "sfac_tc_long.cu"]
 HEADERS = ["sfac_fft.cuh", "sfac_pass.cuh", "sfac_internal.h", "sfac_host.h", "sfac_batch.cuh",
-           "sfac_batch_launch.h", "sfac_diag.h", "sfac_tma.cuh", "sfac_steps.h",
+           "sfac_batch_launch.h", "sfac_diag.h", "sfac_diag_rule.h", "sfac_tma.cuh", "sfac_steps.h",
            "sfac_tc.h", "sfac_tcgen05.cuh", "sfac_jq_fixed.cuh", "sfac_tc_tile.cuh", "sfac_tc_tile_f32.cuh", "sfac_tc_launch.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -140,9 +140,9 @@ diag_reduce_kernel(const double3* __restrict__ partial, long long n, double* __r
 // Small grids. The FFT passes above are latency bound there (2D 127^2: about 35 us
 // an axis for 64 line pairs, four launches, whatever the arithmetic): n^2 / 2
 // multiply-adds a line, spread over a CTA, take less up to a few hundred points.
-// Side by side on one GB300: a 127^2 FP64 step with diagnostics 101 -> 57 us. The
-// FP64 pipes do 304 multiply-adds a clock, so kDiagDirectMost of them take 42 us,
-// where the FFT passes are no slower.
+// Side by side on one GB300: a 127^2 FP64 step with diagnostics 101 -> 57 us. A
+// line stays on one SM (n = 1024: 190 us), so few long lines lose to the FFTs, and
+// so do many short ones (1/140 us a CTA): diag_direct_pays draws the line.
 template <typename Rin>
 __global__ void __launch_bounds__(DIAG_THREADS) diag_direct_kernel(const DiagDirect g) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -284,7 +284,7 @@ cudaError_t launch_diag_direct(bool f64_field, const DiagDirect& d, cudaStream_t
         blocks += d.lines[ax];
         nmax = d.n[ax] > nmax ? d.n[ax] : nmax;
     }
-    const size_t smem = 2 * sizeof(double) * (size_t)nmax;  // n <= 2048: 32 KB
+    const size_t smem = 2 * sizeof(double) * (size_t)nmax;  // n <= 1024: 16 KB
     if (f64_field) diag_direct_kernel<double><<<(unsigned)blocks, DIAG_THREADS, smem, s>>>(d);
     else diag_direct_kernel<float><<<(unsigned)blocks, DIAG_THREADS, smem, s>>>(d);
     return cudaGetLastError();

@@ -34,8 +34,7 @@ struct DiagDirect {
     unsigned int* counter;  // arrivals, modulo the CTAs of a launch: 0 before and after
     double* out;            // out[0..2] as launch_diag_axis
 };
-// Most multiply-adds (sum over lines of n^2 / 2) of a grid that takes this route.
-constexpr double kDiagDirectMost = 2.4e7;
+// (for grids that diag_direct_pays admits: lines of at most 1024 points)
 cudaError_t launch_diag_direct(bool f64_field, const DiagDirect& d, cudaStream_t s);
 
 }  // namespace sfac

@@ -13,6 +13,7 @@
 
 #include "sfac.h"
 #include "sfac_diag.h"
+#include "sfac_diag_rule.h"
 #include "sfac_host.h"
 #include "sfac_internal.h"
 #include "sfac_steps.h"
@@ -411,8 +412,6 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     const size_t rs = real_size(P);
     size_t off[3][11], total = 0;
     long long max_partials = 1, direct_lines = 0;
-    double direct_work = 0.0;
-    int direct_n = 0;
     {
         long long inner = 1;
         for (int l = 0; l < params->dim; ++l) {
@@ -429,12 +428,12 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
             const long long clines = l == 0 ? (outer + 1) / 2 : outer * ((inner + 1) / 2);
             max_partials = std::max(max_partials, sfac::diag_partials_needed(clines, (int)n));
             direct_lines += outer * inner;
-            direct_work += 0.5 * (double)(outer * inner) * params->n[l] * params->n[l];
-            direct_n = std::max(direct_n, params->n[l]);
             inner *= params->n[l];
         }
     }
-    P->diag_direct = direct_work <= sfac::kDiagDirectMost && direct_n <= 2048;
+    int fft_len[3];
+    for (int l = 0; l < params->dim; ++l) fft_len[l] = padded[l] ? pad[l].L : params->n[l];
+    P->diag_direct = sfac::diag_direct_pays(params->dim, params->n, fft_len, padded);
     if (P->diag_direct) max_partials = std::max(max_partials, direct_lines);
     const size_t off_partial = total;
     total += align256(sizeof(double3) * (size_t)max_partials);
@@ -536,7 +535,7 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
         P->ax[l].twid = base + off[l][3];
         P->ax[l].rtwid = rtw[l].empty() ? nullptr : base + off[l][8];
         P->ax[l].padded = padded[l];
-        P->ax[l].fft_len = padded[l] ? pad[l].L : params->n[l];
+        P->ax[l].fft_len = fft_len[l];
         P->ax[l].dA = reinterpret_cast<const double*>(base + off[l][4]);
         P->ax[l].dB = padded[l] ? nullptr : reinterpret_cast<const double*>(base + off[l][5]);
         P->ax[l].dtwist = padded[l] ? nullptr : base + off[l][6];
