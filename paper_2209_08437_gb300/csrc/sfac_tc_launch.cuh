@@ -41,7 +41,7 @@ tc_pass_kernel(const TcArgs<R> g) {
         st.parity = 1;
         st.left = (g.pass.ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x * stages;
         tc_produce<Sh::STAGES, Sh::G>(sh, st, ring, g.img, stages, Sh::OWN_PRODUCER ? st.left : Sh::STAGES,
-                                      g.wait_cycles);
+                                      g.wait_cycles, Sh::STAGES);
     }
     if (warp < NT / 32) {
         pass_wait_for_previous();

@@ -93,9 +93,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
         st.parity = 1;
         st.left = nkc * 2 * kTcSlices / kG;
         const unsigned char* img = g.img + (size_t)rank * nkc * 2 * kTcSlices * kTcBlock;
-        tc_produce<kStages, kG>(sh, st, smem + kRing, img, nkc * 2 * kTcSlices / kG, st.left, limit);
+        tc_produce<kStages, kG>(sh, st, smem + kRing, img, nkc * 2 * kTcSlices / kG, st.left, limit,
+                                kStages);
     } else if (warp == kNT / 32 + 1) {
         // ---- the products ----
+        pass_wait_for_previous();  // no limit runs before the lines can be loaded (tc_produce)
         if (g.hold) alive = tc_wait(&sh.never, 0, limit, &sh.abort);  // the test hook
         const uint64_t a0 = tc_desc(smem_u32(smem + kRing), 2048, 128), b0 = tc_desc(smem_u32(smem), Shape::LBO, 128);
 #pragma unroll 1

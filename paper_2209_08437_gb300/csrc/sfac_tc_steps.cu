@@ -241,12 +241,15 @@ __global__ void __launch_bounds__(kNT + 32, 1) tc_steps_kernel(const TcStepsArgs
     bool alive = true;
     if (warp == kNT / 32) {
         st.parity = 1;
+        long long early = g.single ? kStages : -1;
         for (long long s = 0; alive && s < g.nsteps; ++s)
             for (int ax = 0; alive && ax < g.dim; ++ax) {
                 const int stages = g.parts[ax] * (g.ax[ax].kp >> 5) * kTcSlices / kG;
                 for (long long tile = blockIdx.x; alive && tile < g.ax[ax].ntiles; tile += gridDim.x) {
                     st.left = stages;
-                    alive = tc_produce<kStages, kG>(sh, st, smem + kRing, g.img[ax], stages, stages, g.wait_cycles);
+                    alive = tc_produce<kStages, kG>(sh, st, smem + kRing, g.img[ax], stages, stages, g.wait_cycles,
+                                                    early);
+                    early -= stages;
                 }
             }
     } else {

@@ -337,14 +337,18 @@ __device__ __forceinline__ void tc_prefetch(const TcPassT<R>& g, long long tile,
 }
 
 // The producer: up to `count` more stages of an image of `stages` of them (st.left
-// counts stages too).
+// counts stages too). Before stage number `early` of these it waits for the
+// previous pass: the first ring needs no room, but the room for more comes only
+// once the lines are loaded, and the limit of that wait must not run while the
+// previous pass does (a 4096 x 200 step under a limit of 100 us gave up).
 template <int STAGES, int G>
 __device__ __forceinline__ bool tc_produce(TcShared& sh, TcState& st, unsigned char* ring, const unsigned char* img,
-                                           int stages, long long count, long long limit) {
+                                           int stages, long long count, long long limit, long long early = -1) {
     constexpr unsigned BYTES = G * kTcBlock;
     if (count > st.left) count = st.left;
 #pragma unroll 1
     for (long long c = 0; c < count; ++c) {
+        if (c == early) pass_wait_for_previous();
         if (!tc_wait<true>(&sh.empty[st.stage], st.parity, limit, &sh.abort)) return false;
         if (elect_one()) {
             mbar_expect_tx(&sh.full[st.stage], BYTES);

@@ -34,3 +34,22 @@ def test_field_ends_and_mid_sector_starts(n, prec, start):
         plan.check()
     assert torch.equal(u, torch.roll(want, -roll, 0))
     assert bool((flat[:lo] == 7.0).all()) and bool((flat[lo + pts:] == 7.0).all())
+
+
+@pytest.mark.parametrize("n,limit", [((4096, 200), 200_000), ((4096, 300), 300_000), ((4096, 100), 200_000)], ids=str)
+def test_limits_do_not_run_during_the_previous_pass(n, limit):
+    """A pass may start while the previous one runs (here FP64 FFTs of 4096 points,
+    one wave of CTAs of several 100 us that leaves SMs free). The limit of its own
+    waits, shorter than that but far above what they take, must not count the
+    previous pass: nothing gave up, and the bits are those of the default limit."""
+    prob = I.Problem(n=n, alpha=(1.4, 1.6), eps=0.05, tau=1e-3)
+    u0 = torch.tensor(I.random_field(prob, 84), device="cuda")
+    with S.Plan.for_problem(prob) as plan:
+        want = u0.clone()
+        plan.step(want, 3)
+        plan.check()
+        S.sfac_plan_set_wait_limit(plan.handle, limit, 0)
+        got = u0.clone()
+        plan.step(got, 3)
+        plan.check()
+    assert torch.equal(got, want)
