@@ -148,7 +148,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
     // columns (128 bytes) of 8 lines. A unit: 4 columns and their mirror images.
     const int line = STRIDED ? lane : (warp & 3) * 8 + (lane & 7);
     const int cg = STRIDED ? warp : (warp >> 2) * 4 + (lane >> 3);
-    const int Emin = max(1, 64 - ps.scale);
     long long sum[2][16];  // row (warp & 3) * 32 + lane, lines (warp >> 2) * 16 ..
     if (warp < kNT / 32) {
         pass_wait_for_previous();
@@ -186,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
         }
         atomicMax(&smax[line], m);
         tc_sync<kNT>();
-        const int E = max((int)(smax[line] >> 20), Emin) + ps.headroom;
+        const int E = tc_scale_of((int)(smax[line] >> 20), ps.headroom);
 #pragma unroll
         for (int q = 0; q < 16; ++q) sum[0][q] = sum[1][q] = 0;
         double v[8];
@@ -273,6 +272,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
                 *l = STRIDED ? u % kLT : u / 128;
                 return (int)rank * 128 + *rr < rows ? sbase[*l] : -1;
             };
+            auto cell = [&](int i) {  // value i: B values, then their mirror images
+                int rr, l;
+                where(i % B, &rr, &l);
+                return reinterpret_cast<double*>(smem + kRing + (i / B * 128 + rr) * kPitch + l * 8);
+            };
 #pragma unroll
             for (int i = 0; i < B; ++i) {
                 int rr, l;
@@ -285,17 +289,20 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
             for (int i = 0; i < B; ++i) {
                 int rr, l;
                 where(i, &rr, &l);
-                const int Eb = (int)(smax[l] >> 20);
-                const int E = max(Eb, Emin) + ps.headroom;
+                const int E = tc_scale_of((int)(smax[l] >> 20), ps.headroom);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     double& w = v[h * B + i];
-                    const long long d =
-                        *reinterpret_cast<const long long*>(smem + kRing + (h * 128 + rr) * kPitch + l * 8);
-                    w = tc_to_double(tc_fixed(w, E) + tc_align(d, ps.scale), E);
-                    if (Eb == 2047) w = __longlong_as_double(0x7ff8000000000000LL);
+                    const long long d = __double_as_longlong(*cell(h * B + i));
+                    w = __longlong_as_double(tc_fixed(w, E) + tc_align(d, ps.scale));
                 }
             }
+            auto field = [&](int r) {
+                int rr, l;
+                where(r % B, &rr, &l);
+                return (int)(smax[l] >> 20);
+            };
+            tc_to_doubles(v, ps.headroom, field, cell);
             if (ps.jq_out) jq_flow_fixed_all(v, ps.jout);
 #pragma unroll
             for (int i = 0; i < B; ++i) {

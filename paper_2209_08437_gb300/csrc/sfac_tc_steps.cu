@@ -119,11 +119,10 @@ __device__ __forceinline__ bool tc_small_tile(const TcPass& g, long long tile, u
     }
     tc_sync<kNT>();
     // ---- digits ----
-    const int Emin = max(1, 64 - g.scale);
 #pragma unroll 1
     for (int u = tid; u < units; u += kNT) {
         const int line = u & 7, k = u >> 3 << 1;
-        const int E = max((int)(smax[line] >> 20), Emin) + g.headroom;
+        const int E = tc_scale_of((int)(smax[line] >> 20), g.headroom);
         constexpr int SB = PARTS == 2 ? 7 : 6;
         constexpr unsigned long long bias = (kTcBias << SB) + (1ULL << (SB - 1));
         const double2 v = xs[u];
@@ -201,7 +200,6 @@ __device__ __forceinline__ bool tc_small_tile(const TcPass& g, long long tile, u
         const long long b = base[line];
         if (b < 0) continue;
         const int Eb = (int)(smax[line] >> 20);
-        const int E = max(Eb, Emin) + g.headroom;
         const double2 a = xs[u];
         double v[V] = {a.x, a.y};
         if constexpr (PARTS == 2) {
@@ -209,13 +207,13 @@ __device__ __forceinline__ bool tc_small_tile(const TcPass& g, long long tile, u
             v[2] = w.x;
             v[3] = w.y;
         }
+        auto cell = [&](int r) {
+            return reinterpret_cast<double*>(smem + (r >> 1) * part_bytes + (k + (r & 1)) * PITCH + line * 8);
+        };
 #pragma unroll
-        for (int r = 0; r < V; ++r) {
-            const long long d = *reinterpret_cast<const long long*>(smem + (r >> 1) * part_bytes +
-                                                                    (k + (r & 1)) * PITCH + line * 8);
-            v[r] = tc_to_double(__double_as_longlong(v[r]) + tc_align(d, g.scale), E);
-            if (Eb == 2047) v[r] = __longlong_as_double(0x7ff8000000000000LL);
-        }
+        for (int r = 0; r < V; ++r)
+            v[r] = __longlong_as_double(__double_as_longlong(v[r]) + tc_align(__double_as_longlong(*cell(r)), g.scale));
+        tc_to_doubles(v, g.headroom, [=](int) { return Eb; }, cell);
         if (g.jq_out) jq_flow_fixed_all(v, g.jout);
         double* p = g.dst + b;
 #pragma unroll

@@ -199,15 +199,64 @@ __device__ __forceinline__ long long tc_fixed(double v, int E) {
     return hi < 0 ? -f : f;
 }
 
-// Back to FP64, rounded to nearest (ties away). E >= 64: the result is normal.
+// Exponent field of a line's scale, from its largest value's field Eb (0: zero or
+// subnormal values).
+__device__ __forceinline__ int tc_scale_of(int Eb, int headroom) { return max(Eb, 1) + headroom; }
+// Whether every result of the line is zero or a normal number.
+__device__ __forceinline__ bool tc_plain(int Eb) { return (unsigned)(Eb - 61) <= 2041u - 61u; }
+
+// Back to FP64, rounded to nearest (ties away), in a plain line: |y| < 2^63.
 __device__ __forceinline__ double tc_to_double(long long y, int E) {
     if (y == 0) return 0.0;
     const unsigned long long m = y < 0 ? 0ULL - (unsigned long long)y : (unsigned long long)y;
     const int lz = __clzll((long long)m);
     const unsigned long long t = (((m << lz) >> 10) + 1) >> 1;  // 2^52 .. 2^53
     const int e = E + 3 - lz;                                   // exponent field less one
-    const long long bits = e >= 2046 ? 0x7ff0000000000000LL : (long long)t + ((long long)e << 52);
+    const long long bits = (long long)t + ((long long)e << 52);
     return __longlong_as_double(bits | (y & (long long)0x8000000000000000ULL));
+}
+// The same in any line: subnormal results, infinities, and NaN throughout a line
+// that holds an infinity or a NaN (Eb = 2047).
+__device__ __forceinline__ double tc_to_double_any(long long y, int E, int Eb) {
+    if (Eb == 2047) return __longlong_as_double(0x7ff8000000000000LL);
+    if (y == 0) return 0.0;
+    const unsigned long long m = y < 0 ? 0ULL - (unsigned long long)y : (unsigned long long)y;
+    const int lz = __clzll((long long)m);
+    const int e = E + 3 - lz;
+    long long bits;
+    if (e >= 2046)
+        bits = 0x7ff0000000000000LL;
+    else if (e >= 0)
+        bits = (long long)((((m << lz) >> 10) + 1) >> 1) + ((long long)e << 52);
+    else  // in units of 2^-1074; y is in units of 2^(E - 1082)
+        bits = (long long)(E >= 8 ? m << (E - 8) : (m + (1ULL << (7 - E))) >> (8 - E));
+    return __longlong_as_double(bits | (y & (long long)0x8000000000000000ULL));
+}
+
+// V sums (as bits) back to FP64; Eb(r): the largest field of value r's line,
+// cell(r): a shared-memory word that is this thread's own. The rare lines go through
+// one rolled loop in shared memory (a 3D 63^3 step 138.0 -> 139.6 us): unrolled
+// beside the plain code, or with the values picked out of registers, they took
+// 141 us, as the code of a pass of one round is fetched for one use.
+template <int V, typename F, typename C>
+__device__ __forceinline__ void tc_to_doubles(double (&x)[V], int headroom, F Eb, C cell) {
+    bool plain = true;
+#pragma unroll
+    for (int r = 0; r < V; ++r) plain = plain && tc_plain(Eb(r));
+    if (__builtin_expect(plain, 1)) {
+#pragma unroll
+        for (int r = 0; r < V; ++r) x[r] = tc_to_double(__double_as_longlong(x[r]), tc_scale_of(Eb(r), headroom));
+    } else {
+#pragma unroll
+        for (int r = 0; r < V; ++r) *cell(r) = x[r];
+#pragma unroll 1
+        for (int r = 0; r < V; ++r) {
+            double* p = cell(r);
+            *p = tc_to_double_any(__double_as_longlong(*p), tc_scale_of(Eb(r), headroom), Eb(r));
+        }
+#pragma unroll
+        for (int r = 0; r < V; ++r) x[r] = *cell(r);
+    }
 }
 
 // Digit place q (0: most significant) of two biased values whose lowest digit is at
@@ -454,7 +503,6 @@ __device__ __forceinline__ bool tc_tiles(const TcPass& g, unsigned char* smem, u
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int n = g.n, rows = g.rows, kp = g.kp, nch = kp >> 3;
     const int part_bytes = Sh::part_bytes(kp);
-    const int Emin = max(1, 64 - g.scale);
 
     // Units (line, chunk c of 8 columns, and their mirror images). Strided axis:
     // lanes along the lines; contiguous axis: a warp takes 4 chunks (256 bytes) of
@@ -532,7 +580,7 @@ __device__ __forceinline__ bool tc_tiles(const TcPass& g, unsigned char* smem, u
         const bool issues = warp < 2;
 #pragma unroll
         for (int it = 0; it < UPT; ++it) {
-            const int E = max((int)(smax[max(uline[it], 0)] >> 20), Emin) + g.headroom;
+            const int E = tc_scale_of((int)(smax[max(uline[it], 0)] >> 20), g.headroom);
 #pragma unroll
             for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(tc_fixed(x[it][r], E));
             digits(it, 0);
@@ -634,17 +682,16 @@ __device__ __forceinline__ bool tc_tiles(const TcPass& g, unsigned char* smem, u
             const long long L = tile * LT + line;
             if (line >= 0 && L < g.lines) {
                 const int Eb = (int)(smax[line] >> 20);
-                const int E = max(Eb, Emin) + g.headroom;
+                auto cell = [&](int r) {
+                    return reinterpret_cast<double*>(smem + (8 * c + (r & 7)) * Sh::PITCH + line * 8 +
+                                                     (r >> 3) * part_bytes);
+                };
 #pragma unroll
                 for (int r = 0; r < VPU; ++r) {
-                    const int off = (8 * c + (r & 7)) * Sh::PITCH + line * 8 + (r >> 3) * part_bytes;
-                    const long long v = *reinterpret_cast<const long long*>(smem + off);
-                    x[it][r] = tc_to_double(__double_as_longlong(x[it][r]) + tc_align(v, g.scale), E);
+                    const long long v = __double_as_longlong(*cell(r));
+                    x[it][r] = __longlong_as_double(__double_as_longlong(x[it][r]) + tc_align(v, g.scale));
                 }
-                if (Eb == 2047) {  // a line that holds an infinity or a NaN
-#pragma unroll
-                    for (int r = 0; r < VPU; ++r) x[it][r] = __longlong_as_double(0x7ff8000000000000LL);
-                }
+                tc_to_doubles(x[it], g.headroom, [=](int) { return Eb; }, cell);
                 if (g.jq_out) jq_flow_fixed_all(x[it], g.jout);
                 double* p = g.dst + (STRIDED ? tc_line_base(L, g.inner, n) : L * n);
                 if (!STRIDED && 8 * c + 8 <= rows) {

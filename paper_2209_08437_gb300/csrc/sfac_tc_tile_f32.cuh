@@ -147,16 +147,21 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
     }
     tc_sync<NT>();
     // ---- digits: x in units of 2^(E - 154) (parts) or 2^(E - 155), sums below 2^29 ----
-    constexpr int Emin = 28;
+    constexpr int Emin = 28;  // below, the factor has no exponent left: two factors
 #pragma unroll
     for (int it = 0; it < UPT; ++it) {
         if (uline[it] < 0) continue;
-        const int E = max((int)(smax[uline[it]] >> 23), Emin);
-        const float m = __uint_as_float((unsigned)((PARTS == 2 ? 281 : 282) - E) << 23);
+        const int E = max((int)(smax[uline[it]] >> 23), 1);
+        const float m = __uint_as_float((unsigned)((PARTS == 2 ? 281 : 282) - max(E, Emin)) << 23);
         unsigned char* chunk = smem + uc[it] * LBO;
         int X[VPU];
 #pragma unroll
         for (int r = 0; r < VPU; ++r) X[r] = __float2int_rn(fmaf(x[it][r], m, d[it][r] * m));
+        if (__builtin_expect(E < Emin, 0)) {
+            const float up = (float)(1 << (Emin - E));
+#pragma unroll
+            for (int r = 0; r < VPU; ++r) X[r] = __float2int_rn(fmaf(x[it][r], m, d[it][r] * m) * up);
+        }
         unsigned F[8];
         if constexpr (PARTS == 2) {
 #pragma unroll
@@ -233,9 +238,10 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
         const long long L = tile * LT + line;
         if (line < 0 || L >= g.lines) continue;
         const int Eb = (int)(smax[line] >> 23);
-        // the sums are in units of 2^(E - 145); NaN for a line that holds an infinity or a NaN
-        const float sc = Eb == 255 ? __uint_as_float(0x7fc00000u)
-                                   : __uint_as_float((unsigned)(max(Eb, Emin) - 18) << 23);
+        // the sums are in units of 2^(E - 145), a subnormal for E < 19; NaN for a line
+        // that holds an infinity or a NaN
+        const int E = max(Eb, 1);
+        const float sc = __uint_as_float(Eb == 255 ? 0x7fc00000u : E > 18 ? (unsigned)(E - 18) << 23 : 16u << E);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
             const int off = (8 * c + r) * Sh::PITCH + line * 4;
