@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_long_kernel(const TcLongArgs g
     const long long limit = g.wait_cycles, inner = ps.inner;
     if (tid < kLT) {
         const long long L = tile * kLT + tid;
-        smax[tid] = 0;
+        smax[tid] = L >= ps.lines ? 1023u << 20 : 0;  // a missing line is not a rare one (tc_plain)
         sbase[tid] = L >= ps.lines ? -1 : STRIDED ? L / inner * n * inner + L % inner : L * n;
     }
     if (tid == 0) {

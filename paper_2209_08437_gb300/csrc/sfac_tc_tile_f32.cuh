@@ -147,21 +147,19 @@ __device__ __forceinline__ bool tc_tile_f32(const TcPassT<float>& g, long long t
     }
     tc_sync<NT>();
     // ---- digits: x in units of 2^(E - 154) (parts) or 2^(E - 155), sums below 2^29 ----
-    constexpr int Emin = 28;  // below, the factor has no exponent left: two factors
+    // Below E = 28 the factor has no exponent left: a second one, for every line, which
+    // costs less than a branch (3D 200^3 x 2: 287 us without, 289, with a branch 293).
+    constexpr int Emin = 28;
 #pragma unroll
     for (int it = 0; it < UPT; ++it) {
         if (uline[it] < 0) continue;
         const int E = max((int)(smax[uline[it]] >> 23), 1);
         const float m = __uint_as_float((unsigned)((PARTS == 2 ? 281 : 282) - max(E, Emin)) << 23);
+        const float up = __uint_as_float((unsigned)(127 + max(Emin - E, 0)) << 23);
         unsigned char* chunk = smem + uc[it] * LBO;
         int X[VPU];
 #pragma unroll
-        for (int r = 0; r < VPU; ++r) X[r] = __float2int_rn(fmaf(x[it][r], m, d[it][r] * m));
-        if (__builtin_expect(E < Emin, 0)) {
-            const float up = (float)(1 << (Emin - E));
-#pragma unroll
-            for (int r = 0; r < VPU; ++r) X[r] = __float2int_rn(fmaf(x[it][r], m, d[it][r] * m) * up);
-        }
+        for (int r = 0; r < VPU; ++r) X[r] = __float2int_rn(fmaf(x[it][r], m, d[it][r] * m) * up);
         unsigned F[8];
         if constexpr (PARTS == 2) {
 #pragma unroll
