@@ -84,10 +84,11 @@ typedef struct sfac_plan sfac_plan;
  * 1024 points, and zero-padded FP32 axes of 65 to 256, apply the same factor as
  * a dense operator on the tensor cores (exact sums of fixed-point digit products;
  * the plan keeps the operator's digits, up to 6.3 MB an axis at 1024 points, and
- * an axis whose operator would not keep them exact stays with the FFTs). Other
+ * up to 4.3 MB an axis in which they were built; an axis whose operator would not
+ * keep them exact stays with the FFTs, whose tables are only then computed). Other
  * lengths return SFAC_EUNSUPPORTED. The plan owns its device tables and
  * any staging buffer; free it with sfac_plan_destroy. On success *out is set;
- * on failure *out is NULL. The call synchronises `stream` once (upload). */
+ * on failure *out is NULL. The call synchronises `stream` (uploads). */
 sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan** out);
 
 /* How the plan runs axis `axis` (0-based): *fft_len receives the FFT length of

@@ -95,21 +95,17 @@ int padded_length(int n) {
     return L;
 }
 
-void increment_columns(const AxisHost& T, double tau, std::vector<double>* g, std::vector<double>* h) {
+void increment_columns(const AxisHost& T, std::vector<double>* g, std::vector<double>* h) {
     const int n = T.n;
     std::vector<double> cs(2 * n), sn(2 * n);
     for (int m = 0; m < 2 * n; ++m) sincospi_frac(m, n, &cs[m], &sn[m]);
-    // From expm1 of the spectra:
+    // From the expm1 values of the spectra:
     //   g_d = (1/n) sum_j expm1(t lambda_j) cos(2 pi j d / n),     d = 0 .. n-1
     //   h_d = (1/n) sum_j expm1(tau mu_j) cos(pi d (2j - 1) / n),  d = 0 .. n-1 (h_{-d} = h_d)
     // (the identity's share sum_j cos(...) vanishes for d != 0 mod n).
-    std::vector<double> xc(n), xs(n);
+    const std::vector<double>&xc = T.incC, &xs = T.incS;
     g->resize(n);
     h->resize(n);
-    for (int j = 0; j < n; ++j) {
-        xc[j] = std::expm1(0.5 * tau * T.lambda[j]);
-        xs[j] = std::expm1(tau * T.mu[j]);
-    }
     const int two_n = 2 * n;
     for (int d = 0; d < n; ++d) {
         KahanSum sg, sh;
@@ -129,50 +125,60 @@ void increment_columns(const AxisHost& T, double tau, std::vector<double>* g, st
     }
 }
 
-std::vector<double> increment_spectra(const AxisHost& T, double tau) {
-    const int n = T.n;
-    std::vector<double> out(4 * (size_t)n);
-    for (int j = 0; j < n; ++j) {
-        out[j] = std::expm1(0.5 * tau * T.lambda[j]);
-        out[n + j] = std::expm1(tau * T.mu[j]);
+std::vector<double> increment_spectra(const AxisHost& T) {
+    const size_t n = T.n;
+    std::vector<double> out(4 * n);
+    for (size_t j = 0; j < n; ++j) {
+        out[j] = T.incC[j];
+        out[n + j] = T.incS[j];
+        out[2 * n + j] = T.twist[2 * j];    // cos(pi j / n)
+        out[3 * n + j] = -T.twist[2 * j];
     }
-    double s;
-    for (int m = 0; m < 2 * n; ++m) sincospi_frac(m, n, &out[2 * (size_t)n + m], &s);
     return out;
 }
 
-void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P) {
-    const int n = T.n;
+namespace {
+
+// The DFT (over L, incl. 1/L) of a symmetric column: offset d in (-n, n) at index d
+// mod L. The circulant part repeats its column with period n (c_d = g_{d mod n}).
+// Real, because the column is symmetric.
+void padded_spectrum(int n, int L, const std::vector<double>& col, bool circulant, double diag_add,
+                     std::vector<double>* out) {
+    std::vector<double> re(L, 0.0), im(L, 0.0);
+    for (int d = -(n - 1); d <= n - 1; ++d) {
+        const int src = circulant ? ((d % n) + n) % n : (d < 0 ? -d : d);
+        re[(d % L + L) % L] = col[src];
+    }
+    re[0] += diag_add;
+    fft_pow2(re, im);
+    out->resize(L);
+    for (int k = 0; k < L; ++k) (*out)[k] = re[k] / (double)L;
+}
+
+}  // namespace
+
+void padded_factors(const AxisHost& T, bool increments, std::vector<double>* mC, std::vector<double>* mS) {
+    std::vector<double> g, h;
+    increment_columns(T, &g, &h);
+    const int L = padded_length(T.n);
+    padded_spectrum(T.n, L, g, true, increments ? 0.0 : 1.0, mC);
+    padded_spectrum(T.n, L, h, false, increments ? 0.0 : 1.0, mS);
+}
+
+void padded_operator(const AxisHost& T, std::vector<double>* mB) {
+    padded_spectrum(T.n, padded_length(T.n), T.bcol, false, 0.0, mB);
+}
+
+std::vector<double> padded_twiddles(int n) {
     const int L = padded_length(n);
-    P->n = n;
-    P->L = L;
-    std::vector<double> g1, h1;
-    increment_columns(T, tau, &g1, &h1);
-    // Padded, symmetric columns: offset d in (-n, n) at index d mod L. The
-    // circulant part repeats its column with period n (c_d = g_{d mod n}).
-    auto spectrum = [&](const std::vector<double>& col, bool circulant, double diag_add, std::vector<double>* out) {
-        std::vector<double> re(L, 0.0), im(L, 0.0);
-        for (int d = -(n - 1); d <= n - 1; ++d) {
-            const int src = circulant ? ((d % n) + n) % n : (d < 0 ? -d : d);
-            re[(d % L + L) % L] = col[src];
-        }
-        re[0] += diag_add;
-        fft_pow2(re, im);
-        out->resize(L);
-        for (int k = 0; k < L; ++k) (*out)[k] = re[k] / (double)L;  // real: the column is symmetric
-    };
-    spectrum(T.bcol, false, 0.0, &P->mB);
-    spectrum(g1, true, 1.0, &P->mC);
-    spectrum(h1, false, 1.0, &P->mS);
-    spectrum(g1, true, 0.0, &P->mC1);
-    spectrum(h1, false, 0.0, &P->mS1);
-    P->twid.resize(2 * L);
+    std::vector<double> twid(2 * (size_t)L);
     for (int k = 0; k < L; ++k) {
         double c, s;
         sincospi_frac(2LL * k, L, &c, &s);
-        P->twid[2 * k] = c;
-        P->twid[2 * k + 1] = -s;
+        twid[2 * k] = c;
+        twid[2 * k + 1] = -s;
     }
+    return twid;
 }
 
 bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
@@ -236,13 +242,17 @@ void compute_axis(double alpha, double eps, double tau, double a, double b, int 
     // Factors with the inverse-FFT normalisation 1/n folded in.
     T->eC.resize(n);
     T->eS.resize(n);
+    T->incC.resize(n);
+    T->incS.resize(n);
     T->dC.resize(n);
     T->dS.resize(n);
     for (int j = 0; j < n; ++j) {
         T->eC[j] = std::exp(0.5 * tau * T->lambda[j]) / (double)n;
         T->eS[j] = std::exp(tau * T->mu[j]) / (double)n;
-        T->dC[j] = std::expm1(0.5 * tau * T->lambda[j]) / (double)n;
-        T->dS[j] = std::expm1(tau * T->mu[j]) / (double)n;
+        T->incC[j] = std::expm1(0.5 * tau * T->lambda[j]);
+        T->incS[j] = std::expm1(tau * T->mu[j]);
+        T->dC[j] = T->incC[j] / (double)n;
+        T->dS[j] = T->incS[j] / (double)n;
     }
     // Twist e^{i pi k/n} and FFT twiddles e^{-2 pi i m/n}.
     T->twist.resize(2 * n);

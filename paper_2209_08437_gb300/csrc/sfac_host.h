@@ -10,19 +10,8 @@ struct AxisHost {
     int n = 0;
     std::vector<double> bcol, cfirst, sfirst, lambda, mu;
     std::vector<double> eC, eS, twist, twid;  // twist, twid: interleaved complex
-    std::vector<double> dC, dS;               // expm1 forms for the FP32 increment passes
-};
-
-// Zero-padded form of one axis, for any n: e^{t C} and e^{tau S} are symmetric
-// Toeplitz matrices, so each is a linear convolution of the line with its
-// first column; padded to a power of two L >= 2n - 1 the convolution is
-// circular and its multiplier (the DFT of the symmetric padded column) is real.
-struct AxisPadded {
-    int n = 0, L = 0;
-    std::vector<double> mC, mS;    // L real multipliers incl. 1/L: e^{tau/2 C}, e^{tau S}
-    std::vector<double> mC1, mS1;  // the same for (e^{tX} - I): increment forms
-    std::vector<double> mB;        // L real multipliers incl. 1/L of B itself (diagnostics)
-    std::vector<double> twid;      // L complex e^{-2 pi i m / L}, interleaved
+    std::vector<double> incC, incS;           // e^{tau/2 lambda} - 1, e^{tau mu} - 1
+    std::vector<double> dC, dS;               // the same over n, for the FP32 increment passes
 };
 
 bool is_pow2(int v);
@@ -32,14 +21,24 @@ int padded_length(int n);
 
 // First columns of e^{tau/2 C} - I and e^{tau S} - I (both symmetric Toeplitz, n
 // values each) of the axis in T.
-void increment_columns(const AxisHost& T, double tau, std::vector<double>* g, std::vector<double>* h);
+void increment_columns(const AxisHost& T, std::vector<double>* g, std::vector<double>* h);
 
 // The n expm1 values of each spectrum (e^{tau/2 C} - I, then e^{tau S} - I) and
 // cos(pi m / n) for m = 0 .. 2n - 1, from which the columns are summed.
-std::vector<double> increment_spectra(const AxisHost& T, double tau);
+std::vector<double> increment_spectra(const AxisHost& T);
 
-// Padded tables of one axis (needs the spectra of compute_axis in T).
-void compute_axis_padded(const AxisHost& T, double tau, AxisPadded* P);
+// Zero-padded form of one axis, for any n (needs the spectra of compute_axis in T):
+// e^{t C} and e^{tau S} are symmetric Toeplitz matrices, so each is a linear
+// convolution of the line with its first column; padded to a power of two L >= 2n - 1
+// (padded_length) the convolution is circular and its multiplier (the DFT of the
+// symmetric padded column) is real.
+// mC, mS: L real multipliers incl. 1/L of e^{tau/2 C} and e^{tau S}, or (increments)
+// of those less the identity.
+void padded_factors(const AxisHost& T, bool increments, std::vector<double>* mC, std::vector<double>* mS);
+// L real multipliers incl. 1/L of B itself (diagnostics).
+void padded_operator(const AxisHost& T, std::vector<double>* mB);
+// L complex e^{-2 pi i m / L}, interleaved.
+std::vector<double> padded_twiddles(int n);
 
 // Tables of one axis for Riesz order alpha, interface parameter eps, step tau,
 // domain [a, b] and n interior unknowns.

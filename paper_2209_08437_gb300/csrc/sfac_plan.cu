@@ -94,6 +94,7 @@ struct sfac_plan {
     int device = 0;
     long long npts = 0;
     void* dev_tables = nullptr;
+    void* fft_tables = nullptr;  // of axes with a tensor-core pass, where an operator was refused
     struct Ax {
         const void* eC;
         const void* eS;
@@ -303,6 +304,64 @@ sfac_status run_steps(sfac_plan* P, void* u, long long nsteps, cudaStream_t st, 
     return SFAC_OK;
 }
 
+// Tables on their way to one device block, each 256-byte aligned.
+struct TableBlock {
+    std::vector<unsigned char> bytes;
+    size_t zeros(size_t count) {
+        const size_t at = bytes.size();
+        bytes.resize(at + align256(count), 0);
+        return at;
+    }
+    size_t add(const std::vector<double>& v, bool f64 = true) {
+        const size_t at = zeros(v.size() * (f64 ? sizeof(double) : sizeof(float)));
+        if (f64) {
+            if (!v.empty()) std::memcpy(bytes.data() + at, v.data(), v.size() * sizeof(double));
+        } else {
+            float* f = reinterpret_cast<float*>(bytes.data() + at);
+            for (size_t i = 0; i < v.size(); ++i) f[i] = (float)v[i];  // rounded once
+        }
+        return at;
+    }
+};
+
+// Offsets of the tables of one axis's FFT pass: the factors' multipliers, twist and
+// twiddles in the plan's precision, and the FP64 ratio twiddles (kNone: not there).
+constexpr size_t kNone = ~(size_t)0;
+struct FftTables {
+    size_t eC = kNone, eS = kNone, twist = kNone, twid = kNone, rtwid = kNone;
+};
+
+FftTables add_fft_tables(TableBlock& b, const AxisHost& T, bool padded, bool f64) {
+    FftTables t;
+    if (padded) {
+        std::vector<double> mC, mS;
+        sfac::padded_factors(T, !f64, &mC, &mS);
+        t.eC = b.add(mC, f64);
+        t.eS = b.add(mS, f64);
+        t.twid = b.add(sfac::padded_twiddles(T.n), f64);
+    } else {
+        t.eC = b.add(f64 ? T.eC : T.dC, f64);
+        t.eS = b.add(f64 ? T.eS : T.dS, f64);
+        t.twist = b.add(T.twist, f64);
+        t.twid = b.add(T.twid, f64);
+    }
+    if (f64) {
+        const int N = padded ? sfac::padded_length(T.n) : T.n;
+        const std::vector<double> r = sfac::ratio_twiddles(N, sfac::f64_elems_per_thread(N));
+        if (!r.empty()) t.rtwid = b.add(r);
+    }
+    return t;
+}
+
+void set_fft_tables(sfac_plan* P, int l, const unsigned char* base, const FftTables& t) {
+    auto at = [&](size_t off) -> const void* { return off == kNone ? nullptr : base + off; };
+    P->ax[l].eC = at(t.eC);
+    P->ax[l].eS = at(t.eS);
+    P->ax[l].twist = at(t.twist);
+    P->ax[l].twid = at(t.twid);
+    P->ax[l].rtwid = at(t.rtwid);
+}
+
 }  // namespace
 
 extern "C" {
@@ -353,194 +412,158 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     P->jq_full_E = std::exp(-2.0 * params->tau);
     P->jq_full_1mE = -std::expm1(-2.0 * params->tau);
 
+    // Any allocation of the host that fails from here on comes back as SFAC_ENOMEM; P
+    // goes with the scope until it is handed out.
+    struct Owner {
+        sfac_plan* plan;
+        ~Owner() {
+            if (!plan) return;
+            if (plan->dev_tables) cudaFree(plan->dev_tables);
+            if (plan->fft_tables) cudaFree(plan->fft_tables);
+            delete plan;
+        }
+    } owner{P};
+    const int dim = params->dim;
+    const bool f64 = params->prec == SFAC_FP64;
     AxisHost host[3];
-    sfac::AxisPadded pad[3];
-    bool padded[3] = {false, false, false};
-    try {
+    bool padded[3] = {false, false, false}, tc[3] = {false, false, false};
+    int fft_len[3] = {0, 0, 0};
+    {
         long long inner = 1;
-        for (int l = 0; l < params->dim; ++l) {
-            compute_axis(params->alpha[l], params->eps, params->tau, params->a, params->b, params->n[l], &host[l]);
+        for (int l = 0; l < dim; ++l) {
+            const int n = params->n[l];
+            compute_axis(params->alpha[l], params->eps, params->tau, params->a, params->b, n, &host[l]);
             // Zero-padded pass for lengths that are not powers of two >= 4, and for
             // any strided axis (l > 0) whose stride (the product of the earlier
             // extents) is odd: its column pairs are not 2-vector aligned.
-            padded[l] = !(is_pow2(params->n[l]) && params->n[l] >= 4) || (l > 0 && (inner & 1));
-            if (padded[l]) sfac::compute_axis_padded(host[l], params->tau, &pad[l]);
-            inner *= params->n[l];
-        }
-    } catch (const std::bad_alloc&) {
-        delete P;
-        return fail(SFAC_ENOMEM, "host allocation failed");
-    }
-    cudaError_t err = cudaGetDevice(&P->device);
-    if (err != cudaSuccess) {
-        delete P;
-        return cuda_fail(err, "cudaGetDevice");
-    }
-    // FP64 ratio twiddles of each axis's FFT length; the spectra from which the
-    // operators of axes with a tensor-core pass are built.
-    std::vector<double> rtw[3], spectra[3];
-    bool tc[3] = {false, false, false};
-    if (params->prec == SFAC_FP64) {
-        try {
-            for (int l = 0; l < params->dim; ++l) {
-                const int N = padded[l] ? pad[l].L : params->n[l];
-                const int E = sfac::f64_elems_per_thread(N);
-                if (E <= 16) rtw[l] = sfac::ratio_twiddles(N, E);
-            }
-        } catch (const std::bad_alloc&) {
-            delete P;
-            return fail(SFAC_ENOMEM, "host allocation failed");
-        }
-    }
-    try {
-        for (int l = 0; l < params->dim; ++l) {
+            padded[l] = !(is_pow2(n) && n >= 4) || (l > 0 && (inner & 1));
+            fft_len[l] = padded[l] ? sfac::padded_length(n) : n;
             // FP32: zero-padded axes only. There the FFTs run at twice the length or
             // more (side by side: 3D 255^3 passes 168/243/253 -> 80/72/72 us, 255 x 100 x
             // 127 39/35/29 -> 26/29/23 us); the power-of-two passes are as fast or
             // faster on the FMA pipes (256^3: 60 against 68 us), and so are padded
             // lines of up to 64 points (63^3: 8.9 against 9.4 us).
-            tc[l] = params->prec == SFAC_FP64 ? params->n[l] >= sfac::kTcMinN && params->n[l] <= sfac::kTcLongMaxN
-                                              : padded[l] && params->n[l] > 64 && params->n[l] <= sfac::kTcMaxN;
-            if (tc[l]) spectra[l] = sfac::increment_spectra(host[l], params->tau);
+            tc[l] = f64 ? n >= sfac::kTcMinN && n <= sfac::kTcLongMaxN : padded[l] && n > 64 && n <= sfac::kTcMaxN;
+            inner *= n;
         }
-    } catch (const std::bad_alloc&) {
-        delete P;
-        return fail(SFAC_ENOMEM, "host allocation failed");
     }
-    // One device block: per axis eC[n], eS[n], twist[2n], twid[2n] reals, the
-    // FP64 diagnostic tables, and the ratio twiddles.
-    const size_t rs = real_size(P);
-    size_t off[3][11], total = 0;
+    cudaError_t err = cudaGetDevice(&P->device);
+    if (err != cudaSuccess) return cuda_fail(err, "cudaGetDevice");
+    P->diag_direct = sfac::diag_direct_pays(dim, params->n, fft_len, padded);
+
+    // One device block, uploaded at once: the tables of the FFT passes (of axes
+    // without a tensor-core pass, see below for the others), the spectra from which
+    // the operators of the others are built, the FP64 diagnostic tables, and zeroed
+    // words. Behind it, not part of the upload, the digit images of the tensor-core
+    // passes and their builder's scratch.
+    TableBlock block;
+    FftTables fft[3];
+    size_t off_spectra[3] = {0, 0, 0}, off_diag[3][4] = {}, off_col[3] = {0, 0, 0};
     long long max_partials = 1, direct_lines = 0;
     {
         long long inner = 1;
-        for (int l = 0; l < params->dim; ++l) {
-            const size_t n = padded[l] ? (size_t)pad[l].L : (size_t)params->n[l];
-            const size_t sz[11] = {n * rs, n * rs, padded[l] ? 0 : 2 * n * rs, 2 * n * rs,
-                                  n * 8,  padded[l] ? 0 : n * 8, padded[l] ? 0 : 2 * n * 8, 2 * n * 8,
-                                  rtw[l].size() * sizeof(double),
-                                  spectra[l].size() * sizeof(double), (size_t)params->n[l] * sizeof(double)};
-            for (int q = 0; q < 11; ++q) {
-                off[l][q] = total;
-                total += align256(sz[q]);
-            }
-            const long long outer = P->npts / ((long long)params->n[l] * inner);
-            const long long clines = l == 0 ? (outer + 1) / 2 : outer * ((inner + 1) / 2);
-            max_partials = std::max(max_partials, sfac::diag_partials_needed(clines, (int)n));
-            direct_lines += outer * inner;
-            inner *= params->n[l];
-        }
-    }
-    int fft_len[3];
-    for (int l = 0; l < params->dim; ++l) fft_len[l] = padded[l] ? pad[l].L : params->n[l];
-    P->diag_direct = sfac::diag_direct_pays(params->dim, params->n, fft_len, padded);
-    if (P->diag_direct) max_partials = std::max(max_partials, direct_lines);
-    const size_t off_partial = total;
-    total += align256(sizeof(double3) * (size_t)max_partials);
-    const size_t off_out = total;
-    total += align256(4 * sizeof(double));
-    const size_t off_status = total;
-    total += align256(sizeof(unsigned int));
-    const size_t off_bar = total;
-    total += align256(2 * sizeof(unsigned int));
-    // Not part of the upload: the digit images of the tensor-core passes and the
-    // builder's scratch (used by one axis after the other).
-    const int slices = params->prec == SFAC_FP64 ? sfac::kTcSlices : sfac::kTcSlices32;
-    size_t off_img[3] = {0, 0, 0}, alloc = total, scratch = 0;
-    for (int l = 0; l < params->dim; ++l) {
-        if (!tc[l]) continue;
-        off_img[l] = alloc;
-        alloc += align256(sfac::tc_image_bytes(params->n[l], slices));
-        scratch = std::max(scratch, sfac::tc_scratch_bytes(params->n[l]));
-    }
-    const size_t off_scratch = alloc;
-    alloc += align256(scratch);
-    std::vector<unsigned char> blob;
-    try {
-        blob.assign(total, 0);
-    } catch (const std::bad_alloc&) {
-        delete P;
-        return fail(SFAC_ENOMEM, "host allocation failed");
-    }
-    for (int l = 0; l < params->dim; ++l) {
-        const bool f64 = params->prec == SFAC_FP64;
-        const std::vector<double> none;
-        const std::vector<double>* src[4] = {f64 ? &host[l].eC : &host[l].dC, f64 ? &host[l].eS : &host[l].dS,
-                                             &host[l].twist, &host[l].twid};
-        if (padded[l]) {
-            src[0] = f64 ? &pad[l].mC : &pad[l].mC1;
-            src[1] = f64 ? &pad[l].mS : &pad[l].mS1;
-            src[2] = &none;
-            src[3] = &pad[l].twid;
-        }
-        // FP64 diagnostic tables
-        std::vector<double> lamN, muN;
-        if (!padded[l]) {
-            const double inv = 1.0 / (double)params->n[l];
-            lamN.resize(params->n[l]);
-            muN.resize(params->n[l]);
-            for (int j = 0; j < params->n[l]; ++j) {
-                lamN[j] = host[l].lambda[j] * inv;
-                muN[j] = host[l].mu[j] * inv;
-            }
-        }
-        const std::vector<double>* dsrc[4] = {padded[l] ? &pad[l].mB : &lamN, padded[l] ? &none : &muN,
-                                              padded[l] ? &none : &host[l].twist,
-                                              padded[l] ? &pad[l].twid : &host[l].twid};
-        for (int q = 0; q < 4; ++q)
-            if (!dsrc[q]->empty())
-                std::memcpy(blob.data() + off[l][4 + q], dsrc[q]->data(), dsrc[q]->size() * sizeof(double));
-        if (!rtw[l].empty())
-            std::memcpy(blob.data() + off[l][8], rtw[l].data(), rtw[l].size() * sizeof(double));
-        if (tc[l]) std::memcpy(blob.data() + off[l][9], spectra[l].data(), spectra[l].size() * sizeof(double));
-        std::memcpy(blob.data() + off[l][10], host[l].bcol.data(), host[l].bcol.size() * sizeof(double));
-        for (int q = 0; q < 4; ++q) {
-            unsigned char* dst = blob.data() + off[l][q];
-            const std::vector<double>& v = *src[q];
-            if (rs == sizeof(double)) {
-                std::memcpy(dst, v.data(), v.size() * sizeof(double));
+        for (int l = 0; l < dim; ++l) {
+            const int n = params->n[l];
+            if (!tc[l]) fft[l] = add_fft_tables(block, host[l], padded[l], f64);
+            else off_spectra[l] = block.add(sfac::increment_spectra(host[l]));
+            if (P->diag_direct) {
+                off_col[l] = block.add(host[l].bcol);
+            } else if (padded[l]) {
+                std::vector<double> mB;
+                sfac::padded_operator(host[l], &mB);
+                off_diag[l][0] = block.add(mB);
+                off_diag[l][3] = block.add(sfac::padded_twiddles(n));
             } else {
-                float* f = reinterpret_cast<float*>(dst);
-                for (size_t i = 0; i < v.size(); ++i) f[i] = (float)v[i];  // rounded once
+                std::vector<double> lamN(host[l].lambda), muN(host[l].mu);
+                for (double& v : lamN) v *= 1.0 / (double)n;
+                for (double& v : muN) v *= 1.0 / (double)n;
+                off_diag[l][0] = block.add(lamN);
+                off_diag[l][1] = block.add(muN);
+                off_diag[l][2] = block.add(host[l].twist);
+                off_diag[l][3] = block.add(host[l].twid);
             }
+            const long long outer = P->npts / ((long long)n * inner);
+            const long long clines = l == 0 ? (outer + 1) / 2 : outer * ((inner + 1) / 2);
+            max_partials = std::max(max_partials, sfac::diag_partials_needed(clines, fft_len[l]));
+            direct_lines += outer * inner;
+            inner *= n;
         }
     }
+    const size_t off_out = block.zeros(4 * sizeof(double));
+    const size_t off_status = block.zeros(sizeof(unsigned int));
+    const size_t off_bar = block.zeros(2 * sizeof(unsigned int));
+    const size_t off_report = block.zeros(3 * sizeof(sfac::TcReport));
+    const int slices = f64 ? sfac::kTcSlices : sfac::kTcSlices32;
+    size_t off_img[3] = {0, 0, 0}, alloc = block.bytes.size(), scratch = 0;
+    auto reserve = [&](size_t bytes) {
+        const size_t at = alloc;
+        alloc += align256(bytes);
+        return at;
+    };
+    const size_t off_partial = reserve(sizeof(double3) * (size_t)(P->diag_direct ? direct_lines : max_partials));
+    for (int l = 0; l < dim; ++l) {
+        if (!tc[l]) continue;
+        off_img[l] = reserve(sfac::tc_image_bytes(params->n[l], slices));
+        scratch += sfac::tc_scratch_bytes(params->n[l]);
+    }
+    const size_t off_scratch = reserve(scratch);
     err = cudaMalloc(&P->dev_tables, alloc);
     if (err != cudaSuccess) {
-        delete P;
+        P->dev_tables = nullptr;
         cudaGetLastError();
         return fail(SFAC_ENOMEM, std::string("cudaMalloc of tables: ") + cudaGetErrorString(err));
     }
     cudaStream_t st_ = static_cast<cudaStream_t>(stream);
     unsigned char* base = static_cast<unsigned char*>(P->dev_tables);
-    int report[3][8] = {};
-    err = cudaMemcpyAsync(P->dev_tables, blob.data(), total, cudaMemcpyHostToDevice, st_);
-    for (int l = 0; l < params->dim && err == cudaSuccess; ++l)
+    sfac::TcReport report[3] = {};
+    sfac::TcBuildAxis build[3];
+    int nbuild = 0;
+    for (int l = 0; l < dim; ++l)
         if (tc[l])
-            err = sfac::tc_build(params->n[l], slices, params->prec == SFAC_FP64 ? sfac::kTcBits : sfac::kTcBits32,
-                                 reinterpret_cast<const double*>(base + off[l][9]), base + off_img[l],
-                                 base + off_scratch, report[l], st_);
-    if (err == cudaSuccess) err = cudaStreamSynchronize(st_);
-    if (err != cudaSuccess) {
-        cudaFree(P->dev_tables);
-        delete P;
-        return cuda_fail(err, "table upload");
+            build[nbuild++] = {params->n[l], reinterpret_cast<const double*>(base + off_spectra[l]), base + off_img[l],
+                               reinterpret_cast<sfac::TcReport*>(base + off_report) + l};
+    err = cudaMemcpyAsync(P->dev_tables, block.bytes.data(), block.bytes.size(), cudaMemcpyHostToDevice, st_);
+    if (nbuild > 0) {
+        if (err == cudaSuccess)
+            err = sfac::tc_build(nbuild, build, slices, f64 ? sfac::kTcBits : sfac::kTcBits32, base + off_scratch, st_);
+        if (err == cudaSuccess)
+            err = cudaMemcpyAsync(report, base + off_report, sizeof(report), cudaMemcpyDeviceToHost, st_);
     }
-    for (int l = 0; l < params->dim; ++l)
-        if (tc[l]) sfac::tc_accept(params->n[l], slices, base + off_img[l], report[l], &P->ax[l].tc);
-    for (int l = 0; l < params->dim; ++l) {
-        P->ax[l].eC = base + off[l][0];
-        P->ax[l].eS = base + off[l][1];
-        P->ax[l].twist = padded[l] ? nullptr : base + off[l][2];
-        P->ax[l].twid = base + off[l][3];
-        P->ax[l].rtwid = rtw[l].empty() ? nullptr : base + off[l][8];
+    if (err == cudaSuccess) err = cudaStreamSynchronize(st_);
+    if (err != cudaSuccess) return cuda_fail(err, "table upload");
+    bool refused = false;
+    for (int l = 0; l < dim; ++l)
+        if (tc[l] && !sfac::tc_accept(params->n[l], slices, base + off_img[l], report[l], &P->ax[l].tc)) refused = true;
+    for (int l = 0; l < dim; ++l) {
         P->ax[l].padded = padded[l];
         P->ax[l].fft_len = fft_len[l];
-        P->ax[l].dA = reinterpret_cast<const double*>(base + off[l][4]);
-        P->ax[l].dB = padded[l] ? nullptr : reinterpret_cast<const double*>(base + off[l][5]);
-        P->ax[l].dtwist = padded[l] ? nullptr : base + off[l][6];
-        P->ax[l].dtwid = base + off[l][7];
-        P->ax[l].dcol = reinterpret_cast<const double*>(base + off[l][10]);
+        if (!tc[l]) set_fft_tables(P, l, base, fft[l]);
+        if (P->diag_direct) {
+            P->ax[l].dcol = reinterpret_cast<const double*>(base + off_col[l]);
+            continue;
+        }
+        P->ax[l].dA = reinterpret_cast<const double*>(base + off_diag[l][0]);
+        P->ax[l].dB = padded[l] ? nullptr : reinterpret_cast<const double*>(base + off_diag[l][1]);
+        P->ax[l].dtwist = padded[l] ? nullptr : base + off_diag[l][2];
+        P->ax[l].dtwid = base + off_diag[l][3];
+    }
+    if (refused) {
+        // An operator stays with the FFTs (rare, see tc_accept): only now the tables of
+        // those passes, of every such axis, as the whole-call launch then takes FFTs for all.
+        TableBlock more;
+        for (int l = 0; l < dim; ++l)
+            if (tc[l]) fft[l] = add_fft_tables(more, host[l], padded[l], f64);
+        err = cudaMalloc(&P->fft_tables, more.bytes.size());
+        if (err != cudaSuccess) {
+            P->fft_tables = nullptr;
+            cudaGetLastError();
+            return fail(SFAC_ENOMEM, std::string("cudaMalloc of tables: ") + cudaGetErrorString(err));
+        }
+        err = cudaMemcpyAsync(P->fft_tables, more.bytes.data(), more.bytes.size(), cudaMemcpyHostToDevice, st_);
+        if (err == cudaSuccess) err = cudaStreamSynchronize(st_);
+        if (err != cudaSuccess) return cuda_fail(err, "table upload");
+        for (int l = 0; l < dim; ++l)
+            if (tc[l]) set_fft_tables(P, l, static_cast<unsigned char*>(P->fft_tables), fft[l]);
     }
     P->diag_partial = reinterpret_cast<double3*>(base + off_partial);
     P->diag_out = reinterpret_cast<double*>(base + off_out);
@@ -551,11 +574,10 @@ sfac_status sfac_plan_create(const sfac_params* params, void* stream, sfac_plan*
     if (err != cudaSuccess) {
         cudaGetLastError();
         P->status_host = nullptr;
-        cudaFree(P->dev_tables);
-        delete P;
         return fail(SFAC_ENOMEM, std::string("cudaMallocHost of the status word: ") + cudaGetErrorString(err));
     }
     *P->status_host = 0;
+    owner.plan = nullptr;
     *out = P;
     return SFAC_OK;
 } catch (...) {
@@ -570,6 +592,7 @@ sfac_status sfac_plan_destroy(sfac_plan* plan) try {
         cudaError_t err = cudaDeviceSynchronize();
         if (err != cudaSuccess) st = cuda_fail(err, "synchronise before destroy");
         if (plan->dev_tables) cudaFree(plan->dev_tables);
+        if (plan->fft_tables) cudaFree(plan->fft_tables);
         if (plan->staging) cudaFree(plan->staging);
         if (plan->status_host) cudaFreeHost(plan->status_host);
     }

@@ -37,20 +37,33 @@ constexpr int kTcLongMaxN = 1024;
 __host__ __device__ constexpr bool tc_groups_inside(long long i, long long total) { return i >= 3 && i + 11 <= total; }
 
 // Device bytes of the digit image of an axis of n points, and of the scratch
-// the builder needs.
+// the builder needs for it.
 size_t tc_image_bytes(int n, int slices);
 size_t tc_scratch_bytes(int n);
 
-// Builds the image from increment_spectra's 4n values (device), on stream s. The
-// host words report[0..7] receive, after the stream is synchronised: the scale
-// exponent, then for each of six digit places the largest sum of |digit| over a
-// row's 128 columns, and the largest row sum of |entries| in units of 2^(f - 10).
-cudaError_t tc_build(int n, int slices, int bits, const double* spectra, void* img, void* scratch, int* report_host,
-                     cudaStream_t s);
+// What the builder says of an operator, in device memory that is zero before: the
+// bits of the largest |entry|; the scale exponent, then for each of six digit places
+// the largest sum of |digit| over a row's 128 columns, and the largest row sum of
+// |entries| in units of 2^(f - 10).
+struct TcReport {
+    unsigned long long largest;
+    int values[8];
+};
+
+struct TcBuildAxis {
+    int n;
+    const double* spectra;  // increment_spectra's 4n values (device)
+    void* img;              // tc_image_bytes
+    TcReport* report;
+};
+
+// Builds the images of `count` (at most 3) axes on stream s; scratch: the sum of
+// their tc_scratch_bytes.
+cudaError_t tc_build(int count, const TcBuildAxis* axes, int slices, int bits, void* scratch, cudaStream_t s);
 
 // Fills *ax from the builder's report; false where the sums could leave the
 // range in which the products are exact (the axis then keeps its FFT pass).
-bool tc_accept(int n, int slices, const void* img, const int* report, TcAxis* ax);
+bool tc_accept(int n, int slices, const void* img, const TcReport& report, TcAxis* ax);
 
 // One axis pass (the arguments of launch_pass_f64 / _f32) through the tensor cores.
 cudaError_t launch_pass_tc_f64(const TcAxis& ax, const PassArgs& a, cudaStream_t s);

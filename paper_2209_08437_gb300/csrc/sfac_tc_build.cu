@@ -4,8 +4,16 @@
 // symmetric Toeplitz with first columns g, h) the linear factor of an axis is
 //   P = (I + G)(I + H)(I + G) = I + D,  D = G + W + G W,  W = H + G + H G.
 // D is formed in FP64 from the increments, so its rounding is relative to D
-// itself. It runs once per plan (n = 256: 17 M multiply-adds an axis; plan creation for
-// 3D 256^3 0.7 -> 1.3 ms, for 2D 1024^2 4.6 -> 9.0 ms).
+// itself. Only its first column takes matrix-vector products. With Z the cyclic
+// shift, Z E_C Z^-1 = E_C, and Z E_S Z^-1 - E_S = -2 (e_0 v^T + v e_0^T) with v = h but
+// v_0 = 0 (h_{n-k} = -h_k); hence along a diagonal
+//   D_{i+1,j+1} = D_{ij} + 2 (g_{i+1} w_{j+1} + w_{i+1} g_{j+1}),  w = (I + G) v.
+// So D takes n^2 operations, not two products of n^3 / 2 on the FP64 pipe, and against
+// 80-bit arithmetic its largest error is 1.8e-18 at n = 256 (the products: 5.9e-18).
+// It runs once per plan, all axes in one set of launches (n = 1024, two axes: columns
+// 52 us, vectors 28, diagonals 64, largest entry 21, digits 45). Plan creation side by
+// side, with the products / now / without operators (ms): 2D 64^2 0.69 / 0.56 / 0.51,
+// 255^2 1.64 / 0.84 / 1.25, 1024^2 8.99 / 4.93 / 4.70, 3D 256^3 1.45 / 0.99 / 0.93.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -16,65 +24,174 @@
 namespace sfac {
 namespace {
 
-int parts_of(int n) { return n <= 128 ? 1 : 2; }
-int rows_of(int n) { return n <= 128 ? n : (n + 1) / 2; }
-int kp_of(int n) { return (rows_of(n) + 31) / 32 * 32; }
+__host__ __device__ int parts_of(int n) { return n <= 128 ? 1 : 2; }
+__host__ __device__ int rows_of(int n) { return n <= 128 ? n : (n + 1) / 2; }
+__host__ __device__ int kp_of(int n) { return (rows_of(n) + 31) / 32 * 32; }
+
+// One axis at work; its arrays but the first and the last two in the scratch.
+struct TcBuild {
+    int n;
+    const double* spectra;
+    double *g, *h, *wc, *wc_low, *w, *d0, *d0_low, *D;
+    void* img;
+    TcReport* report;
+};
+// All axes of a plan: blockIdx.z of every launch.
+struct TcBuilds {
+    TcBuild axis[3];
+    int slices, bits;
+};
+
+// Compensated sum s + c: Knuth's branch-free two-sum collects the rounding of s in c.
+struct TcSum {
+    double s = 0.0, c = 0.0;
+    __device__ __forceinline__ void add(double v) {
+        const double t = __dadd_rn(s, v), b = __dadd_rn(t, -s);
+        c = __dadd_rn(c, __dadd_rn(__dadd_rn(s, -__dadd_rn(t, -b)), __dadd_rn(v, -b)));
+        s = t;
+    }
+};
+
+constexpr int kTcSumThreads = 128;
+
+// The sum over the CTA's threads, in thread 0.
+__device__ double tc_cta_sum(double a) {
+    __shared__ double part[kTcSumThreads / 32];
+    for (int w = 16; w > 0; w >>= 1) a += __shfl_xor_sync(0xffffffffu, a, w);
+    if (threadIdx.x % 32 == 0) part[threadIdx.x / 32] = a;
+    __syncthreads();
+    return (part[0] + part[1]) + (part[2] + part[3]);
+}
+__device__ double tc_cta_sum(TcSum a) {
+    __shared__ double part[2][kTcSumThreads];
+    const int tid = threadIdx.x;
+    part[0][tid] = a.s;
+    part[1][tid] = a.c;
+    for (int w = kTcSumThreads / 2; w > 0; w >>= 1) {
+        __syncthreads();
+        if (tid < w) {
+            a.add(part[0][tid + w]);
+            a.c += part[1][tid + w];
+            part[0][tid] = a.s;
+            part[1][tid] = a.c;
+        }
+    }
+    return a.s + a.c;
+}
 
 // First columns g, h from the expm1 values xc, xs of the spectra and cs[m] =
 // cos(pi m / n):  g_d = (1/n) sum_j xc_j cos(2 pi j d / n),
-// h_d = (1/n) sum_j xs_j cos(pi d (2j - 1) / n). One CTA per d; each thread sums
-// with compensation (Neumaier), the partial sums are added in a fixed order.
-__global__ void __launch_bounds__(128) tc_columns(int n, const double* __restrict__ spectra, double* __restrict__ g,
-                                                  double* __restrict__ h) {
-    const int d = blockIdx.x, skew = blockIdx.y, two_n = 2 * n;
-    const double* x = spectra + skew * n;
-    const double* cs = spectra + two_n;
-    __shared__ double part[2][128];
-    double s = 0.0, c = 0.0;
-    auto add = [&](double v) {
-        const double t = __dadd_rn(s, v);
-        c += fabs(s) >= fabs(v) ? __dadd_rn(__dadd_rn(s, -t), v) : __dadd_rn(__dadd_rn(v, -t), s);
-        s = t;
-    };
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const int m = (int)((skew ? (long long)d * (2 * j - 1) + two_n * (long long)n : 2LL * d * j) % two_n);
-        add(__dmul_rn(x[j], cs[m]));
-    }
-    part[0][threadIdx.x] = s;
-    part[1][threadIdx.x] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int t = 1; t < blockDim.x; ++t) {
-            add(part[0][t]);
-            c += part[1][t];
-        }
-        (skew ? h : g)[d] = (s + c) / n;
-    }
+// h_d = (1/n) sum_j xs_j cos(pi d (2j - 1) / n); g_{n-d} = g_d, h_{n-d} = -h_d. One
+// CTA per d <= n / 2 and column.
+__global__ void __launch_bounds__(kTcSumThreads) tc_columns(const __grid_constant__ TcBuilds all) {
+    const TcBuild& b = all.axis[blockIdx.z];
+    const int n = b.n, d = blockIdx.x, skew = blockIdx.y;
+    if (2 * d > n) return;
+    const unsigned two_n = 2 * n;
+    const double* x = b.spectra + skew * n;
+    const double* cs = b.spectra + two_n;
+    TcSum a;
+    for (int j = threadIdx.x; j < n; j += kTcSumThreads)
+        a.add(__dmul_rn(x[j], cs[(unsigned)(skew ? d * (2 * j - 1) + d * 2 * n : 2 * d * j) % two_n]));
+    double v = tc_cta_sum(a) / n;
+    if (threadIdx.x != 0) return;
+    if (skew && 2 * d == n) v = 0.0;
+    double* column = skew ? b.h : b.g;
+    column[d] = v;
+    if (d > 0) column[n - d] = skew ? -v : v;
 }
 
-// out = X + Y + X Y with X[i][p] = x[|i - p|]; Y = y[|p - j|] (first product) or
-// the stored matrix Ym. All of them are centrosymmetric (M[i][j] =
-// M[n-1-i][n-1-j]): only the first ceil(n/2) rows are formed and stored.
-__global__ void __launch_bounds__(256) tc_product(int n, const double* __restrict__ x, const double* __restrict__ y,
-                                                  const double* __restrict__ Ym, double* __restrict__ out) {
-    const int j = blockIdx.x * 32 + threadIdx.x, i = blockIdx.y * 8 + threadIdx.y;
-    const int half = (n + 1) / 2;
-    if (i >= half || j >= n) return;
-    double s[4] = {0, 0, 0, 0};
-    for (int p0 = 0; p0 < n; p0 += 4) {
+// a + (b + c), with the rounding of the two additions in *low.
+__device__ double tc_add3(double a, double b, double c, double* low) {
+    TcSum s;
+    s.s = b;
+    s.add(c);
+    s.add(a);
+    const double hi = s.s + s.c;
+    *low = s.c - (hi - s.s);
+    return hi;
+}
+
+// One CTA per entry i: wc = (H + G + H G) e_0 = h + g + H g and w = v + G v (see above).
+// The rounding of wc, and below of D's first column, is kept: it would go into every
+// entry of a diagonal alike, and from there into every step of a call.
+__global__ void __launch_bounds__(kTcSumThreads) tc_vectors(const __grid_constant__ TcBuilds all) {
+    const TcBuild& b = all.axis[blockIdx.z];
+    const int n = b.n, i = blockIdx.x, second = blockIdx.y;
+    if (i >= n) return;
+    const double *m = second ? b.g : b.h, *x = second ? b.h : b.g;
+    double a = 0.0;
+    for (int p = threadIdx.x + (second && threadIdx.x == 0 ? kTcSumThreads : 0); p < n; p += kTcSumThreads)
+        a = fma(m[abs(i - p)], x[p], a);
+    a = tc_cta_sum(a);
+    if (threadIdx.x != 0) return;
+    if (second) b.w[i] = i > 0 ? a + b.h[i] : a;
+    else b.wc[i] = tc_add3(a, b.h[i], b.g[i], &b.wc_low[i]);
+}
+
+// One CTA per entry i of D's first column, g + wc + G wc.
+__global__ void __launch_bounds__(kTcSumThreads) tc_first(const __grid_constant__ TcBuilds all) {
+    const TcBuild& b = all.axis[blockIdx.z];
+    const int n = b.n, i = blockIdx.x;
+    if (i >= n) return;
+    double a = 0.0;
+    for (int p = threadIdx.x; p < n; p += kTcSumThreads) a = fma(b.g[abs(i - p)], b.wc[p], a);
+    a = tc_cta_sum(a);
+    if (threadIdx.x == 0) b.d0[i] = tc_add3(a + b.wc_low[i], b.wc[i], b.g[i], &b.d0_low[i]);
+}
+
+// The diagonals of D, 32 a CTA. D is symmetric and centrosymmetric (D[i][j] =
+// D[n-1-i][n-1-j]): only the first ceil(n/2) rows are formed and stored. Each warp
+// walks a quarter of the rows twice, for their sum and then, from the sum of the
+// quarters before, for the entries. The FP64 pipe bounds it (a warp alone on its
+// scheduler issues one FP64 operation in 64 cycles): the terms of eight rows are
+// summed plainly, which are small beside the entry, and only their sum is added with
+// compensation. n = 1024, two axes: 215 us with every term compensated by one warp.
+__global__ void __launch_bounds__(128) tc_diagonals(const __grid_constant__ TcBuilds all) {
+    constexpr int U = 8;
+    const TcBuild& b = all.axis[blockIdx.z];
+    const int n = b.n, lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int d = blockIdx.x * 32 + lane, half = (n + 1) / 2;
+    __shared__ double part[2][3][32];
+    const double *g = b.g, *w = b.w;
+    const int rows = min(half, n - d);  // of this diagonal; none for d >= n
+    const int quarter = (half + 2) / 4, first = 1 + warp * quarter, last = min(rows, first + quarter);
+    double* D = b.D;
+    auto put = [&](int i, double v) {
+        D[(size_t)i * n + i + d] = v;
+        if (i + d < half) D[(size_t)(i + d) * n + i] = v;
+    };
+    auto walk = [&](TcSum& a, bool store) {
+        for (int i0 = first; i0 < last; i0 += U) {
+            double p = 0.0;
+            const double v = a.s + a.c;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int p = p0 + q;
-            if (p < n)
-                s[q] = fma(x[abs(i - p)],
-                           !Ym        ? y[abs(p - j)]
-                           : p < half ? Ym[(size_t)p * n + j]
-                                      : Ym[(size_t)(n - 1 - p) * n + (n - 1 - j)],
-                           s[q]);
+            for (int q = 0; q < U; ++q) {
+                const int i = i0 + q;
+                if (i >= last) continue;
+                p = fma(2.0 * __ldg(g + i), __ldg(w + i + d), fma(2.0 * __ldg(w + i), __ldg(g + i + d), p));
+                if (store) put(i, v + p);
+            }
+            a.add(p);
         }
+    };
+    TcSum a;
+    if (warp < 3) {
+        walk(a, false);
+        part[0][warp][lane] = a.s;
+        part[1][warp][lane] = a.c;
     }
-    const double yij = Ym ? Ym[(size_t)i * n + j] : y[abs(i - j)];
-    out[(size_t)i * n + j] = ((s[0] + s[1]) + (s[2] + s[3])) + (x[abs(i - j)] + yij);
+    __syncthreads();
+    if (rows <= 0) return;
+    a = TcSum();
+    a.s = b.d0[d];
+    a.c = b.d0_low[d];
+    if (warp == 0) put(0, a.s);
+    for (int k = 0; k < warp; ++k) {
+        a.add(part[0][k][lane]);
+        a.c += part[1][k][lane];
+    }
+    walk(a, true);
 }
 
 // Entry (k, j) of part p of the operator: D itself, or its action on the sums
@@ -91,15 +208,18 @@ __device__ double tc_entry(const double* D, int n, int parts, int rows, int p, i
     return (mid_j || mid_k) ? 0.0 : a - b;
 }
 
-__global__ void __launch_bounds__(256) tc_max(int n, int parts, int rows, const double* __restrict__ D,
-                                              unsigned long long* out) {
+__global__ void __launch_bounds__(256) tc_max(const __grid_constant__ TcBuilds all) {
+    const TcBuild& b = all.axis[blockIdx.z];
+    const int n = b.n, parts = parts_of(n), rows = rows_of(n);
+    const double* D = b.D;
     double m = 0.0;
     const int total = parts * rows * rows;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
         const int p = t / (rows * rows), r = t % (rows * rows);
         m = fmax(m, fabs(tc_entry(D, n, parts, rows, p, r / rows, r % rows)));
     }
-    atomicMax(out, (unsigned long long)__double_as_longlong(m));
+    for (int w = 16; w > 0; w >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, w));
+    if (threadIdx.x % 32 == 0) atomicMax(&b.report->largest, (unsigned long long)__double_as_longlong(m));
 }
 
 // Digits of every entry (NS places of B bits), written as 8 KB blocks of 128 rows x
@@ -107,11 +227,15 @@ __global__ void __launch_bounds__(256) tc_max(int n, int parts, int rows, const 
 // blocks, the order in which a CTA streams them: (part, 32 columns, place) up to
 // 256 points, (128 rows, 32 columns, part, place) above. One CTA per (row,
 // part); report as in tc_build.
-__global__ void __launch_bounds__(128) tc_digits(int n, int parts, int rows, int kp, const double* __restrict__ D,
-                                                 const unsigned long long* __restrict__ maxbits, int NS, int B,
-                                                 __half* __restrict__ img, int* report) {
+__global__ void __launch_bounds__(128) tc_digits(const __grid_constant__ TcBuilds all) {
+    const TcBuild& b = all.axis[blockIdx.z];
+    const int n = b.n, parts = parts_of(n), rows = rows_of(n), kp = kp_of(n), NS = all.slices, B = all.bits;
     const int row = blockIdx.x, p = blockIdx.y, nkc = kp / 32;
-    const double m = __longlong_as_double((long long)*maxbits);
+    if (p >= parts || row >= (rows + 127) / 128 * 128) return;
+    const double* D = b.D;
+    __half* img = static_cast<__half*>(b.img);
+    int* report = b.report->values;
+    const double m = __longlong_as_double((long long)b.report->largest);
     int f = 0;
     if (m > 0.0) {
         f = ilogb(m) + 1;  // m < 2^f: the top digit has one bit more
@@ -152,32 +276,43 @@ __global__ void __launch_bounds__(128) tc_digits(int n, int parts, int rows, int
 }  // namespace
 
 size_t tc_image_bytes(int n, int slices) { return (size_t)parts_of(n) * ((rows_of(n) + 127) / 128) * (kp_of(n) / 32) * slices * 8192; }
-size_t tc_scratch_bytes(int n) { return 2 * sizeof(double) * ((size_t)((n + 1) / 2) * n + n) + 64; }
+size_t tc_scratch_bytes(int n) { return sizeof(double) * ((size_t)((n + 1) / 2) * n + 7 * (size_t)n); }
 
-cudaError_t tc_build(int n, int slices, int bits, const double* spectra, void* img, void* scratch, int* report_host,
-                     cudaStream_t s) {
-    const int parts = parts_of(n), rows = rows_of(n), kp = kp_of(n);
-    double* W = static_cast<double*>(scratch);
-    double* D = W + (size_t)((n + 1) / 2) * n;
-    double* g = D + (size_t)((n + 1) / 2) * n;
-    double* h = g + n;
-    unsigned long long* mx = reinterpret_cast<unsigned long long*>(h + n);
-    int* report = reinterpret_cast<int*>(mx + 1);
-    cudaError_t err = cudaMemsetAsync(mx, 0, 64, s);
-    if (err != cudaSuccess) return err;
-    const dim3 grid((n + 31) / 32, ((n + 1) / 2 + 7) / 8), block(32, 8);
-    tc_columns<<<dim3(n, 2), 128, 0, s>>>(n, spectra, g, h);
-    tc_product<<<grid, block, 0, s>>>(n, h, g, nullptr, W);
-    tc_product<<<grid, block, 0, s>>>(n, g, nullptr, W, D);
-    tc_max<<<std::max(1, std::min(64, n / 4)), 256, 0, s>>>(n, parts, rows, D, mx);
-    tc_digits<<<dim3((rows + 127) / 128 * 128, parts), 128, 0, s>>>(n, parts, rows, kp, D, mx, slices, bits, static_cast<__half*>(img),
-                                             report);
-    err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
-    return cudaMemcpyAsync(report_host, report, (2 + kTcSlices) * sizeof(int), cudaMemcpyDeviceToHost, s);
+cudaError_t tc_build(int count, const TcBuildAxis* axes, int slices, int bits, void* scratch, cudaStream_t s) {
+    TcBuilds all{};
+    all.slices = slices;
+    all.bits = bits;
+    unsigned char* at = static_cast<unsigned char*>(scratch);
+    int n = 0, rows = 0, parts = 1;
+    for (int l = 0; l < count; ++l) {
+        TcBuild& b = all.axis[l];
+        b.n = axes[l].n;
+        b.spectra = axes[l].spectra;
+        b.img = axes[l].img;
+        b.report = axes[l].report;
+        double* d = reinterpret_cast<double*>(at);
+        double** arrays[7] = {&b.g, &b.h, &b.wc, &b.wc_low, &b.w, &b.d0, &b.d0_low};
+        for (double** a : arrays) {
+            *a = d;
+            d += b.n;
+        }
+        b.D = d;
+        at += tc_scratch_bytes(b.n);
+        n = std::max(n, b.n);
+        rows = std::max(rows, (rows_of(b.n) + 127) / 128 * 128);
+        parts = std::max(parts, parts_of(b.n));
+    }
+    tc_columns<<<dim3(n / 2 + 1, 2, count), kTcSumThreads, 0, s>>>(all);
+    tc_vectors<<<dim3(n, 2, count), kTcSumThreads, 0, s>>>(all);
+    tc_first<<<dim3(n, 1, count), kTcSumThreads, 0, s>>>(all);
+    tc_diagonals<<<dim3((n + 31) / 32, 1, count), 128, 0, s>>>(all);
+    tc_max<<<dim3(std::max(1, std::min(64, n / 4)), 1, count), 256, 0, s>>>(all);
+    tc_digits<<<dim3(rows, parts, count), 128, 0, s>>>(all);
+    return cudaGetLastError();
 }
 
-bool tc_accept(int n, int slices, const void* img, const int* report, TcAxis* ax) {
+bool tc_accept(int n, int slices, const void* img, const TcReport& r, TcAxis* ax) {
+    const int* report = r.values;
     constexpr int NS = kTcSlices, B = kTcBits;
     ax->n = n;
     ax->parts = parts_of(n);
