@@ -41,13 +41,16 @@ __host__ __device__ constexpr bool tc_groups_inside(long long i, long long total
 size_t tc_image_bytes(int n, int slices);
 size_t tc_scratch_bytes(int n);
 
-// What the builder says of an operator, in device memory that is zero before: the
-// bits of the largest |entry|; the scale exponent, then for each of six digit places
-// the largest sum of |digit| over a row's 128 columns, and the largest row sum of
-// |entries| in units of 2^(f - 10).
+// What the builder says of an operator, in device memory that is zero before. The
+// products of a row and 128 columns are summed in one accumulator per order s = i + j
+// of the digit places, s = 2..6 here; sums[h][s - 2] is the largest over all rows and
+// column groups of what that accumulator can reach, in units of 2^(B - 1), with the
+// top digit of the lines at most 2^B (h = 0) or 2^(B - 1) (h = 1).
 struct TcReport {
-    unsigned long long largest;
-    int values[8];
+    unsigned long long largest;  // bits of the largest |entry|
+    int scale;                   // exponent f: the entries are below 2^f
+    int row_sum;                 // largest row sum of |entries| in units of 2^(f - 10)
+    int sums[2][5];
 };
 
 struct TcBuildAxis {

@@ -234,14 +234,14 @@ __global__ void __launch_bounds__(128) tc_digits(const __grid_constant__ TcBuild
     if (p >= parts || row >= (rows + 127) / 128 * 128) return;
     const double* D = b.D;
     __half* img = static_cast<__half*>(b.img);
-    int* report = b.report->values;
+    TcReport* report = b.report;
     const double m = __longlong_as_double((long long)b.report->largest);
     int f = 0;
     if (m > 0.0) {
         f = ilogb(m) + 1;  // m < 2^f: the top digit has one bit more
         f = f < -200 ? -200 : f;
     }
-    if (row == 0 && p == 0 && threadIdx.x == 0) report[0] = f;
+    if (row == 0 && p == 0 && threadIdx.x == 0) report->scale = f;
     __shared__ int sum[kTcSlices];
     __shared__ unsigned long long total;
     if (threadIdx.x == 0) total = 0;
@@ -268,9 +268,16 @@ __global__ void __launch_bounds__(128) tc_digits(const __grid_constant__ TcBuild
             }
         }
         __syncthreads();
-        if (threadIdx.x < kTcSlices) atomicMax(&report[1 + threadIdx.x], sum[threadIdx.x]);
+        // order s takes the row's places 1 .. s - 1, the last of them times the top
+        // digit of the line (see TcReport)
+        if (threadIdx.x < 10) {
+            const int h = threadIdx.x / 5, s = 2 + threadIdx.x % 5;
+            int reach = sum[s - 2] << (1 - h);
+            for (int j = 0; j < s - 2; ++j) reach += sum[j];
+            atomicMax(&report->sums[h][s - 2], reach);
+        }
     }
-    if (threadIdx.x == 0) atomicMax(&report[1 + kTcSlices], (int)(total >> 10));
+    if (threadIdx.x == 0) atomicMax(&report->row_sum, (int)(total >> 10));
 }
 
 }  // namespace
@@ -311,41 +318,38 @@ cudaError_t tc_build(int count, const TcBuildAxis* axes, int slices, int bits, v
     return cudaGetLastError();
 }
 
-bool tc_accept(int n, int slices, const void* img, const TcReport& r, TcAxis* ax) {
-    const int* report = r.values;
-    constexpr int NS = kTcSlices, B = kTcBits;
+bool tc_accept(int n, int slices, const void* img, const TcReport& report, TcAxis* ax) {
     ax->n = n;
     ax->parts = parts_of(n);
     ax->rows = rows_of(n);
     ax->kp = kp_of(n);
-    ax->scale = report[0];
+    ax->scale = report.scale;
     ax->headroom = 0;
     if (slices != kTcSlices) {
         // FP32: the sums are rounded to 24 bits like any FP32 sum. With entries of 1/2
         // and more (long steps: D cancels most of x) the FFT passes are the more
         // accurate ones; a tiny f would leave the exponent range of the closing products.
-        if (report[0] > -1 || report[0] < -60) return false;
+        if (report.scale > -1 || report.scale < -60) return false;
         ax->img = img;
         return true;
     }
-    // Largest sum the accumulator of order s = i + j can reach: digits of x are at
-    // most 2^(B-1) in size, the top one 2^B (over 128 columns), or 2^(B-1) too if lines are scaled by
-    // one more bit. Orders up to 5 must stay within 2^24 (FP32 holds every integer
-    // of that size), order 6 within 2^25 and order 7 anywhere: a unit lost there is
-    // below 2^-56 of the line's largest value.
+    // Digits of x are at most 2^(B-1) in size, the top one 2^B, or 2^(B-1) too if lines
+    // are scaled by one more bit (headroom). The accumulators of orders up to 5 must
+    // stay within 2^24 (FP32 holds every integer of that size), order 6 within 2^25 and
+    // order 7 anywhere: a unit lost there is below 2^-56 of the line's largest value.
+    // The reach of each order is that of one row: added up from the largest sum of each
+    // place over all rows it came to 1.25 times as much, and refused 1 in 40 ordinary
+    // parameter sets at 1024 points, whose passes then took 205 us instead of 62.
     int headroom = -1;
     for (int h = 0; h < 2 && headroom < 0; ++h) {
         bool ok = true;
-        for (int s = 2; s <= 6; ++s) {
-            double bound = std::ldexp((double)report[s - 1], B - h);
-            for (int j = 1; j < s - 1; ++j) bound += std::ldexp((double)report[j], B - 1);
-            ok = ok && bound <= std::ldexp(1.0, s <= 5 ? 24 : 25);
-        }
+        for (int s = 2; s <= 6; ++s)
+            ok = ok && std::ldexp((double)report.sums[h][s - 2], kTcBits - 1) <= std::ldexp(1.0, s <= 5 ? 24 : 25);
         if (ok) headroom = h;
     }
     if (headroom < 0) return false;
     // a row's sum of |entries| / 2^f, so that the 64-bit sums of the pass cannot overflow
-    if (report[1 + NS] > 4 << 10 || report[0] > 2) return false;
+    if (report.row_sum > 4 << 10 || report.scale > 2) return false;
     ax->headroom = headroom;
     ax->img = img;
     return true;

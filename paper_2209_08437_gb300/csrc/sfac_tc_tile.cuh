@@ -11,9 +11,10 @@
 //    54 fractional bits, cut into six signed digits of 9 bits (FP16 integers);
 //    D's entries likewise, once per plan (sfac_tc_build.cu);
 //  - the products of digit place i of x with place j of D are summed by
-//    tcgen05.mma into one FP32 accumulator per order i + j = 2..7. All of them
-//    are whole numbers of at most 2^24, so every sum is exact (tc_accept checks
-//    the bound for the plan's own D); orders from 8 on are left out;
+//    tcgen05.mma into one FP32 accumulator per order i + j = 2..7, whole numbers
+//    all. Orders 2..5 stay within 2^24, so their sums are exact; order 6 within
+//    2^25, and a unit lost there or in order 7 is below 2^-56 of the line's largest
+//    value (tc_accept checks the plan's own D); orders from 8 on are left out;
 //  - the six sums are added with their weights in 64-bit integers, and
 //    y = x + D x is rounded once.
 // Against 80-bit arithmetic the increment is within 0.1e-16 to 3e-16 (2-norm,

@@ -102,3 +102,34 @@ def test_fp32_refused_operator_takes_the_padded_fft():
         plan.check()
     ref = O.apply_axis(u0.astype(np.float64), P, 1)
     assert np.abs(u.double().cpu().numpy() - ref).max() <= 1e-5
+
+
+# Operators whose sums stay in range row by row, though the largest sums of each
+# digit place over all rows, added up, would not: (n, alpha, eps, tau) on (0, 1)
+IN_RANGE = [(1024, 1.726, 0.0679, 0.05), (1024, 1.65, 0.0965, 0.05), (1000, 1.838, 7.192, 0.005567),
+            (600, 1.636, 0.161, 1.199)]
+
+
+@pytest.mark.parametrize("n,alpha,eps,tau", IN_RANGE, ids=str)
+def test_operators_in_range_are_taken(n, alpha, eps, tau):
+    """They run on the tensor cores: lines scale exactly, each by itself."""
+    prob = I.Problem(n=(n, 6), alpha=(alpha, 1.5), eps=eps, tau=tau, a=0.0, b=1.0)
+    u0 = I.random_field(prob, 92, -1.0, 1.0)
+    scale = np.ldexp(1.0, -30 * (np.arange(6) % 2))[:, None]
+    got = one_pass(prob, u0, 0)
+    assert np.array_equal(got * scale, one_pass(prob, u0 * scale, 0))
+    assert np.abs(got - factor(prob, u0, 0)).max() <= 2e-14 * np.abs(u0).max()
+
+
+@pytest.mark.parametrize("n,ax", [((2048, 6), 0), ((6, 2048), 1), ((4096, 4), 0), ((9, 14), 0), ((14, 9), 1)], ids=str)
+@pytest.mark.parametrize("tau", [2e-3, 0.5])
+def test_flow_of_the_fft_passes(n, ax, tau):
+    """FP64 axes outside 17..1024 points keep the FP64 form of the flow (the probe
+    of tests/test_gpu_probe.py runs the fixed-point form): both flows around a
+    factor that is the identity to 1e-15. Bar: the rounding of six FFTs and two
+    flows of three units each."""
+    prob = I.Problem(n=n, alpha=(1.5, 1.5), eps=1e-10, tau=tau)
+    u0 = I.random_field(prob, 93, -1.0, 1.0)
+    u0.flat[::17] = 0.0
+    ref = O.nonlinear_flow(O.nonlinear_flow(u0, 0.5 * tau), tau)
+    assert np.abs(one_pass(prob, u0, ax, (1, 2)) - ref).max() <= 2e-14
