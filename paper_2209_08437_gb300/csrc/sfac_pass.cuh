@@ -954,6 +954,9 @@ cudaError_t set_smem_spread(K kern, LaunchSetup& ls, int* dev_out) {
 // 64 x 128 x 64 25.1 / 28.7 / 17.5, 64 x 128 x 128 31.2 / 29.2 / 21.9, 256 x 256 22.2 /
 // 10.9 / 10.6 (17.9 without the four warps, which keep room beside the previous
 // pass's CTAs). axis_pass_kernel stays as it is: 1024 x 1024 31.2 / 26.8 / 29.0.
+// Two plans on two streams, which then share fewer SMs, lose nothing by it (a step of
+// both, plain launches / spread: 64 x 128 x 64 32.1 / 28.3 us, 256 x 256 26.1 / 12.9,
+// 1024 x 256 24.1 / 20.4, 128^3 47.8 / 47.3).
 template <typename... P, typename... A>
 cudaError_t launch_spread(void (*kern)(P...), long long grid, unsigned block, size_t smem, const LaunchSetup& ls,
                           int dev, cudaStream_t s, const A&... args) {

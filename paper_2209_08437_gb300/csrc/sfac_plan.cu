@@ -229,6 +229,8 @@ sfac::StepsArgs steps_args(const sfac_plan* P, void* u, long long nsteps) {
     return g;
 }
 
+// (The residency asked for is that of the FFT kernel. The tensor-core launch, one CTA an
+// SM, is clamped to its own and loops over the tiles, so it runs wherever that one does.)
 bool steps_used(const sfac_plan* P, long long nsteps) {
     return nsteps >= 2 && steps_shape(P) && sfac::steps_fit(P->p.prec, steps_args(P, nullptr, nsteps));
 }
@@ -243,11 +245,14 @@ bool steps_used(const sfac_plan* P, long long nsteps) {
 // mapped into the device's address space (unified addressing; over
 // NVLink-C2C on GB300), so a pass can load from it or store to it directly.
 // That pays off where the first and the last pass have lines enough to hide
-// the link's latency: measured side by side on GB300 (e2e per step, copies vs
-// mapped) 3D 128^3 FP64 0.94 -> 0.79 ms, 256^3 FP64 7.56 -> 6.25 ms, 256^3
-// FP32 0.89 -> 0.77 ms, 100^3 FP64 1.10 -> 1.02 ms; but 2D 1024^2 FP64
-// 0.52 -> 0.54 ms and 64^3 FP64 0.178 -> 0.190 ms (few lines: latency bound).
-// Hence at least kHostRouteLines complex lines in both passes. An FP32 last
+// the link's latency. The line was drawn with FFT passes in both precisions (e2e per
+// step side by side on GB300, copies vs mapped: 3D 256^3 FP32 0.89 -> 0.77 ms; 2D
+// 1024^2 FP64 0.52 -> 0.54 and 64^3 FP64 0.178 -> 0.190: few lines, latency bound).
+// The tensor-core passes gain less from it, as their tiles load, compute and store in
+// turn (copies vs mapped): FP64 256^3 2.17 -> 2.19 ms, 255^3 2.19 -> 2.15, 512 x 128 x
+// 128 1.22 -> 1.08, 128^3 0.302 -> 0.310, 256 x 128 x 64 0.310 -> 0.355; FP32 255^3
+// 0.92 -> 1.07, 100^3 0.101 -> 0.103. The line is the same for all of them:
+// at least kHostRouteLines complex lines in both passes. An FP32 last
 // pass of more than 512 points writes narrow rows (fewer than 4 lines a CTA;
 // 2D 4096^2 FP32 1.38 -> 3.47 ms): the result then goes back by a copy.
 constexpr long long kHostRouteLines = 4096;

@@ -9,7 +9,7 @@
 namespace sfac {
 
 // The linear factor of one axis as a dense operator D = P - I, cut into
-// fixed-point digits (see sfac_tc_pass.cuh). `img` holds the digit blocks in the
+// fixed-point digits (see sfac_tc_tile.cuh). `img` holds the digit blocks in the
 // order the pass streams them.
 struct TcAxis {
     const void* img = nullptr;  // NULL: the axis has no tensor-core pass

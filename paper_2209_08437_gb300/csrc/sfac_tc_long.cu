@@ -15,8 +15,8 @@
 // Eight warps convert, drain and store; one more issues the copies and one the
 // products. Measured on 2D 1024^2 (side by side, passes without the flow): 205 us a
 // pass by FFTs on the FP64 pipe (90% busy), 62 us contiguous and 54 us strided here;
-// 512^2 37 and 33 us. The loads' latency and the conversion bound it (long-scoreboard
-// stalls 4-5 per issue, ALU 25-31%, tensor pipe 18%).
+// 512^2 37 and 33 us. By the times of its parts the loads' latency and the conversion
+// bound it.
 #include <cuda_runtime.h>
 
 #include <atomic>

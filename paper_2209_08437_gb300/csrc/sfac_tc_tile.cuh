@@ -31,7 +31,7 @@
 //
 // Measured (side by side, n = 256, 65536 lines): a pass of six FFTs on the FP64 pipe
 // took 1.90 ms (2.15 ms with the flow), this one 0.21 ms (0.27-0.31 ms). What bounds
-// it now: the phases of a tile follow each other (barrier stalls 3.4 per issue), with
+// it now: the phases of a tile follow each other (barrier stalls 2.2-3.1 per issue), with
 // the integer ALU, 64 operations a clock and SM, 38% busy over the whole pass, the
 // tensor pipe 18%, L2 10%. Tiles of 32 lines in two CTAs an SM did not overlap them:
 // a ring of two blocks each waited for the operator (820 us).
